@@ -211,3 +211,49 @@ def tolerance(case):
     # bf16 results, W_hat rounded to bf16 or not (seen against fp64: 2.4e-3; largest 1.5e-2 in Y, 5.7e-2 in the dX of
     # outlier channels' neighbours)
     return {"rel": 1e-2, "max": 6e-2 if case["kind"] == "forward" else 0.2}
+
+
+# ------------------------------------------------------------------ the same results in 64 bits
+def _unpacked(packed, bits):
+    runs = packed.view(packed.shape[0], -1, bits).to(torch.int64)                      # eight codes in `bits` bytes
+    value = sum(runs[..., i] << (8 * i) for i in range(bits))
+    shifts = torch.arange(0, 8 * bits, bits, device=packed.device)
+    return ((value[..., None] >> shifts) & ((1 << bits) - 1)).reshape(packed.shape[0], -1)
+
+
+def _exact_linear(kind, L):
+    d = L["desc"]
+    out, inp, group = d.out_features, d.in_features, d.group
+
+    def groups(v):
+        return v.view(out, inp // group, group)
+
+    if kind in ("block_ap", "weight"):
+        s, zr, Q = L["s"][..., None], torch.round(L["z"])[..., None], float((1 << d.bits) - 1)
+        r = torch.round(groups(L["W"].float()) / s)                                    # the code is decided in 32 bits
+        p = r + zr
+        inside, c = (p >= 0) & (p <= Q), p.clamp(0, Q) - zr
+        W_hat = (c.double() * s.double()).view(out, inp)
+        partial = torch.where(inside, r.double() - groups(L["W"].double()) / s.double(), c.double())
+        G = L["dW_hat"].double() if kind == "weight" else L["dY"].double().t() @ L["X"].double()
+        results = {"W_hat": W_hat, "dW": (groups(G) * inside).view(out, inp), "ds": (groups(G) * partial).sum(-1),
+                   "dz": (groups(G) * torch.where(inside, 0.0, -s.double())).sum(-1)}
+    else:
+        codes = _unpacked(L["Wq_packed"], d.bits)
+        step, centred = L["s16"].double()[..., None], groups(codes.double()) - L["z"].double()[..., None]
+        W_hat, results = (centred * step).view(out, inp), {}
+        if kind == "e2e_qp":
+            G = groups(L["dY"].double().t() @ L["X"].double())
+            results = {"ds": (G * centred).sum(-1), "dz": -step[..., 0] * G.sum(-1)}
+    if kind != "weight":
+        results["Y"] = L["X"].double() @ W_hat.t()
+    if kind in ("block_ap", "e2e_qp"):
+        results["dX"] = L["dY"].double() @ W_hat
+    return [results[name] for name in _RESULTS[kind] if L[name] is not None]
+
+
+def exact(case, seed):
+    if case["kind"] == "export":
+        return None                                  # compared bit for bit
+    state = prepare(case, seed)
+    return [v for L in state["linears"] for v in _exact_linear(state["kind"], L)]
