@@ -226,12 +226,12 @@ int eqat_unpack_zeros(const eqat_desc* desc, const uint8_t* z_packed, uint8_t* z
  * desc->zero_point_format is EQAT_ZP_FP16. */
 
 /* Y = X * ((W_int - z) * s)^T, the packed codes expanded tile by tile in
- * shared memory inside the GEMM (Eq. 2; Sec. 3.3).  With few tokens (decoding)
- * and groups of at least 64 a matrix-vector kernel streams the packed weight
- * instead and does not round (W_int - z) * s to bf16.  It takes up to eight
- * tokens per launch, and up to 64 tokens go through it in slices (one pass over
- * the packed weight per slice) while that is cheaper than the tiled kernel; a
- * token's result does not depend on how the tokens were sliced.
+ * shared memory inside the GEMM (Eq. 2; Sec. 3.3).  With few tokens (decoding),
+ * up to 64, the codes enter the products as exact integers and the step sizes
+ * multiply fp32 sums, so (W_int - z) * s is not rounded to bf16: a matrix-vector
+ * kernel of up to eight tokens per launch for the smallest batches (groups of at
+ * least 64; a token's result does not depend on how the tokens were sliced into
+ * launches), a kernel on tiles of 128 weight rows otherwise.
  *   X [T,in] bf16, Wq_packed, s16, z (in)   Y [T,out] bf16 (out) */
 int qlinear_packed_fwd(const eqat_desc* desc, const eqat_bf16* X, const uint8_t* Wq_packed,
                        const eqat_fp16* s16, const void* z, eqat_bf16* Y, void* stream);

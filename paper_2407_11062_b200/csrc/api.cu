@@ -5,6 +5,7 @@
 #include "elementwise.cuh"
 #include "gemm.cuh"
 #include "gemv.cuh"
+#include "slim.cuh"
 
 namespace {
 
@@ -151,11 +152,13 @@ size_t eqat_workspace_bytes(const eqat_desc* d, int op) {
 
 int eqat_device_status(int* h_status, int* h_detail) {
   if (h_status == nullptr) return EQAT_ERR_NULL;
-  int st[3] = {0, 0, 0}, det[3] = {0, 0, 0};
+  int st[4] = {0, 0, 0, 0}, det[4] = {0, 0, 0, 0};
   EQAT_TRY(read_device_status(&st[0], &det[0]));      // GEMM kernels
   EQAT_TRY(read_stream_status(&st[1], &det[1]));      // staged streaming kernels
   EQAT_TRY(read_gemv_status(&st[2], &det[2]));        // matrix-vector kernels
-  const int k = st[0] != EQAT_OK ? 0 : (st[1] != EQAT_OK ? 1 : 2);
+  EQAT_TRY(read_slim_status(&st[3], &det[3]));        // weight-row kernels
+  int k = 0;
+  while (k < 3 && st[k] == EQAT_OK) ++k;
   *h_status = st[k];
   if (h_detail != nullptr) *h_detail = det[k];
   return EQAT_OK;
@@ -165,6 +168,7 @@ int eqat_selftest_wait_expiry(int which, void* stream) {
   if (which == 0) return launch_wait_expiry_gemm(as_stream(stream));
   if (which == 1) return launch_wait_expiry_stream(as_stream(stream));
   if (which == 2) return launch_wait_expiry_gemv(as_stream(stream));
+  if (which == 3) return launch_wait_expiry_slim(as_stream(stream));
   return EQAT_ERR_UNSUPPORTED;
 }
 
@@ -251,6 +255,8 @@ int eqat_unpack_zeros(const eqat_desc* d, const uint8_t* z_packed, uint8_t* z8, 
 int qlinear_packed_fwd(const eqat_desc* d, const eqat_bf16* X, const uint8_t* Wq_packed, const eqat_fp16* s16,
                        const void* z, eqat_bf16* Y, void* stream) {
   EQAT_TRY(v_packed_fwd(d, X, Wq_packed, s16, z, Y));
+  SlimPlan plan;
+  if (slim_fwd_applies(*d, plan)) return launch_slim_fwd(*d, X, Wq_packed, s16, z, Y, plan, as_stream(stream));
   // a handful of tokens (decoding): one pass over the packed weight instead of near-empty tensor-core tiles
   if (packed_gemv_applies(*d)) return launch_packed_gemv(*d, X, Wq_packed, s16, z, Y, as_stream(stream));
   return launch_packed_fwd(*d, X, Wq_packed, s16, z, Y, as_stream(stream));

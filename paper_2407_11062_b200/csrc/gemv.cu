@@ -141,11 +141,6 @@ __device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, volatile 
   return true;
 }
 
-// Programmatic dependent launch: let the next launch of the stream start / wait until the launches before this one
-// have completed and their writes are visible (both do nothing in a launch without the attribute).
-__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // (t & mask) | magic on both halves of a register.
 __device__ __forceinline__ uint32_t and_or(uint32_t t, uint32_t mask, uint32_t magic) {
   uint32_t r;
@@ -258,7 +253,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
   // CTA of this grid has got here, and a CTA of this grid may be running while the launch before it still is.
   // Nothing before the wait below touches global memory (the barriers live in this CTA's shared memory); the
   // wait returns once the earlier grids have completed and their writes are visible.
-  grid_dependents_launch();
+  ptx::grid_dependents_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
       ptx::mbar_init(ptx::smem_addr(&ctl->full[s]), 1);
@@ -271,7 +266,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
     ctl->abort = 0;
     ptx::fence_mbar_init();
   }
-  grid_dependency_wait();
+  ptx::grid_dependency_wait();
 
   // Consumers request their first loads before the rest of the set-up: the first unit of the activations and the step
   // sizes / zero points of the first stages.  They are first touches of their pages in this launch, and once the
@@ -647,31 +642,6 @@ __global__ void tc_wait_expiry_kernel(uint64_t limit_ns) {
   (void)tc_wait(ptx::smem_addr(&bar), 0u, &abort_word, WAIT_SELFTEST, 0, limit_ns);
 }
 
-// Tensor map of a byte matrix [outer, inner_bytes] row-major for copies of box_bytes x box_outer rows laid out in
-// shared memory as they are (no swizzle): the 96-byte boxes of 3-bit codes.
-bool make_tmap_u8_plain(CUtensorMap* tm, const void* base, uint64_t inner_bytes, uint64_t outer, uint32_t box_bytes,
-                        uint32_t box_outer) {
-  using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static const EncodeFn enc = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeFn>(p);
-  }();
-  if (enc == nullptr) return false;
-  const cuuint64_t dims[2] = {inner_bytes, outer};
-  const cuuint64_t strides[1] = {inner_bytes};
-  const cuuint32_t box[2] = {box_bytes, box_outer};
-  const cuuint32_t estr[2] = {1, 1};
-  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int BITS, int PARAM_MODE, bool ZF16>
 int launch_tc_mode(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16, const void* zq,
                    eqat_bf16* Y, int group_shift, int stages, cudaStream_t st) {
@@ -679,8 +649,7 @@ int launch_tc_mode(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, co
   if (!opt_in.ensure(packed_gemv_tc_kernel<BITS, PARAM_MODE, ZF16>, (int)kTcSmemBudget)) return EQAT_ERR_CUDA;
   CUtensorMap mw;
   const uint64_t row_bytes = (uint64_t)d.in_features * BITS / 8;
-  if (!(BITS == 3 ? make_tmap_u8_plain(&mw, Wq, row_bytes, (uint64_t)d.out_features, tc_box_bytes(BITS), kTcRows)
-                  : make_tmap_u8(&mw, Wq, row_bytes, (uint64_t)d.out_features, tc_box_bytes(BITS), kTcRows)))
+  if (!make_tmap_u8(&mw, Wq, row_bytes, (uint64_t)d.out_features, tc_box_bytes(BITS), kTcRows, BITS == 3 ? 0 : 128))
     return EQAT_ERR_CUDA;
   const int sms = sm_count();
   if (sms <= 0) return EQAT_ERR_CUDA;
@@ -732,19 +701,14 @@ int launch_tc(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const e
 
 }  // namespace
 
-// How the tokens go through the kernel: in one launch when the shared-memory plan fits all
-// tokens, otherwise (long rows, or more than eight tokens) as several launches over slices of the tokens, each of
-// which streams the packed weight once more.  That is taken only while it is clearly cheaper than the tiled kernel
-// of gemm.cu.  Cost model (from timings on the Llama-2 7B, 13B and 70B shapes): a launch of this kernel takes about
-// 4 us + 0.5 us per token + the packed weight at 2.25 / 2.6 / 3.5 TB/s (2 / 3 / 4-bit codes; 4 % more per further
-// token); the tiled kernel takes about 1 / 1.45 / 1.2 us per 64 input columns for any token count below a full
-// row-tile, because the K loop of a tile is serial.
-struct TcPlan {
-  int launches, slice;                                   // slice = tokens per launch (the last one may have fewer)
-};
-
-static TcPlan tc_plan(const eqat_desc& d) {
-  const TcPlan none{0, 0};
+// How the tokens go through the kernel: in one launch when the shared-memory plan fits all tokens, otherwise (long rows,
+// or more than eight tokens) as several launches over slices of the tokens, each of which streams the packed weight
+// once more.  `us` is the expected time, from timings on the Llama-2 7B, 13B and 70B shapes: a launch takes about 2.8 us,
+// the staging of the activations (1 us per 8192 values) and the packed weight at 2.25 / 2.6 / 3.5 TB/s (2 / 3 / 4-bit
+// codes; 4 % more per further token).
+FewTokenPlan packed_gemv_plan(const eqat_desc& d) {
+  const FewTokenPlan none{0, 0, 0.0};
+  // a 64-column chunk must lie inside one group: groups of 32 go elsewhere
   if (d.bits < 2 || d.bits > 4 || d.group < 64 || d.tokens < 1 || d.tokens > kTcMaxTotalTokens) return none;
   if (((int64_t)d.in_features * d.bits / 8) % 16 != 0) return none;    // the copy engine wants rows of 16-byte multiples
   const int T = (int)d.tokens;
@@ -752,19 +716,18 @@ static TcPlan tc_plan(const eqat_desc& d) {
   while (fit >= 1 && tc_stages_that_fit(fit, d.in_features, d.bits) == 0) --fit;
   if (fit < 1) return none;
   const int launches = (T + fit - 1) / fit, slice = (T + launches - 1) / launches;
-  if (launches > 1) {
-    const double weight_mb = (double)d.out_features * d.in_features * d.bits / 8.0 / 1.0e6;
-    const double stream_tbs = d.bits == 2 ? 2.25 : (d.bits == 3 ? 2.6 : 3.5);
-    const double tiled_us = d.in_features / 64.0 * (d.bits == 2 ? 1.0 : (d.bits == 3 ? 1.45 : 1.2));
-    const double few_us = launches * (4.0 + 0.5 * slice + weight_mb / stream_tbs * (1.0 + 0.04 * (slice - 1)));
-    if (few_us >= 0.8 * tiled_us) return none;
-  }
-  return TcPlan{launches, slice};
+  const double weight_mb = (double)d.out_features * d.in_features * d.bits / 8.0 / 1.0e6;
+  const double stream_tbs = d.bits == 2 ? 2.25 : (d.bits == 3 ? 2.6 : 3.5);
+  const double us = launches * (2.8 + slice * (d.in_features / 8192.0) + weight_mb / stream_tbs * (1.0 + 0.04 * (slice - 1)));
+  return FewTokenPlan{launches, slice, us};
 }
 
 bool packed_gemv_applies(const eqat_desc& d) {
-  // a 64-column chunk must lie inside one group: groups of 32 go through the tiled kernel
-  return d.tokens >= 1 && d.group >= 64 && tc_plan(d).launches > 0;
+  const FewTokenPlan plan = packed_gemv_plan(d);
+  if (plan.launches <= 1) return plan.launches == 1;
+  // several launches only while clearly cheaper than the tiled kernel, which takes about 1 / 1.45 / 1.2 us per 64 input
+  // columns for any token count below a full row-tile, because the K loop of a tile is serial
+  return plan.us < 0.8 * (d.in_features / 64.0 * (d.bits == 2 ? 1.0 : (d.bits == 3 ? 1.45 : 1.2)));
 }
 
 int launch_packed_gemv(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16,
@@ -774,7 +737,7 @@ int launch_packed_gemv(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq
     group_shift = 0;
     while ((1 << group_shift) < d.group) ++group_shift;
   }
-  const TcPlan plan = tc_plan(d);
+  const FewTokenPlan plan = packed_gemv_plan(d);
   if (plan.launches > 0) {
     for (int t0 = 0; t0 < (int)d.tokens; t0 += plan.slice) {
       eqat_desc part = d;

@@ -5,6 +5,14 @@
 
 namespace eqat {
 
+// How the few-token kernel would take a problem: launches over slices of `slice` tokens (0: not at all), and the
+// expected time.
+struct FewTokenPlan {
+  int launches, slice;
+  double us;
+};
+FewTokenPlan packed_gemv_plan(const eqat_desc& d);
+
 // True when the few-token kernel handles this problem: groups of at least 64 elements, at most 64 tokens, staged
 // activations of at least one token that fit in the shared memory of a CTA, and, where the tokens need several
 // launches, a cost estimate below the tiled kernel's.

@@ -660,6 +660,38 @@ def test_few_token_forwards_back_to_back_keep_their_order(eqat, bits, group, tok
     assert eqat.device_status() == (0, 0)
 
 
+@pytest.mark.parametrize("out,in_f,tokens,bits,group,real_z", [
+    (64, 128, 9, 2, 128, False),     # one run of 128 codes, half a row tile, half a stage
+    (64, 128, 16, 4, 32, True),      # four groups and four sums of the activations per run
+    (320, 384, 17, 3, 64, False),    # three runs: the second stage half empty; 32 token columns
+    (192, 640, 33, 2, 64, True),     # fp16 zero points cap a tile at 32 token columns: two token tiles
+    (576, 1408, 48, 4, 128, False),  # odd groups per row, three groups of row threads
+    (1088, 4096, 64, 3, 4096, False),   # one group per row, 64 token columns, K split over a cluster
+    (128, 4352, 64, 2, 64, False),   # 34 runs over eight CTAs of a cluster: slices of four and six runs
+    (4096, 4096, 10, 2, 32, False),  # a cluster of eight per row tile, two CTAs per SM
+    (9472, 1024, 24, 4, 256, True),  # more CTAs than fit at a time, groups of two runs
+    (2048, 8192, 8, 4, 128, False),  # eight tokens: cheaper than the matrix-vector kernel's two launches
+    (64, 28672, 40, 3, 64, False),   # the longest rows
+])
+def test_packed_forward_on_weight_row_tiles(eqat, out, in_f, tokens, bits, group, real_z):
+    """The kernel on tiles of 128 weight rows (up to 64 tokens): nothing is rounded on the way to the fp32 sums, so beside
+    the usual checks the forward is within the rounding of its results to bf16, 2^-9 of each, and 2 % for the sums."""
+    cfg = small_cfg(f"slim_{out}_{in_f}_{tokens}", out, in_f, bits, group, tokens, "student_t4", 0.02, 0.01)
+    r = run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z)
+    check_e2e(r, group)
+    What_o = O.dequantize(r["q"], r["s16"], r["z8"], group, real_zero_point=real_z)
+    assert rel_err(torch_to_f64(r["Y"]), O.linear_fwd(r["X"], What_o)) <= 1.02 * 2.0 ** -9
+    again = run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z)
+    assert torch.equal(r["Y"].view(torch.int16), again["Y"].view(torch.int16))
+    assert eqat.device_status() == (0, 0)
+
+
+def test_weight_row_kernel_wait_runs_out_cleanly(eqat):
+    eqat.eqat_selftest_wait_expiry(3)
+    assert eqat.device_status() == (eqat.EQAT_ERR_TIMEOUT, 9)
+    assert eqat.device_status() == (0, 0)
+
+
 @pytest.mark.parametrize("out,in_f,tokens,bits,group", [
     (192, 384, 300, 2, 64),
     (64, 128, 1, 4, 128),
