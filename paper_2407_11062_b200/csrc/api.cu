@@ -6,6 +6,7 @@
 #include "gemm.cuh"
 #include "gemv.cuh"
 #include "slim.cuh"
+#include "wide.cuh"
 
 namespace {
 
@@ -152,13 +153,14 @@ size_t eqat_workspace_bytes(const eqat_desc* d, int op) {
 
 int eqat_device_status(int* h_status, int* h_detail) {
   if (h_status == nullptr) return EQAT_ERR_NULL;
-  int st[4] = {0, 0, 0, 0}, det[4] = {0, 0, 0, 0};
+  int st[5] = {0, 0, 0, 0, 0}, det[5] = {0, 0, 0, 0, 0};
   EQAT_TRY(read_device_status(&st[0], &det[0]));      // GEMM kernels
   EQAT_TRY(read_stream_status(&st[1], &det[1]));      // staged streaming kernels
   EQAT_TRY(read_gemv_status(&st[2], &det[2]));        // matrix-vector kernels
-  EQAT_TRY(read_slim_status(&st[3], &det[3]));        // weight-row kernels
+  EQAT_TRY(read_slim_status(&st[3], &det[3]));        // weight-row kernels: few tokens,
+  EQAT_TRY(read_wide_status(&st[4], &det[4]));        // prompts
   int k = 0;
-  while (k < 3 && st[k] == EQAT_OK) ++k;
+  while (k < 4 && st[k] == EQAT_OK) ++k;
   *h_status = st[k];
   if (h_detail != nullptr) *h_detail = det[k];
   return EQAT_OK;
@@ -169,6 +171,7 @@ int eqat_selftest_wait_expiry(int which, void* stream) {
   if (which == 1) return launch_wait_expiry_stream(as_stream(stream));
   if (which == 2) return launch_wait_expiry_gemv(as_stream(stream));
   if (which == 3) return launch_wait_expiry_slim(as_stream(stream));
+  if (which == 4) return launch_wait_expiry_wide(as_stream(stream));
   return EQAT_ERR_UNSUPPORTED;
 }
 
@@ -259,6 +262,8 @@ int qlinear_packed_fwd(const eqat_desc* d, const eqat_bf16* X, const uint8_t* Wq
   if (slim_fwd_applies(*d, plan)) return launch_slim_fwd(*d, X, Wq_packed, s16, z, Y, plan, as_stream(stream));
   // a handful of tokens (decoding): one pass over the packed weight instead of near-empty tensor-core tiles
   if (packed_gemv_applies(*d)) return launch_packed_gemv(*d, X, Wq_packed, s16, z, Y, as_stream(stream));
+  WidePlan wide;
+  if (wide_fwd_applies(*d, wide)) return launch_wide_fwd(*d, X, Wq_packed, s16, z, Y, wide, as_stream(stream));
   return launch_packed_fwd(*d, X, Wq_packed, s16, z, Y, as_stream(stream));
 }
 

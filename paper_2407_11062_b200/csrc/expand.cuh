@@ -90,48 +90,35 @@ struct GroupValues<2> {
   }
 };
 
-__device__ __forceinline__ void store_chunk(uint32_t row_sx, int chunk, const float (&v)[8]) {
-  ptx::sts_128(row_sx ^ ((uint32_t)chunk << 4), pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
-               pack_bf16x2(v[6], v[7]));
-}
-
-// Expands 32 consecutive codes (half h of a 64-code row) into chunks 4h .. 4h+3.
+// 32 consecutive codes as 16 registers of bf16 pairs, (q - z) * s rounded once, in the order of the stream.
 template <int BITS>
-__device__ __forceinline__ void dequant_half32(const uint32_t (&w)[BITS], const GroupValues<BITS>& f, uint32_t row_sx, int h) {
+__device__ __forceinline__ void values32(const uint32_t* w, const GroupValues<BITS>& f, uint32_t* o) {
   constexpr uint32_t kMagic = 0x4B000000u;
   if constexpr (BITS == 2) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {                       // word i: codes 16i .. 16i+15 of the half
+    for (int i = 0; i < 2; ++i) {                       // word i: codes 16i .. 16i+15
       uint32_t sel[4];                                  // byte b of sel[r] = selector byte of code 4b + r
 #pragma unroll
       for (int r = 0; r < 4; ++r) sel[r] = ((w[i] >> (2 * r)) & 0x03030303u) * 0x22u + 0x10101010u;
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        uint32_t o[4];
-#pragma unroll
-        for (int pr = 0; pr < 4; ++pr) {
-          const int k = 8 * c + 2 * pr;                 // even code of the pair; k = 4b + r with r in {0, 2}
-          const uint32_t b = (uint32_t)(k >> 2), r = (uint32_t)(k & 3);
-          const uint32_t pair_sel = __byte_perm(sel[r], sel[r + 1], b | ((4u + b) << 4));
-          o[pr] = __byte_perm(f.lut01, f.lut23, pair_sel);
-        }
-        ptx::sts_128(row_sx ^ ((uint32_t)(4 * h + 2 * i + c) << 4), o[0], o[1], o[2], o[3]);
+      for (int pr = 0; pr < 8; ++pr) {
+        const uint32_t b = (uint32_t)(pr >> 1), r = (uint32_t)((2 * pr) & 3);   // even code 2pr = 4b + r, r in {0, 2}
+        o[8 * i + pr] = __byte_perm(f.lut01, f.lut23, __byte_perm(sel[r], sel[r + 1], b | ((4u + b) << 4)));
       }
     }
   } else if constexpr (BITS == 4) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {                       // word i: codes 8i .. 8i+7 of the half
+    for (int i = 0; i < 4; ++i) {                       // word i: codes 8i .. 8i+7
       const uint32_t m0 = w[i] & 0x0F0F0F0Fu, m1 = (w[i] >> 4) & 0x0F0F0F0Fu;   // byte b = code 2b (+1)
-      float v[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e)
-        v[e] = f(__byte_perm((e & 1) ? m1 : m0, kMagic, 0x7044u | ((uint32_t)(e >> 1) << 8)));
-      store_chunk(row_sx, 4 * h + i, v);
+      for (int b = 0; b < 4; ++b)
+        o[4 * i + b] = pack_bf16x2(f(__byte_perm(m0, kMagic, 0x7044u | ((uint32_t)b << 8))),
+                                   f(__byte_perm(m1, kMagic, 0x7044u | ((uint32_t)b << 8))));
     }
   } else {
     // 32 codes = 3 words = 96 bits, code j at bit 3j.  Triple m (codes 3m .. 3m+2) is brought to bits 12..20 of a
     // register by one shift of the stream: the 32-bit window that starts at bit 9m - 12.
-    float v[32];
+    float v[33];
 #pragma unroll
     for (int m = 0; m < 11; ++m) {
       const int start = 9 * m - 12;
@@ -148,8 +135,18 @@ __device__ __forceinline__ void dequant_half32(const uint32_t (&w)[BITS], const 
         if (3 * m + k < 32) v[3 * m + k] = f.at(k, win);
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) store_chunk(row_sx, 4 * h + c, *reinterpret_cast<const float(*)[8]>(v + 8 * c));
+    for (int i = 0; i < 16; ++i) o[i] = pack_bf16x2(v[2 * i], v[2 * i + 1]);
   }
+}
+
+// Expands 32 consecutive codes (half h of a 64-code row) into chunks 4h .. 4h+3.
+template <int BITS>
+__device__ __forceinline__ void dequant_half32(const uint32_t (&w)[BITS], const GroupValues<BITS>& f, uint32_t row_sx, int h) {
+  uint32_t o[16];
+  values32<BITS>(w, f, o);
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    ptx::sts_128(row_sx ^ ((uint32_t)(4 * h + c) << 4), o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
 }
 
 // 64 codes = 2*BITS consecutive 32-bit words, at a multiple of 8*BITS bytes.

@@ -14,7 +14,7 @@ bool make_tmap_bf16(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t 
 bool make_tmap_blocks_bf16(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t outer, uint32_t box_outer,
                            uint32_t blocks);
 // Tensor map of a byte matrix [outer, inner_bytes] row-major for copies of box_bytes (a multiple of 16, at most
-// swizzle_bytes) x box_outer rows, swizzled by 128 or 64 bytes or (0) not at all; bytes outside the matrix are delivered
+// swizzle_bytes) x box_outer rows, swizzled by 128, 64 or 32 bytes or (0) not at all; bytes outside the matrix are delivered
 // as zeros.
 bool make_tmap_u8(CUtensorMap* tm, const void* base, uint64_t inner_bytes, uint64_t outer, uint32_t box_bytes,
                   uint32_t box_outer, uint32_t swizzle_bytes);

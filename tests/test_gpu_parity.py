@@ -686,8 +686,28 @@ def test_packed_forward_on_weight_row_tiles(eqat, out, in_f, tokens, bits, group
     assert eqat.device_status() == (0, 0)
 
 
-def test_weight_row_kernel_wait_runs_out_cleanly(eqat):
-    eqat.eqat_selftest_wait_expiry(3)
+@pytest.mark.parametrize("out,in_f,tokens,bits,group,real_z", [
+    (64, 512, 65, 2, 64, False),      # one row tile of a pair, half of it; the other CTA has no rows
+    (320, 640, 96, 3, 32, True),      # four groups per run of 128 codes, five runs over a split of K
+    (576, 1408, 129, 4, 128, False),  # odd groups per row, a ragged last token
+    (1024, 4096, 256, 2, 256, False), # one full token tile, eight CTAs per cluster
+    (1088, 8192, 257, 4, 8192, False),   # one group per row, one token more than a tile
+    (4096, 1024, 700, 3, 64, True),   # several token tiles, more clusters than fit at a time
+    (11008, 512, 333, 2, 64, False),  # four runs: every group of row threads gets one
+])
+def test_packed_forward_for_prompts(eqat, out, in_f, tokens, bits, group, real_z):
+    """The kernel on pairs of weight-row tiles, against the oracle and against itself."""
+    cfg = small_cfg(f"wide_{out}_{in_f}_{tokens}", out, in_f, bits, group, tokens, "student_t4", 0.02, 0.01)
+    r = run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z)
+    check_e2e(r, group)
+    again = run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z)
+    assert torch.equal(r["Y"].view(torch.int16), again["Y"].view(torch.int16))
+    assert eqat.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("which", [3, 4])
+def test_weight_row_kernels_wait_runs_out_cleanly(eqat, which):
+    eqat.eqat_selftest_wait_expiry(which)
     assert eqat.device_status() == (eqat.EQAT_ERR_TIMEOUT, 9)
     assert eqat.device_status() == (0, 0)
 
