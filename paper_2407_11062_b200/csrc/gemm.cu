@@ -23,7 +23,7 @@
 // MT = 2 feeds two MMAs from each B stage):
 //   warp 0      TMA producer: fills a ring of 128B-swizzled shared-memory stages;
 //               in a pair the bytes are counted on the first CTA's barrier
-//   warp 1      MMA issuer (first CTA of a pair only): one thread issues tcgen05.mma,
+//   warp 1      MMA issuer (first CTA of a pair only): an elected lane issues tcgen05.mma,
 //               frees stages in both CTAs with tcgen05.commit; owns the TMEM allocation
 //   warps 2-5   epilogue: tcgen05.ld the finished accumulator (one TMEM lane
 //               quadrant each)
@@ -581,7 +581,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (first CTA of a pair)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((A_MN ? 1u : 0u) << 15) |
                                  ((B_MN ? 1u : 0u) << 16) | ((uint32_t)(BN >> 3) << 17) |
                                  ((uint32_t)((C::kCtas * BM) >> 4) << 24);
@@ -609,33 +609,40 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
             break;
           }
           ptx::tc_fence_after();
-          const uint32_t a_addr = smem_base + C::a_offset(stage);
-          const uint32_t b_addr = smem_base + C::b_offset(PACKED ? stage_b : stage);
+          if (ptx::elect_one()) {
+            const uint32_t a_addr = smem_base + C::a_offset(stage);
+            const uint32_t b_addr = smem_base + C::b_offset(PACKED ? stage_b : stage);
 #pragma unroll
-          for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-            const uint64_t b_desc = smem_desc(b_addr + kk * b_step, b_lbo);
+            for (int kk = 0; kk < BK / UMMA_K; ++kk) {
+              const uint64_t b_desc = smem_desc(b_addr + kk * b_step, b_lbo);
 #pragma unroll
-            for (int h = 0; h < MT; ++h) {
-              const uint64_t a_desc = smem_desc(a_addr + h * a_half + kk * a_step, a_lbo);
-              if (PAIR) ptx::mma_bf16_ss_pair(d_tmem + h * BN, a_desc, b_desc, idesc, (kb | kk) != 0 ? 1u : 0u);
-              else ptx::mma_bf16_ss(d_tmem + h * BN, a_desc, b_desc, idesc, (kb | kk) != 0 ? 1u : 0u);
+              for (int h = 0; h < MT; ++h) {
+                const uint64_t a_desc = smem_desc(a_addr + h * a_half + kk * a_step, a_lbo);
+                if (PAIR) ptx::mma_bf16_ss_pair(d_tmem + h * BN, a_desc, b_desc, idesc, (kb | kk) != 0 ? 1u : 0u);
+                else ptx::mma_bf16_ss(d_tmem + h * BN, a_desc, b_desc, idesc, (kb | kk) != 0 ? 1u : 0u);
+              }
             }
+            commit_both(ptx::smem_addr(&ctl->empty[stage]));
+            if (PACKED) commit_both(ptx::smem_addr(&ctl->empty_b[stage_b]));
           }
-          commit_both(ptx::smem_addr(&ctl->empty[stage]));
+          __syncwarp();
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
           if (PACKED) {
-            commit_both(ptx::smem_addr(&ctl->empty_b[stage_b]));
             if (++stage_b == C::kStagesB) { stage_b = 0; phase_b ^= 1u; }
           }
         }
         if (!ok) break;
-        commit_both(ptx::smem_addr(&ctl->acc_full[acc]));
+        if (ptx::elect_one()) commit_both(ptx::smem_addr(&ctl->acc_full[acc]));
+        __syncwarp();
         if (++acc == C::kAccSets) { acc = 0; acc_phase ^= 1u; }
       }
       // All MMAs of this thread must have retired before TMEM is freed (and, in a pair, before either CTA leaves:
       // the commits above signal barriers in both).
-      if (PAIR) ptx::mma_commit_pair(ptx::smem_addr(&ctl->drain));
-      else ptx::mma_commit(ptx::smem_addr(&ctl->drain));
+      if (ptx::elect_one()) {
+        if (PAIR) ptx::mma_commit_pair(ptx::smem_addr(&ctl->drain));
+        else ptx::mma_commit(ptx::smem_addr(&ctl->drain));
+      }
+      __syncwarp();
       wait_bounded(ptx::smem_addr(&ctl->drain), 0u, abort_flag, WAIT_TEARDOWN, 64, kDrainLimitNs * 4);
     }
   } else if (!PACKED) {
