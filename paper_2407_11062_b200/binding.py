@@ -94,16 +94,24 @@ def make_desc(bits, group, out_features, in_features, tokens=0, dz_mode=0, zero_
                      int(zero_point_format))
 
 
+# Addresses and the stream go to the library as plain integers (the argtypes make pointers of them), and the stream is
+# asked of the runtime without a torch.cuda.Stream object around it (0.3 instead of 3 to 4 us per call): a decoding step
+# is a call of a few microseconds per layer, and marshalling was more than half of its host time.
 def _ptr(t):
     if t is None:
         return None
-    if not t.is_cuda or not t.is_contiguous():
+    if not (t.is_cuda and t.is_contiguous()):
         raise ValueError("expected a contiguous CUDA tensor")
-    return c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+_raw_stream, _device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream():
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is None or _device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
 
 
 def _check(rc, where):
@@ -205,11 +213,6 @@ def qlinear_packed_bwd_ds(desc, X, dY, Wq_packed, z8, s16, ds, dz=None, workspac
            "qlinear_packed_bwd_ds")
 
 
-def _addr(t):
-    p = _ptr(t)
-    return None if p is None else p.value
-
-
 def _nbytes(t):
     return 0 if t is None else t.numel() * t.element_size()
 
@@ -225,9 +228,9 @@ def _run_block(fn, struct, rows, where):
 def eqat_block_ap_step(linears):
     """Block-AP forward + backward of every linear of a block in one call.  `linears`: dicts with desc, X, dY, W,
     s, z, Y, W_hat (or None), dX, dW, ds, dz (or None), workspace (or None)."""
-    rows = [eqat_block_ap_linear(L["desc"], _addr(L["X"]), _addr(L["dY"]), _addr(L["W"]), _addr(L["s"]), _addr(L["z"]),
-                                 _addr(L["Y"]), _addr(L.get("W_hat")), _addr(L["dX"]), _addr(L["dW"]), _addr(L["ds"]),
-                                 _addr(L.get("dz")), _addr(L.get("workspace")), _nbytes(L.get("workspace")))
+    rows = [eqat_block_ap_linear(L["desc"], _ptr(L["X"]), _ptr(L["dY"]), _ptr(L["W"]), _ptr(L["s"]), _ptr(L["z"]),
+                                 _ptr(L["Y"]), _ptr(L.get("W_hat")), _ptr(L["dX"]), _ptr(L["dW"]), _ptr(L["ds"]),
+                                 _ptr(L.get("dz")), _ptr(L.get("workspace")), _nbytes(L.get("workspace")))
             for L in linears]
     _run_block(lib.eqat_block_ap_step, eqat_block_ap_linear, rows, "eqat_block_ap_step")
 
@@ -235,8 +238,8 @@ def eqat_block_ap_step(linears):
 def eqat_e2e_qp_step(linears):
     """E2E-QP forward, dX and ds (dz) of every linear of a block in one call.  `linears`: dicts with desc, X, dY,
     Wq_packed, s16, z, Y, dX, ds, dz (or None), workspace (or None)."""
-    rows = [eqat_e2e_qp_linear(L["desc"], _addr(L["X"]), _addr(L["dY"]), _addr(L["Wq_packed"]), _addr(L["s16"]),
-                               _addr(L["z"]), _addr(L["Y"]), _addr(L["dX"]), _addr(L["ds"]), _addr(L.get("dz")),
-                               _addr(L.get("workspace")), _nbytes(L.get("workspace")))
+    rows = [eqat_e2e_qp_linear(L["desc"], _ptr(L["X"]), _ptr(L["dY"]), _ptr(L["Wq_packed"]), _ptr(L["s16"]),
+                               _ptr(L["z"]), _ptr(L["Y"]), _ptr(L["dX"]), _ptr(L["ds"]), _ptr(L.get("dz")),
+                               _ptr(L.get("workspace")), _nbytes(L.get("workspace")))
             for L in linears]
     _run_block(lib.eqat_e2e_qp_step, eqat_e2e_qp_linear, rows, "eqat_e2e_qp_step")
