@@ -1,9 +1,6 @@
-// Streaming (HBM-bound) kernels: fake quantiser, its straight-through
-// backward with per-group reductions, min/max initialisation and the N-bit
-// codec.  Every kernel moves 16-byte vectors with fully coalesced accesses; a
-// quantisation group (contiguous along in_features, hence contiguous in the
-// flattened weight) is owned by group/8 adjacent lanes of one warp, so group
-// sums are fixed-order warp shuffles and the results are run-to-run identical.
+// Streaming (HBM-bound) kernels beside the TMA-staged ones of stream.cu: the
+// straight-through backward and the min/max initialisation of groups longer
+// than 256 elements (a block per group, fixed-order sums) and the N-bit codec.
 #include "common.cuh"
 #include "codec.cuh"
 #include "elementwise.cuh"
@@ -44,41 +41,6 @@ __device__ __forceinline__ void quant_terms(float w, float s, float zr, float& t
   t = __fdiv_rn(w, s);
   r = rintf(t);
   p = r + zr;
-}
-
-__device__ __forceinline__ float clamp_code(float p, float Q) { return fminf(fmaxf(p, 0.0f), Q); }
-
-// ------------------------------------------------------------------ Eq. 1 + Eq. 2
-// (used for groups longer than 256 elements; shorter groups take the staged kernel in stream.cu)
-__global__ void __launch_bounds__(kThreads)
-fakequant_kernel(const eqat_bf16* __restrict__ W, const float* __restrict__ s, const float* __restrict__ z,
-                 eqat_bf16* __restrict__ What, size_t n_vec, uint32_t vec_per_group, float Q) {
-  const size_t base = (size_t)blockIdx.x * (kThreads * 2) + threadIdx.x;
-  const size_t vi[2] = {base, base + kThreads};
-  Vec8 w[2];
-  float sv[2], zv[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    if (vi[u] < n_vec) {
-      w[u] = load_bf16x8(W, vi[u]);
-      const uint32_t g = (uint32_t)vi[u] / vec_per_group;
-      sv[u] = __ldg(s + g);
-      zv[u] = rintf(__ldg(z + g));
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    if (vi[u] < n_vec) {
-      Vec8 o;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        float t, r, p;
-        quant_terms(w[u].v[i], sv[u], zv[u], t, r, p);
-        o.v[i] = (clamp_code(p, Q) - zv[u]) * sv[u];
-      }
-      store_bf16x8(What, vi[u], o);
-    }
-  }
 }
 
 // ------------------------------------------------------------------ Eqs. 3-5 + group sums
@@ -192,38 +154,6 @@ __device__ __forceinline__ void load_words(const uint8_t* packed, size_t chunk, 
   }
 }
 
-// One thread quantises 32 consecutive weights (one 64-byte run) and emits their packed words.
-template <int BITS>
-__global__ void __launch_bounds__(kThreads)
-quantize_pack_kernel(const eqat_bf16* __restrict__ W, const float* __restrict__ s, const float* __restrict__ z,
-                     uint8_t* __restrict__ packed, uint8_t* __restrict__ z8, eqat_fp16* __restrict__ s16,
-                     size_t n_chunk, uint32_t chunk_per_group) {
-  const size_t c = (size_t)blockIdx.x * kThreads + threadIdx.x;
-  if (c >= n_chunk) return;
-  constexpr float Q = (float)((1 << BITS) - 1);
-  const uint32_t g = (uint32_t)c / chunk_per_group;
-  const float sv = __ldg(s + g);
-  const float zr = rintf(__ldg(z + g));
-  uint32_t codes[32];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const Vec8 w = load_bf16x8(W, c * 4 + k);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      float t, r, p;
-      quant_terms(w.v[i], sv, zr, t, r, p);
-      codes[8 * k + i] = (uint32_t)clamp_code(p, Q);
-    }
-  }
-  uint32_t words[BITS];
-  pack32<BITS>(codes, words);
-  store_words<BITS>(packed, c, words);
-  if ((uint32_t)c % chunk_per_group == 0) {
-    z8[g] = (uint8_t)clamp_code(zr, Q);
-    s16[g] = __half_as_ushort(__float2half_rn(sv));
-  }
-}
-
 template <int BITS>
 __global__ void __launch_bounds__(kThreads)
 pack_kernel(const uint8_t* __restrict__ codes8, uint8_t* __restrict__ packed, size_t n_chunk) {
@@ -294,16 +224,6 @@ inline unsigned blocks_for(size_t items, size_t per_block) { return (unsigned)((
 }  // namespace
 
 // ------------------------------------------------------------------ host launchers
-int launch_fakequant(const eqat_desc& d, const eqat_bf16* W, const float* s, const float* z, eqat_bf16* What,
-                     cudaStream_t st) {
-  if (d.group <= 256) return launch_fakequant_stream(d, W, s, z, What, st);
-  const size_t n_vec = (size_t)d.out_features * d.in_features / 8;
-  const float Q = (float)((1 << d.bits) - 1);
-  fakequant_kernel<<<blocks_for(n_vec, kThreads * 2), kThreads, 0, st>>>(W, s, z, What, n_vec,
-                                                                         (uint32_t)d.group / 8, Q);
-  return launch_status();
-}
-
 int launch_ste_bwd(const eqat_desc& d, const eqat_bf16* dWhat, const eqat_bf16* W, const float* s, const float* z,
                    eqat_bf16* dW, float* ds, float* dz, cudaStream_t st) {
   if (d.group <= 256) return launch_ste_bwd_stream(d, dWhat, W, s, z, dW, ds, dz, st);
@@ -319,20 +239,6 @@ int launch_minmax(const eqat_desc& d, const eqat_bf16* W, float* s, float* z, cu
   const float Q = (float)((1 << d.bits) - 1);
   const size_t n_groups = (size_t)d.out_features * d.in_features / d.group;
   minmax_long_group_kernel<<<(unsigned)n_groups, kThreads, 0, st>>>(W, s, z, d.group / 8, Q);
-  return launch_status();
-}
-
-int launch_quantize_pack(const eqat_desc& d, const eqat_bf16* W, const float* s, const float* z, uint8_t* packed,
-                         uint8_t* z8, eqat_fp16* s16, cudaStream_t st) {
-  if (d.group <= 256) return launch_quantize_pack_stream(d, W, s, z, packed, z8, s16, st);
-  const size_t n_chunk = (size_t)d.out_features * d.in_features / 32;
-  const unsigned nb = blocks_for(n_chunk, kThreads);
-  const uint32_t cpg = (uint32_t)d.group / 32;
-  switch (d.bits) {
-    case 2: quantize_pack_kernel<2><<<nb, kThreads, 0, st>>>(W, s, z, packed, z8, s16, n_chunk, cpg); break;
-    case 3: quantize_pack_kernel<3><<<nb, kThreads, 0, st>>>(W, s, z, packed, z8, s16, n_chunk, cpg); break;
-    default: quantize_pack_kernel<4><<<nb, kThreads, 0, st>>>(W, s, z, packed, z8, s16, n_chunk, cpg); break;
-  }
   return launch_status();
 }
 

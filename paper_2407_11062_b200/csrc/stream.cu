@@ -1,6 +1,6 @@
-// Streaming kernels with TMA-staged inputs: fake quantiser (Eq. 1 + Eq. 2), its
-// straight-through backward (Eqs. 3-5), min/max initialisation and quantise +
-// pack, for groups of at most 256 elements.
+// Streaming kernels with TMA-staged inputs: fake quantiser (Eq. 1 + Eq. 2) and
+// quantise + pack for every group length; the straight-through backward
+// (Eqs. 3-5) and the min/max initialisation for groups of at most 256 elements.
 //
 // These kernels move 2-6 bytes per element and would be bound by HBM bandwidth
 // if the instruction stream per element were short enough; at 10-25 executed
@@ -195,12 +195,22 @@ struct GroupParams {
   float s, z;
 };
 
+// Group of a lane's elements.  Groups of up to 256 elements are powers of two; a longer one is any multiple of a lane's
+// 32 elements, and one 32-bit division per lane and tile finds it (a weight has at most 2^34 elements).
+template <bool LONG>
+__device__ __forceinline__ size_t group_index(size_t e0, int group) {
+  return LONG ? (size_t)((uint32_t)(e0 >> 5) / (uint32_t)group) : e0 >> group;
+}
+
+// `group`: log2 of the group length, or (LONG) the length in units of 32 elements.
+template <bool LONG = false>
 __device__ __forceinline__ GroupParams fetch_group(const float* __restrict__ s, const float* __restrict__ z, size_t e0,
-                                                   size_t n_elem, int group_shift) {
+                                                   size_t n_elem, int group) {
   GroupParams p{1.0f, 0.0f};
   if (e0 < n_elem) {
-    p.s = __ldg(s + (e0 >> group_shift));
-    p.z = __ldg(z + (e0 >> group_shift));
+    const size_t g = group_index<LONG>(e0, group);
+    p.s = __ldg(s + g);
+    p.z = __ldg(z + g);
   }
   return p;
 }
@@ -221,13 +231,14 @@ __device__ __forceinline__ void store_lane(eqat_bf16* dst, const uint4 (&o)[4], 
 
 // ------------------------------------------------------------------ Eq. 1 + Eq. 2
 // (clamp(r + z, 0, Q) - z) * s == clamp(r, -z, Q - z) * s for integer r and z.
+template <bool LONG>
 __global__ void __launch_bounds__(kThreadsS, kCtas1)
 fakequant_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* __restrict__ s,
-                        const float* __restrict__ z, eqat_bf16* __restrict__ What, size_t n_elem, int group_shift,
+                        const float* __restrict__ z, eqat_bf16* __restrict__ What, size_t n_elem, int group,
                         float Q, int wide) {
   const CUtensorMap* const maps[1] = {&map_w};
   stream_tiles<1, kStages1, GroupParams>(maps, n_elem,
-      [&](size_t e0) { return fetch_group(s, z, e0, n_elem, group_shift); },
+      [&](size_t e0) { return fetch_group<LONG>(s, z, e0, n_elem, group); },
       [&](size_t e0, const uint4 (&raw)[1][4], const GroupParams& gp) {
     if (e0 >= n_elem) return;
     const float sv = gp.s;
@@ -241,7 +252,10 @@ fakequant_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* 
       unpack8(raw[0][u], w);
       quotient_round8(w, sv, rs, r, rt);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) w[i] = fminf(fmaxf(r[i], lo), hi) * sv;
+      for (int i = 0; i < 8; ++i) {
+        const float c = fminf(fmaxf(r[i], lo), hi);
+        w[i] = LONG ? fmaf(c, sv, 0.0f) : c * sv;         // (LONG: a zero is always +0)
+      }
       o[u] = pack8(w);
     }
     store_lane(What + e0, o, wide != 0);
@@ -373,18 +387,18 @@ minmax_stream_kernel(const __grid_constant__ CUtensorMap map_w, float* __restric
 // is redone with the defining sequence.  Two multiply-adds and one logic
 // operation per element, and the clamped t feeds the bit packing directly: its
 // low bits ARE the code.
-template <int BITS>
+template <int BITS, bool LONG>
 __global__ void __launch_bounds__(kThreadsS, kCtas1)
 quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* __restrict__ s,
                             const float* __restrict__ z, uint8_t* __restrict__ packed, uint8_t* __restrict__ z8,
-                            eqat_fp16* __restrict__ s16, size_t n_elem, int group_shift) {
+                            eqat_fp16* __restrict__ s16, size_t n_elem, int group) {
   const CUtensorMap* const maps[1] = {&map_w};
   constexpr float Q = (float)((1 << BITS) - 1);
   constexpr float kTwo23 = 8388608.0f;
   // sum over the 8 codes of a vector of the bit pattern of 2^23 shifted to the code's place (mod 2^32)
   constexpr uint32_t kBias = (uint32_t)(0x4B000000ull * (((1ull << (8 * BITS)) - 1ull) / ((1ull << BITS) - 1ull)));
   stream_tiles<1, kStages1, GroupParams>(maps, n_elem,
-      [&](size_t e0) { return fetch_group(s, z, e0, n_elem, group_shift); },
+      [&](size_t e0) { return fetch_group<LONG>(s, z, e0, n_elem, group); },
       [&](size_t e0, const uint4 (&raw)[1][4], const GroupParams& gp) {
     if (e0 >= n_elem) return;
     const float sv = gp.s;
@@ -425,8 +439,8 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
         acc = (acc << BITS) + __float_as_uint(fminf(fmaxf(t[i], kTwo23), kTwo23 + Q));
       piece[u] = acc - kBias;
     }
-    if ((e0 & (((size_t)1 << group_shift) - 1)) == 0) {
-      const size_t g = e0 >> group_shift;
+    const size_t g = group_index<LONG>(e0, group);
+    if (e0 == (LONG ? g * (size_t)group << 5 : g << group)) {          // the group's first lane
       z8[g] = (uint8_t)(__float_as_uint(fminf(fmaxf(zr, 0.0f), Q) + 8388608.0f) & 0xFFu);
       s16[g] = __half_as_ushort(__float2half_rn(sv));
     }
@@ -497,14 +511,17 @@ inline int group_shift_of(int group) {
 
 }  // namespace
 
-int launch_fakequant_stream(const eqat_desc& d, const eqat_bf16* W, const float* s, const float* z, eqat_bf16* What,
+int launch_fakequant(const eqat_desc& d, const eqat_bf16* W, const float* s, const float* z, eqat_bf16* What,
                             cudaStream_t st) {
   const size_t n_elem = (size_t)d.out_features * d.in_features;
   const float Q = (float)((1 << d.bits) - 1);
   CUtensorMap mw;
   if (!weight_map(&mw, W, n_elem)) return EQAT_ERR_CUDA;
-  return launch_stream<fakequant_stream_kernel>(Ring<1, kStages1>::kSmemBytes, n_elem, st, mw, s, z, What, n_elem,
-                                                group_shift_of(d.group), Q, (int)aligned32(What));
+  constexpr int smem = Ring<1, kStages1>::kSmemBytes;
+  const int wide = (int)aligned32(What);
+  if (d.group > 256)
+    return launch_stream<fakequant_stream_kernel<true>>(smem, n_elem, st, mw, s, z, What, n_elem, d.group / 32, Q, wide);
+  return launch_stream<fakequant_stream_kernel<false>>(smem, n_elem, st, mw, s, z, What, n_elem, group_shift_of(d.group), Q, wide);
 }
 
 int launch_ste_bwd_stream(const eqat_desc& d, const eqat_bf16* dWhat, const eqat_bf16* W, const float* s,
@@ -537,17 +554,21 @@ int launch_minmax_stream(const eqat_desc& d, const eqat_bf16* W, float* s, float
   }
 }
 
-int launch_quantize_pack_stream(const eqat_desc& d, const eqat_bf16* W, const float* s, const float* z,
+int launch_quantize_pack(const eqat_desc& d, const eqat_bf16* W, const float* s, const float* z,
                                 uint8_t* packed, uint8_t* z8, eqat_fp16* s16, cudaStream_t st) {
   const size_t n_elem = (size_t)d.out_features * d.in_features;
-  const int gs = group_shift_of(d.group);
+  const bool longer = d.group > 256;
+  const int group = longer ? d.group / 32 : group_shift_of(d.group);
   CUtensorMap mw;
   if (!weight_map(&mw, W, n_elem)) return EQAT_ERR_CUDA;
   constexpr int smem = Ring<1, kStages1>::kSmemBytes;
-  switch (d.bits) {
-    case 2:  return launch_stream<quantize_pack_stream_kernel<2>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, gs);
-    case 3:  return launch_stream<quantize_pack_stream_kernel<3>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, gs);
-    default: return launch_stream<quantize_pack_stream_kernel<4>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, gs);
+  switch (d.bits * 2 + (longer ? 1 : 0)) {
+    case 4:  return launch_stream<quantize_pack_stream_kernel<2, false>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, group);
+    case 5:  return launch_stream<quantize_pack_stream_kernel<2, true>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, group);
+    case 6:  return launch_stream<quantize_pack_stream_kernel<3, false>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, group);
+    case 7:  return launch_stream<quantize_pack_stream_kernel<3, true>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, group);
+    case 8:  return launch_stream<quantize_pack_stream_kernel<4, false>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, group);
+    default: return launch_stream<quantize_pack_stream_kernel<4, true>>(smem, n_elem, st, mw, s, z, packed, z8, s16, n_elem, group);
   }
 }
 

@@ -71,6 +71,18 @@ def test_streaming_kernels_tiny_and_ragged(eqat, out, in_f, bits, group):
     check_streaming_kernels(eqat, bits, group, out, in_f)
 
 
+@pytest.mark.parametrize("out,in_f,bits,group", [
+    (5, 384, 4, 384),         # the shortest long group, twelve lanes: groups start in the middle of a warp
+    (3, 1152, 3, 288),        # nine lanes a group, four groups a row
+    (70, 8192, 2, 4096),      # half a tile of the copy engine per group
+    (33, 16384, 3, 16384),    # two tiles per group
+    (2, 32768, 4, 32768),     # the longest group
+])
+def test_staged_kernels_on_groups_longer_than_256(eqat, out, in_f, bits, group):
+    """Fake quantiser and quantise + pack find a lane's group by a division there."""
+    check_streaming_kernels(eqat, bits, group, out, in_f)
+
+
 def check_streaming_kernels(eqat, bits, group, out, in_f):
     cfg = small_cfg(f"ew_{bits}_{group}", out, in_f, bits, group, 0, "student_t4", 0.02, 0.01)
     Wb = weight_for(cfg, cfg.linears[0]); W32 = f32(Wb)
