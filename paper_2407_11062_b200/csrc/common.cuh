@@ -74,4 +74,26 @@ struct SmemOptIn {
   }
 };
 
+// Launch with programmatic stream serialisation: the CTAs of this grid may start, and set themselves up, while the last
+// ones of the grid before still run.  The kernel waits for the grids before it (ptx::grid_dependency_wait) before its
+// first access to global memory; behind a kernel that never signals its dependents the launch is an ordinary one.
+template <typename... P, typename... A>
+int launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return EQAT_ERR_CUDA;
+  }
+  return launch_status();
+}
+
 }  // namespace eqat

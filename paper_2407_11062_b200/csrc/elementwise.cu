@@ -4,6 +4,7 @@
 #include "common.cuh"
 #include "codec.cuh"
 #include "elementwise.cuh"
+#include "ptx.cuh"
 
 namespace eqat {
 
@@ -51,6 +52,8 @@ ste_bwd_long_group_kernel(const eqat_bf16* __restrict__ dWhat, const eqat_bf16* 
                           const float* __restrict__ s, const float* __restrict__ z,
                           eqat_bf16* __restrict__ dW, float* __restrict__ ds, float* __restrict__ dz,
                           int vec_per_group, float Q, int dz_literal) {
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
   __shared__ float red_s[kThreads / 32], red_z[kThreads / 32];
   const size_t g = blockIdx.x;
   const float sv = __ldg(s + g);
@@ -105,6 +108,8 @@ __device__ __forceinline__ void minmax_finish(float mx, float mn, float Q, float
 __global__ void __launch_bounds__(kThreads)
 minmax_long_group_kernel(const eqat_bf16* __restrict__ W, float* __restrict__ s, float* __restrict__ z,
                          int vec_per_group, float Q) {
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
   __shared__ float red_mx[kThreads / 32], red_mn[kThreads / 32];
   const size_t g = blockIdx.x;
   float mx = -INFINITY, mn = INFINITY;
@@ -157,6 +162,8 @@ __device__ __forceinline__ void load_words(const uint8_t* packed, size_t chunk, 
 template <int BITS>
 __global__ void __launch_bounds__(kThreads)
 pack_kernel(const uint8_t* __restrict__ codes8, uint8_t* __restrict__ packed, size_t n_chunk) {
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
   const size_t c = (size_t)blockIdx.x * kThreads + threadIdx.x;
   if (c >= n_chunk) return;
   constexpr uint32_t mask = (1u << BITS) - 1u;
@@ -178,6 +185,8 @@ pack_kernel(const uint8_t* __restrict__ codes8, uint8_t* __restrict__ packed, si
 template <int BITS, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
 unpack_kernel(const uint8_t* __restrict__ packed, uint8_t* __restrict__ codes8, size_t n_chunk) {
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
   const size_t c = (size_t)blockIdx.x * kThreads + threadIdx.x;
   if (c >= n_chunk) return;
   uint32_t words[BITS];
@@ -229,28 +238,26 @@ int launch_ste_bwd(const eqat_desc& d, const eqat_bf16* dWhat, const eqat_bf16* 
   if (d.group <= 256) return launch_ste_bwd_stream(d, dWhat, W, s, z, dW, ds, dz, st);
   const float Q = (float)((1 << d.bits) - 1);
   const size_t n_groups = (size_t)d.out_features * d.in_features / d.group;
-  ste_bwd_long_group_kernel<<<(unsigned)n_groups, kThreads, 0, st>>>(dWhat, W, s, z, dW, ds, dz, d.group / 8, Q,
-                                                                     d.dz_mode == 1);
-  return launch_status();
+  return launch_overlapped(ste_bwd_long_group_kernel, dim3((unsigned)n_groups), dim3(kThreads), 0, st, dWhat, W, s, z, dW,
+                           ds, dz, d.group / 8, Q, (int)(d.dz_mode == 1));
 }
 
 int launch_minmax(const eqat_desc& d, const eqat_bf16* W, float* s, float* z, cudaStream_t st) {
   if (d.group <= 256) return launch_minmax_stream(d, W, s, z, st);
   const float Q = (float)((1 << d.bits) - 1);
   const size_t n_groups = (size_t)d.out_features * d.in_features / d.group;
-  minmax_long_group_kernel<<<(unsigned)n_groups, kThreads, 0, st>>>(W, s, z, d.group / 8, Q);
-  return launch_status();
+  return launch_overlapped(minmax_long_group_kernel, dim3((unsigned)n_groups), dim3(kThreads), 0, st, W, s, z,
+                           d.group / 8, Q);
 }
 
 int launch_pack(const eqat_desc& d, const uint8_t* codes, uint8_t* packed, cudaStream_t st) {
   const size_t n_chunk = (size_t)d.out_features * d.in_features / 32;
   const unsigned nb = blocks_for(n_chunk, kThreads);
   switch (d.bits) {
-    case 2: pack_kernel<2><<<nb, kThreads, 0, st>>>(codes, packed, n_chunk); break;
-    case 3: pack_kernel<3><<<nb, kThreads, 0, st>>>(codes, packed, n_chunk); break;
-    default: pack_kernel<4><<<nb, kThreads, 0, st>>>(codes, packed, n_chunk); break;
+    case 2: return launch_overlapped(pack_kernel<2>, dim3(nb), dim3(kThreads), 0, st, codes, packed, n_chunk);
+    case 3: return launch_overlapped(pack_kernel<3>, dim3(nb), dim3(kThreads), 0, st, codes, packed, n_chunk);
+    default: return launch_overlapped(pack_kernel<4>, dim3(nb), dim3(kThreads), 0, st, codes, packed, n_chunk);
   }
-  return launch_status();
 }
 
 int launch_unpack(const eqat_desc& d, const uint8_t* packed, uint8_t* codes, cudaStream_t st) {
@@ -258,14 +265,13 @@ int launch_unpack(const eqat_desc& d, const uint8_t* packed, uint8_t* codes, cud
   const unsigned nb = blocks_for(n_chunk, kThreads);
   const bool wide = (reinterpret_cast<uintptr_t>(codes) & 31u) == 0;
   switch (d.bits * 2 + (wide ? 1 : 0)) {
-    case 4: unpack_kernel<2, false><<<nb, kThreads, 0, st>>>(packed, codes, n_chunk); break;
-    case 5: unpack_kernel<2, true><<<nb, kThreads, 0, st>>>(packed, codes, n_chunk); break;
-    case 6: unpack_kernel<3, false><<<nb, kThreads, 0, st>>>(packed, codes, n_chunk); break;
-    case 7: unpack_kernel<3, true><<<nb, kThreads, 0, st>>>(packed, codes, n_chunk); break;
-    case 8: unpack_kernel<4, false><<<nb, kThreads, 0, st>>>(packed, codes, n_chunk); break;
-    default: unpack_kernel<4, true><<<nb, kThreads, 0, st>>>(packed, codes, n_chunk); break;
+    case 4: return launch_overlapped(unpack_kernel<2, false>, dim3(nb), dim3(kThreads), 0, st, packed, codes, n_chunk);
+    case 5: return launch_overlapped(unpack_kernel<2, true>, dim3(nb), dim3(kThreads), 0, st, packed, codes, n_chunk);
+    case 6: return launch_overlapped(unpack_kernel<3, false>, dim3(nb), dim3(kThreads), 0, st, packed, codes, n_chunk);
+    case 7: return launch_overlapped(unpack_kernel<3, true>, dim3(nb), dim3(kThreads), 0, st, packed, codes, n_chunk);
+    case 8: return launch_overlapped(unpack_kernel<4, false>, dim3(nb), dim3(kThreads), 0, st, packed, codes, n_chunk);
+    default: return launch_overlapped(unpack_kernel<4, true>, dim3(nb), dim3(kThreads), 0, st, packed, codes, n_chunk);
   }
-  return launch_status();
 }
 
 int launch_pack_zeros(const eqat_desc& d, const uint8_t* z8, uint8_t* packed, cudaStream_t st) {

@@ -235,6 +235,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   // A barrier that both CTAs of a pair signal lives in the first CTA: `lead(bar)` is its address there.
   auto lead = [&](uint32_t bar) -> uint32_t { return PAIR ? ptx::map_to_cta(bar, 0) : bar; };
 
+  ptx::grid_dependents_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
       ptx::mbar_init(ptx::smem_addr(&ctl->full[s]), C::kCtas);
@@ -274,6 +275,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   }
   ptx::tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
+  ptx::grid_dependency_wait();                                     // nothing above touches global memory
 
   // ---------------------------------------------------------------- epilogue of one tile
   // Run by four warps, one per TMEM lane quadrant (warp index mod 4).  `m0` is the first output row of this CTA's
@@ -860,6 +862,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
 __global__ void finish_row_sums_kernel(const float* __restrict__ partial, int num_n, int out_features,
                                        const eqat_fp16* __restrict__ s16, float* __restrict__ ds, float* __restrict__ dz) {
   const int o = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  ptx::grid_dependents_launch();
+  ptx::grid_dependency_wait();
   if (o >= out_features) return;
   float a = 0.0f, b = 0.0f;
   for (int n = 0; n < num_n; ++n) {
@@ -991,13 +995,15 @@ int launch(const Operand& a, const Operand& b, const GemmParams& p, cudaStream_t
   cfg.blockDim = dim3(C::kThreads, 1, 1);
   cfg.dynamicSmemBytes = C::kSmemBytes;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C::kCtas;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see launch_overlapped
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = C::kCtas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = PAIR ? 1 : 0;
+  cfg.numAttrs = PAIR ? 2 : 1;
   if (cudaLaunchKernelEx(&cfg, kern, ta, tb, p) != cudaSuccess) {
     (void)cudaGetLastError();
     return EQAT_ERR_CUDA;
@@ -1172,8 +1178,8 @@ int launch_packed_ds(const eqat_desc& d, const eqat_bf16* X, const eqat_bf16* dY
   }
   if (rc != EQAT_OK || !whole_row) return rc;
   const int num_n = (d.in_features + BN - 1) / BN;
-  finish_row_sums_kernel<<<(d.out_features + 255) / 256, 256, 0, st>>>(p.partial, num_n, d.out_features, s16, ds, dz);
-  return launch_status();
+  return launch_overlapped(finish_row_sums_kernel, dim3((d.out_features + 255) / 256), dim3(256), 0, st, p.partial, num_n,
+                           d.out_features, s16, ds, dz);
 }
 
 int launch_wait_expiry_gemm(cudaStream_t st) {

@@ -108,6 +108,7 @@ __device__ __forceinline__ void stream_tiles(const CUtensorMap* const (&maps)[NI
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t n_tiles = (n_elem + kTileElems - 1) / kTileElems;
 
+  ptx::grid_dependents_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < R::kStages; ++s) {
       ptx::mbar_init(ptx::smem_addr(&ctl->full[s]), 1);
@@ -115,14 +116,15 @@ __device__ __forceinline__ void stream_tiles(const CUtensorMap* const (&maps)[NI
     }
     ctl->abort = 0;
     ptx::fence_mbar_init();
+#pragma unroll
+    for (int i = 0; i < NIN; ++i) ptx::tma_prefetch_desc(maps[i]);
   }
   __syncthreads();
+  ptx::grid_dependency_wait();
 
   if (warp == kConsumers / 32) {
     // ---------------------------------------------------------------- producer
     if (lane == 0) {
-#pragma unroll
-      for (int i = 0; i < NIN; ++i) ptx::tma_prefetch_desc(maps[i]);
       int stage = 0;
       uint32_t phase = 0;
       size_t issued = 0;
@@ -499,8 +501,7 @@ int launch_stream(int smem_bytes, size_t n_elem, cudaStream_t st, Args... args) 
   const size_t tiles = (n_elem + kTileElems - 1) / kTileElems;
   const size_t resident = (size_t)sms * per_sm;
   const unsigned grid = (unsigned)(tiles < resident ? tiles : resident);
-  kernel<<<grid, kThreadsS, smem_bytes, st>>>(args...);
-  return launch_status();
+  return launch_overlapped(kernel, dim3(grid), dim3(kThreadsS), (size_t)smem_bytes, st, args...);
 }
 
 inline int group_shift_of(int group) {
