@@ -226,7 +226,7 @@ int eqat_unpack_zeros(const eqat_desc* desc, const uint8_t* z_packed, uint8_t* z
  * desc->zero_point_format is EQAT_ZP_FP16. */
 
 /* Y = X * ((W_int - z) * s)^T, the packed codes expanded tile by tile in
- * shared memory inside the GEMM (Eq. 2; Sec. 3.3).  With few tokens (decoding),
+ * shared or tensor memory inside the GEMM (Eq. 2; Sec. 3.3).  With few tokens (decoding),
  * up to 64, the codes enter the products as exact integers and the step sizes
  * multiply fp32 sums, so (W_int - z) * s is not rounded to bf16: a matrix-vector
  * kernel of up to eight tokens per launch for the smallest batches (groups of at
