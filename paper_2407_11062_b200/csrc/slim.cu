@@ -29,6 +29,8 @@
 // SM where the eight MMAs of a run take 340 (an MMA of 16 columns costs its A operand's 4 KB).
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "expand.cuh"
 #include "gemm.cuh"
@@ -77,6 +79,7 @@ struct SlimCtl {
   uint64_t a_full[3], d_ready[3];      // per group
   uint32_t tmem_base;
   int abort;
+  int past127;                         // some zero point byte of the slice is past 127
 };
 
 // Shared memory and tensor memory of a CTA for token tiles of 16*NT columns and ND accumulators per run.
@@ -155,7 +158,8 @@ struct Magics {
 };
 
 // Negated offsets of a group: -(bias + z) for the biases 128 and 8 that the expansion leaves on a code, as bf16 pairs.
-// (z is an integer of at most 7 bits, so every one of them, and every difference below, is exact in bf16.)
+// z is an integer of at most 7 bits here, so every one of them, and every difference below, is exact in bf16; a zero
+// point byte past 127, which no hand-off produces, comes off in a second addition (q - z has at most eight bits then).
 struct Offsets {
   uint32_t n128, n8;
   __device__ __forceinline__ explicit Offsets(float z)
@@ -268,6 +272,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       ptx::mbar_init(ptx::smem_addr(&ctl->d_ready[g]), 1);
     }
     ctl->abort = 0;
+    ctl->past127 = 0;
     ptx::fence_mbar_init();
     ptx::tma_prefetch_desc(&map_x);
     ptx::tma_prefetch_desc(&map_w);
@@ -365,6 +370,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       const int rstep = 32 >> k, rows_live = min(kRows, p.out_features - m0);
       const int steps = ((kRows / rstep) + C::kRowWarps - 1) / C::kRowWarps;
       constexpr int kBatch = 8;                            // items in flight per lane
+      uint32_t all_z = 0u;
       for (int c = lane & ((1 << k) - 1); c < items; c += 32) {
         for (int i0 = 0; i0 < steps; i0 += kBatch) {
           uint32_t vs[kBatch], vz[kBatch];
@@ -388,6 +394,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 #pragma unroll
           for (int i = 0; i < kBatch; ++i) {
             const int rr = ((i0 + i) * C::kRowWarps + warp - 2) * rstep + (lane >> k);
+            all_z |= vz[i];
             if (rr < kRows) {
               if (pairs) {
                 const uint32_t z0 = zf ? vz[i] & 0xFFFFu : vz[i] & 0xFFu, z1 = zf ? vz[i] >> 16 : vz[i] >> 8;
@@ -400,6 +407,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
           }
         }
       }
+      if (!zf && (all_z & 0x8080u) != 0u) ctl->past127 = 1;
       __syncwarp();
       asm volatile("bar.sync 1, %0;" ::"n"(C::kRowWarps * 32) : "memory");
     }
@@ -432,6 +440,26 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     auto word_zero_point = [&](uint32_t v) {
       return zf ? __half2float(__ushort_as_half((unsigned short)(v >> 16))) : (float)(v >> 16);
     };
+    // A run into the group's buffer.  PAST127: the zero point takes an addition of its own.
+    auto expand_run = [&](const uint32_t (&w)[4 * BITS], const uint32_t (&gp)[ND], auto PAST127) {
+      uint32_t a[32];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {                      // 32 codes: always inside one group
+          const float z = zf ? 0.0f : word_zero_point(gp[(2 * h + q) * ND / 4]);
+          const Offsets f(PAST127.value ? 0.0f : z);
+          expand32<BITS>(w + (2 * h + q) * BITS, f, magics, a + 16 * q);
+          if constexpr (PAST127.value) {
+            const uint32_t nz = pack_bf16x2(-z, -z);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) a[16 * q + i] = add_bf16x2(a[16 * q + i], nz);
+          }
+        }
+        ptx::tmem_st_32x32(t_a + (uint32_t)(32 * h), a);
+      }
+    };
+    const bool past127 = ctl->past127 != 0;
     bool ok = true;
     for (int r = g; r < nruns; r += kGroups) {
       const int box = r / kBoxRuns, st = box % C::kStages;
@@ -446,16 +474,8 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl->empty[st]));
       if (r != g && !(ok = collect())) break;              // the accumulators of the run before
-      uint32_t a[32];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {                      // 32 codes: always inside one group
-          const Offsets f(zf ? 0.0f : word_zero_point(gp[(2 * h + q) * ND / 4]));
-          expand32<BITS>(w + (2 * h + q) * BITS, f, magics, a + 16 * q);
-        }
-        ptx::tmem_st_32x32(t_a + (uint32_t)(32 * h), a);
-      }
+      if (!past127) expand_run(w, gp, std::false_type{});
+      else expand_run(w, gp, std::true_type{});
 #pragma unroll
       for (int i = 0; i < ND; ++i) {
         s_run[i] = __half2float(__ushort_as_half((unsigned short)(gp[i] & 0xFFFFu)));

@@ -698,6 +698,19 @@ def test_packed_forward_on_weight_row_tiles(eqat, out, in_f, tokens, bits, group
     assert eqat.device_status() == (0, 0)
 
 
+@pytest.mark.parametrize("tokens,bits,group", [(40, 4, 128), (16, 2, 32), (64, 3, 64)])
+def test_packed_forward_takes_any_zero_point_byte(eqat, tokens, bits, group):
+    """Zero points are bytes: values past the code range, and past 127, mean what they say."""
+    out, in_f = 320, 1024
+    P, _, s16, X = few_token_problem(out, in_f, tokens, 7, bits, group)
+    z8 = torch.arange(out * (in_f // group), device="cuda").mul_(37).remainder_(256).to(torch.uint8).view(out, -1)
+    Y = torch.full((tokens, out), float("nan"), dtype=torch.bfloat16, device="cuda")
+    eqat.qlinear_packed_fwd(eqat.make_desc(bits, group, out, in_f, tokens), X, P, s16, z8, Y)
+    q = O.unpack_rows(P.cpu().numpy(), bits, in_f)
+    What_o = O.dequantize(q, s16.cpu().numpy().astype(np.float32), z8.cpu().numpy(), group)
+    assert rel_err(torch_to_f64(Y), O.linear_fwd(torch_to_f64(X), What_o)) <= 1.02 * 2.0 ** -9
+
+
 @pytest.mark.parametrize("out,in_f,tokens,bits,group,real_z", [
     (64, 512, 65, 2, 64, False),      # one row tile of a pair, half of it; the other CTA has no rows
     (320, 640, 96, 3, 32, True),      # four groups per run of 128 codes, five runs over a split of K
