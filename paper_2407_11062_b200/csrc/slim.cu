@@ -463,6 +463,10 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     bool ok = true;
     for (int r = g; r < nruns; r += kGroups) {
       const int box = r / kBoxRuns, st = box % C::kStages;
+      // A wait by parity tells a phase from the one before it only.  With two groups every group has waited for every box.
+      // With three a group skips boxes, and the box that used the stage last may be one of them: the group's run before is
+      // collected first, since its MMAs come after those of that box.
+      if (kGroups > 2 && r != g && !(ok = collect())) break;
       const bool got = slim_wait(ptx::smem_addr(&ctl->full[st]), (uint32_t)(box / C::kStages) & 1u, abort_flag, WAIT_STREAM_FULL, 0);
       if (!__all_sync(0xFFFFFFFFu, got)) { ok = false; break; }
       uint32_t w[4 * BITS], gp[ND];                        // codes of the run, parameters of its groups
@@ -473,7 +477,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       ptx::fence_proxy_async_smem();                       // the codes are in registers
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&ctl->empty[st]));
-      if (r != g && !(ok = collect())) break;              // the accumulators of the run before
+      if (kGroups <= 2 && r != g && !(ok = collect())) break;   // the accumulators of the run before
       if (!past127) expand_run(w, gp, std::false_type{});
       else expand_run(w, gp, std::true_type{});
 #pragma unroll

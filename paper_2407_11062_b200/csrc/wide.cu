@@ -130,15 +130,17 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     ptx::fence_mbar_init();
     ptx::tma_prefetch_desc(&map_x);
   }
+  __syncthreads();
+  ptx::cluster_arrive();
+  ptx::grid_dependency_wait();
+  ptx::cluster_wait();                                     // the other CTAs run, and their barriers exist, from here on
+  // an operation of the pair: not before the other CTA is known to run
   if (warp == 1) {
     ptx::tmem_alloc_pair(ptx::smem_addr(&ctl->tmem_base), 512);
     ptx::tmem_relinquish_pair();
   }
   ptx::tc_fence_before();
   __syncthreads();
-  ptx::cluster_arrive();                                   // the other CTA's barriers exist from here on
-  ptx::grid_dependency_wait();
-  ptx::cluster_wait();
   ptx::tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
 
@@ -208,6 +210,18 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     auto fetch = [&](int r) { load_group_params(p, g_row + (size_t)(((run0 + r) * kRun) >> p.group_shift), g_count, gp); };
     if (g < nruns) fetch(g);
     for (int r = g; r < nruns; r += kGroups) {
+      // First the group's run before has to have left its TMEM buffer, i.e. its stage is empty: its MMAs, and with them those
+      // of every run before it, are done.  The order matters for the wait after it too.  A wait by parity tells a phase
+      // from the one before it only: the run that used stage `st` last belongs to another group, and if its codes were
+      // still on their way the wait for this run's would pass at once.  There are at least as many stages as groups, so
+      // that run is not after the group's run before, whose MMAs are done.
+      if (r != g) {
+        const int before = r - kGroups;
+        const bool fr = wide_wait(ptx::smem_addr(&ctl->empty[before % stages]), (uint32_t)(before / stages) & 1u, abort_flag,
+                                  WAIT_DEQ_OPERAND_EMPTY, 0);
+        if (!__all_sync(0xFFFFFFFFu, fr)) break;
+        ptx::tc_fence_after();
+      }
       const int st = r % stages;
       const bool got = wide_wait(ptx::smem_addr(&ctl->full_c[st]), (uint32_t)(r / stages) & 1u, abort_flag, WAIT_STREAM_FULL, 0);
       if (!__all_sync(0xFFFFFFFFu, got)) break;
@@ -226,15 +240,6 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
           gv[q] = gv[q - 1];
       }
       if (r + kGroups < nruns) fetch(r + kGroups);
-      if (r != g) {
-        // The group's run before has left its TMEM buffer when its stage is empty.  (The stage cannot be a phase further:
-        // there are at least as many stages as groups, so its next run comes after this one.)
-        const int before = r - kGroups;
-        const bool fr = wide_wait(ptx::smem_addr(&ctl->empty[before % stages]), (uint32_t)(before / stages) & 1u, abort_flag,
-                                  WAIT_DEQ_OPERAND_EMPTY, 0);
-        if (!__all_sync(0xFFFFFFFFu, fr)) break;
-        ptx::tc_fence_after();
-      }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         uint32_t a[32];
@@ -284,6 +289,20 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   ptx::tc_fence_before();
   ptx::cluster_arrive();
   ptx::cluster_wait();
+  // Tensor memory goes back here, where both CTAs of a pair stand, and no CTA leaves before all have given theirs back (the
+  // wait at the end): the release is an operation of the pair, and an SM whose CTA is gone may already hold a CTA of the
+  // next cluster or launch, with columns of its own.
+  if (warp == 1) {
+    if (*abort_flag) {                                     // outwait the MMAs in flight (microseconds)
+      const uint64_t w0 = ptx::globaltimer_ns();
+      while (ptx::globaltimer_ns() - w0 < 2000000ull) __nanosleep(1000);
+    }
+    __syncwarp();
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc_pair(tmem, 512);
+  }
+  __syncwarp();
+  ptx::cluster_arrive_relaxed();
   if (!*abort_flag) {
     // a lane sums four columns of two neighbouring rows; a warp stores 128 bytes of each column
     const int cols = min(slice, p.T - t0 - ks * slice);
@@ -309,15 +328,8 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       }
     }
   }
-  if (warp == 1) {
-    if (*abort_flag) {                                     // outwait the MMAs in flight (microseconds)
-      const uint64_t w0 = ptx::globaltimer_ns();
-      while (ptx::globaltimer_ns() - w0 < 2000000ull) __nanosleep(1000);
-    }
-    __syncwarp();
-    ptx::tc_fence_after();
-    ptx::tmem_dealloc_pair(tmem, 512);
-  }
+  __syncwarp();
+  ptx::cluster_wait();
 }
 
 // The give-up path of wide_wait alone: one warp, a barrier nothing signals, a short limit.
