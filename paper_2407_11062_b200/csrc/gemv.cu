@@ -412,9 +412,56 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
     // ---------------------------------------------------------------- reducer
     int buf = 0;
     uint32_t ready_phase[2] = {0u, 0u};
+    // Zero point bytes past 127, which no hand-off produces: the consumers' correction weights hold seven bits of a byte,
+    // and this warp looks for the eighth and takes -128 s xs off the results itself.  Looked for by the consumers it cost 2
+    // to 3 % of one-token decoding; fetched here without the lead of a task, 7 % of 11008 x 4096 at seven tokens, where a
+    // task is one stage and this warp sets the pace.
+    constexpr int kZAhead = 2;                             // 16-byte pieces per lane: rows of up to 64 groups
+    uint4 z_next[kZAhead];
+    const uint4* const z_pieces = static_cast<const uint4*>(zq);   // a task's bytes are contiguous: groups_per_row pieces
+    auto z_fetch = [&](int task) {
+#pragma unroll
+      for (int i = 0; i < kZAhead; ++i) {
+        z_next[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (task < n_tasks && lane + 32 * i < groups_per_row)
+          z_next[i] = __ldg(z_pieces + (size_t)task * groups_per_row + lane + 32 * i);
+      }
+    };
+    auto eighth_bits = [&](int row, int n) {               // -128 s xs over the groups of a row whose zero point has it
+      float v = 0.0f;
+#pragma unroll 1
+      for (int cg = 0; cg < chunks; ++cg) {
+        const size_t grp = (size_t)row * groups_per_row + ((cg << 6) >> group_shift);
+        if ((__ldg(z8 + grp) & 0x80u) == 0u) continue;
+        // the three parts of xs: the last value of quad lane 0's correction item, the first two of lane 1's
+        const uint2* item = xb + ((size_t)cg * 4 * T + n) * kTcItems + 4;
+        const uint32_t p0 = item[0].y, p12 = item[(size_t)T * kTcItems].x;
+        const float xs = (__uint_as_float(p0 & 0xFFFF0000u) + __uint_as_float(p12 << 16)) + __uint_as_float(p12 & 0xFFFF0000u);
+        v = fmaf(-128.0f * __half2float(__ushort_as_half(__ldg(s16 + grp))), xs, v);
+      }
+      return v;
+    };
+    if constexpr (!ZF16) z_fetch(blockIdx.x);
     for (int task = blockIdx.x; task < n_tasks; task += gridDim.x) {
+      uint32_t z_seen = 0u;
+      if constexpr (!ZF16) {
+#pragma unroll
+        for (int i = 0; i < kZAhead; ++i) z_seen |= z_next[i].x | z_next[i].y | z_next[i].z | z_next[i].w;
+        z_fetch(task + gridDim.x);
+        for (int i = lane + 32 * kZAhead; i < groups_per_row; i += 32) {
+          const uint4 v = __ldg(z_pieces + (size_t)task * groups_per_row + i);
+          z_seen |= v.x | v.y | v.z | v.w;
+        }
+      }
       const bool got = tc_wait(ptx::smem_addr(&ctl->part_ready[buf]), ready_phase[buf], abort_flag, WAIT_EPI_ACC_FULL, 0);
       if (!__all_sync(0xFFFFFFFFu, got)) break;
+      if (!ZF16 && __any_sync(0xFFFFFFFFu, (z_seen & 0x80808080u) != 0u)) {      // into the first warp's sums
+#pragma unroll 1
+        for (int idx = lane; idx < kTcRows * T; idx += 32) {
+          const int r = idx & (kTcRows - 1), n = idx >> 4;
+          part[(buf * kTcWarps * kTcRows + r) * kTcMaxTokens + n] += eighth_bits(task * kTcRows + r, n);
+        }
+      }
       for (int idx = lane; idx < kTcRows * T; idx += 32) {
         const int r = idx & (kTcRows - 1), n = idx >> 4;
         float v = 0.0f;
@@ -494,7 +541,8 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
     }
 
     // Correction weights by quad lane: lane 0 holds slots 0, 1 (-1, -1) and 8, 9 (-1, -(128 + z)), lane 1 slots
-    // 2, 3 (-(128 + z) twice), lanes 2 and 3 zeros.  0xBF80 = -1, 0xC300 | z = -(128 + z) for z < 128.
+    // 2, 3 (-(128 + z) twice), lanes 2 and 3 zeros.  0xBF80 = -1, 0xC300 | z = -(128 + z) for z < 128; the reducer takes the
+    // eighth bit of a zero point byte off.
     const uint32_t mask_a = q == 1 ? 0x007F007Fu : 0u, const_a = q == 0 ? 0xBF80BF80u : (q == 1 ? 0xC300C300u : 0u);
     const uint32_t mask_b = q == 0 ? 0x007F0000u : 0u, const_b = q == 0 ? 0xC300BF80u : 0u;
     // + chunk and item offsets.  Lanes whose token column does not exist read the last token's entry instead of

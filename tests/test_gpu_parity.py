@@ -711,6 +711,34 @@ def test_packed_forward_takes_any_zero_point_byte(eqat, tokens, bits, group):
     assert rel_err(torch_to_f64(Y), O.linear_fwd(torch_to_f64(X), What_o)) <= 1.02 * 2.0 ** -9
 
 
+@pytest.mark.parametrize("tokens", [1, 2, 8, 9])
+@pytest.mark.parametrize("bits,group,in_f", [
+    (2, 64, 1024),        # four groups of a row per lane and stage, fetched with one load
+    (4, 64, 1152),        # eighteen groups per row: chunk by chunk, the last chunks of a stage absent
+    (3, 128, 1024),       # two groups
+    (4, 256, 512),        # one group
+    (2, 1024, 1024),      # one group per row
+    (2, 64, 5120),        # eighty groups per row, two stages per task
+])
+def test_few_token_forward_takes_any_zero_point_byte(eqat, bits, group, in_f, tokens):
+    """The same in the matrix-vector kernel, whose correction weights hold seven bits of a zero point: rows without, with
+    some and with only zero points past 127."""
+    out = 320
+    P, z8, s16, X = few_token_problem(out, in_f, tokens, 8, bits, group)
+    ng = in_f // group
+    z8[64:192] = torch.arange(128 * ng, device="cuda").mul_(37).remainder_(256).to(torch.uint8).view(128, ng)
+    z8[192:256] = 255
+    z8[256:, ::2] = 128
+    z8[300:, :] = 1
+    z8[301, ng - 1] = 129
+    Y = torch.full((tokens, out), float("nan"), dtype=torch.bfloat16, device="cuda")
+    eqat.qlinear_packed_fwd(eqat.make_desc(bits, group, out, in_f, tokens), X, P, s16, z8, Y)
+    q = O.unpack_rows(P.cpu().numpy(), bits, in_f)
+    What_o = O.dequantize(q, s16.cpu().numpy().astype(np.float32), z8.cpu().numpy(), group)
+    # nothing is rounded before the fp32 sums: the rounding of Y to bf16, 2^-9 of each, and 2 % for the sums
+    assert rel_err(torch_to_f64(Y), O.linear_fwd(torch_to_f64(X), What_o)) <= 1.02 * 2.0 ** -9
+
+
 @pytest.mark.parametrize("out,in_f,tokens,bits,group,real_z", [
     (64, 512, 65, 2, 64, False),      # one row tile of a pair, half of it; the other CTA has no rows
     (320, 640, 96, 3, 32, True),      # four groups per run of 128 codes, five runs over a split of K
