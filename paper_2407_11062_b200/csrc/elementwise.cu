@@ -15,7 +15,7 @@ constexpr int kThreads = 256;
 struct Vec8 { float v[8]; };
 
 __device__ __forceinline__ Vec8 load_bf16x8(const eqat_bf16* p, size_t vec) {
-  const uint4 raw = __ldg(reinterpret_cast<const uint4*>(p) + vec);
+  const uint4 raw = ptx::ld_global(reinterpret_cast<const uint4*>(p) + vec);
   Vec8 o;
   const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
@@ -48,16 +48,16 @@ __device__ __forceinline__ void quant_terms(float w, float s, float zr, float& t
 // (groups of at most 256 elements are handled by the staged kernel in stream.cu)
 // One block per group, for groups longer than 256 elements (e.g. channel-wise).
 __global__ void __launch_bounds__(kThreads)
-ste_bwd_long_group_kernel(const eqat_bf16* __restrict__ dWhat, const eqat_bf16* __restrict__ W,
-                          const float* __restrict__ s, const float* __restrict__ z,
+ste_bwd_long_group_kernel(const eqat_bf16* dWhat, const eqat_bf16* W,
+                          const float* s, const float* z,
                           eqat_bf16* __restrict__ dW, float* __restrict__ ds, float* __restrict__ dz,
                           int vec_per_group, float Q, int dz_literal) {
   ptx::grid_dependents_launch();
   ptx::grid_dependency_wait();
   __shared__ float red_s[kThreads / 32], red_z[kThreads / 32];
   const size_t g = blockIdx.x;
-  const float sv = __ldg(s + g);
-  const float zr = rintf(__ldg(z + g));
+  const float sv = ptx::ld_global(s + g);
+  const float zr = rintf(ptx::ld_global(z + g));
   const float dz_clamped = dz_literal ? -1.0f : -sv;
   float acc_s = 0.0f, acc_z = 0.0f;
   for (int k = threadIdx.x; k < vec_per_group; k += kThreads) {
@@ -106,7 +106,7 @@ __device__ __forceinline__ void minmax_finish(float mx, float mn, float Q, float
 
 // (groups of at most 256 elements are handled by the staged kernel in stream.cu)
 __global__ void __launch_bounds__(kThreads)
-minmax_long_group_kernel(const eqat_bf16* __restrict__ W, float* __restrict__ s, float* __restrict__ z,
+minmax_long_group_kernel(const eqat_bf16* W, float* __restrict__ s, float* __restrict__ z,
                          int vec_per_group, float Q) {
   ptx::grid_dependents_launch();
   ptx::grid_dependency_wait();
@@ -150,18 +150,18 @@ template <int BITS>
 __device__ __forceinline__ void load_words(const uint8_t* packed, size_t chunk, uint32_t (&w)[BITS]) {
   const uint32_t* src = reinterpret_cast<const uint32_t*>(packed) + chunk * BITS;
   if constexpr (BITS == 2) {
-    const uint2 t = __ldg(reinterpret_cast<const uint2*>(src)); w[0] = t.x; w[1] = t.y;
+    const uint2 t = ptx::ld_global(reinterpret_cast<const uint2*>(src)); w[0] = t.x; w[1] = t.y;
   } else if constexpr (BITS == 4) {
-    const uint4 t = __ldg(reinterpret_cast<const uint4*>(src)); w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
+    const uint4 t = ptx::ld_global(reinterpret_cast<const uint4*>(src)); w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
   } else {
 #pragma unroll
-    for (int i = 0; i < BITS; ++i) w[i] = __ldg(src + i);
+    for (int i = 0; i < BITS; ++i) w[i] = ptx::ld_global(src + i);
   }
 }
 
 template <int BITS>
 __global__ void __launch_bounds__(kThreads)
-pack_kernel(const uint8_t* __restrict__ codes8, uint8_t* __restrict__ packed, size_t n_chunk) {
+pack_kernel(const uint8_t* codes8, uint8_t* __restrict__ packed, size_t n_chunk) {
   ptx::grid_dependents_launch();
   ptx::grid_dependency_wait();
   const size_t c = (size_t)blockIdx.x * kThreads + threadIdx.x;
@@ -170,7 +170,7 @@ pack_kernel(const uint8_t* __restrict__ codes8, uint8_t* __restrict__ packed, si
   uint32_t codes[32];
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const uint4 raw = __ldg(reinterpret_cast<const uint4*>(codes8) + c * 2 + k);
+    const uint4 raw = ptx::ld_global(reinterpret_cast<const uint4*>(codes8) + c * 2 + k);
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
     for (int i = 0; i < 16; ++i) codes[16 * k + i] = (w[i >> 2] >> (8 * (i & 3))) & mask;
@@ -184,7 +184,7 @@ pack_kernel(const uint8_t* __restrict__ codes8, uint8_t* __restrict__ packed, si
 // 1 KB contiguous per warp); otherwise as two 16-byte stores.
 template <int BITS, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
-unpack_kernel(const uint8_t* __restrict__ packed, uint8_t* __restrict__ codes8, size_t n_chunk) {
+unpack_kernel(const uint8_t* packed, uint8_t* __restrict__ codes8, size_t n_chunk) {
   ptx::grid_dependents_launch();
   ptx::grid_dependency_wait();
   const size_t c = (size_t)blockIdx.x * kThreads + threadIdx.x;
@@ -210,7 +210,7 @@ unpack_kernel(const uint8_t* __restrict__ packed, uint8_t* __restrict__ codes8, 
 }
 
 // Flat stream of small arrays (zero points): one thread per 8 codes <-> `bits` bytes.
-__global__ void pack8_kernel(const uint8_t* __restrict__ codes8, uint8_t* __restrict__ packed, size_t n8, int bits) {
+__global__ void pack8_kernel(const uint8_t* codes8, uint8_t* __restrict__ packed, size_t n8, int bits) {
   const size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x;
   if (i >= n8) return;
   const uint32_t mask = (1u << bits) - 1u;
@@ -219,7 +219,7 @@ __global__ void pack8_kernel(const uint8_t* __restrict__ codes8, uint8_t* __rest
   for (int b = 0; b < bits; ++b) packed[i * bits + b] = (uint8_t)(acc >> (8 * b));
 }
 
-__global__ void unpack8_kernel(const uint8_t* __restrict__ packed, uint8_t* __restrict__ codes8, size_t n8, int bits) {
+__global__ void unpack8_kernel(const uint8_t* packed, uint8_t* __restrict__ codes8, size_t n8, int bits) {
   const size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x;
   if (i >= n8) return;
   const uint32_t mask = (1u << bits) - 1u;

@@ -153,18 +153,18 @@ __device__ __forceinline__ void dequant_half32(const uint32_t (&w)[BITS], const 
 template <int BITS>
 __device__ __forceinline__ void load_codes64(const uint8_t* p, uint32_t (&w)[2 * BITS]) {
   if constexpr (BITS == 2) {
-    const uint4 t = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint4 t = ptx::ld_global(reinterpret_cast<const uint4*>(p));
     w[0] = t.x; w[1] = t.y; w[2] = t.z; w[3] = t.w;
   } else if constexpr (BITS == 3) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const uint2 t = __ldg(reinterpret_cast<const uint2*>(p) + i);
+      const uint2 t = ptx::ld_global(reinterpret_cast<const uint2*>(p) + i);
       w[2 * i] = t.x; w[2 * i + 1] = t.y;
     }
   } else {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const uint4 t = __ldg(reinterpret_cast<const uint4*>(p) + i);
+      const uint4 t = ptx::ld_global(reinterpret_cast<const uint4*>(p) + i);
       w[4 * i] = t.x; w[4 * i + 1] = t.y; w[4 * i + 2] = t.z; w[4 * i + 3] = t.w;
     }
   }
@@ -180,29 +180,29 @@ struct GroupParamsRaw {
 __device__ __forceinline__ void load_group_params(const PackedWeight& p, size_t gi, int count, GroupParamsRaw& r) {
   const eqat_fp16* sp = p.s16 + gi;
   if (count == 1) {
-    r.s.x = __ldg(sp);
+    r.s.x = ptx::ld_global(sp);
   } else if (count == 2) {
-    r.s.x = __ldg(reinterpret_cast<const uint32_t*>(sp));
+    r.s.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(sp));
   } else {
-    r.s = __ldg(reinterpret_cast<const uint2*>(sp));
+    r.s = ptx::ld_global(reinterpret_cast<const uint2*>(sp));
   }
   if (p.z_fp16) {
     const eqat_fp16* zp = static_cast<const eqat_fp16*>(p.zq) + gi;
     if (count == 1) {
-      r.z.x = __ldg(zp);
+      r.z.x = ptx::ld_global(zp);
     } else if (count == 2) {
-      r.z.x = __ldg(reinterpret_cast<const uint32_t*>(zp));
+      r.z.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(zp));
     } else {
-      r.z = __ldg(reinterpret_cast<const uint2*>(zp));
+      r.z = ptx::ld_global(reinterpret_cast<const uint2*>(zp));
     }
   } else {
     const uint8_t* zp = static_cast<const uint8_t*>(p.zq) + gi;
     if (count == 1) {
-      r.z.x = __ldg(zp);
+      r.z.x = ptx::ld_global(zp);
     } else if (count == 2) {
-      r.z.x = __ldg(reinterpret_cast<const unsigned short*>(zp));
+      r.z.x = ptx::ld_global(reinterpret_cast<const unsigned short*>(zp));
     } else {
-      r.z.x = __ldg(reinterpret_cast<const uint32_t*>(zp));
+      r.z.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(zp));
     }
   }
 }
@@ -216,8 +216,8 @@ __device__ __forceinline__ float zero_point_at(const GroupParamsRaw& r, int i, i
 }
 // Zero point of one group, whichever way it is stored.
 __device__ __forceinline__ float load_zero_point(const PackedWeight& p, size_t gi) {
-  return p.z_fp16 ? __half2float(__ushort_as_half(__ldg(static_cast<const eqat_fp16*>(p.zq) + gi)))
-                  : (float)__ldg(static_cast<const uint8_t*>(p.zq) + gi);
+  return p.z_fp16 ? __half2float(__ushort_as_half(ptx::ld_global(static_cast<const eqat_fp16*>(p.zq) + gi)))
+                  : (float)ptx::ld_global(static_cast<const uint8_t*>(p.zq) + gi);
 }
 
 }  // namespace eqat

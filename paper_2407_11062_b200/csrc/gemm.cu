@@ -335,10 +335,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
           float sv = 1.0f, zr = 0.0f;
           if (live) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) wraw[v] = __ldg(reinterpret_cast<const uint4*>(wrow + col0) + v);
+            for (int v = 0; v < 4; ++v) wraw[v] = ptx::ld_global(reinterpret_cast<const uint4*>(wrow + col0) + v);
             const size_t gi = (size_t)m * groups_per_row + (col0 >> p.group_shift);
-            sv = __ldg(p.s32 + gi);
-            zr = rintf(__ldg(p.z32 + gi));
+            sv = ptx::ld_global(p.s32 + gi);
+            zr = rintf(ptx::ld_global(p.z32 + gi));
           }
           uint32_t r32[32];
           ptx::tmem_ld_32x32(t_row + c * 32, r32);
@@ -391,7 +391,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
               uint32_t words[BITS];
               const uint32_t* src = reinterpret_cast<const uint32_t*>(qrow) + (size_t)(col0 >> 5) * BITS;
 #pragma unroll
-              for (int i = 0; i < BITS; ++i) words[i] = __ldg(src + i);
+              for (int i = 0; i < BITS; ++i) words[i] = ptx::ld_global(src + i);
               uint32_t codes[32];
               unpack32<BITS>(words, codes);
               const size_t gi = (size_t)m * p.groups_per_row + (col0 >> p.group_shift);
@@ -410,7 +410,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
               } else if (col0 < p.N) {
                 const size_t gi = (size_t)m * p.groups_per_row + (col0 >> p.group_shift);
                 p.ds[gi] = acc_s;
-                if (p.dz != nullptr) p.dz[gi] = -__half2float(__ushort_as_half(__ldg(p.s16 + gi))) * acc_g;
+                if (p.dz != nullptr) p.dz[gi] = -__half2float(__ushort_as_half(ptx::ld_global(p.s16 + gi))) * acc_g;
               }
               acc_s = 0.0f;
               acc_g = 0.0f;
@@ -721,11 +721,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
           if constexpr (LATENT) {
             if (valid) {
               const size_t gi = B_MN ? g_row0 + (size_t)kb * BK * p.groups_per_row : g_row0 + (size_t)((kb << 6) >> p.group_shift);
-              ring_ls[j][0] = __ldg(p.s32 + gi);
-              ring_lz[j][0] = __ldg(p.z32 + gi);
+              ring_ls[j][0] = ptx::ld_global(p.s32 + gi);
+              ring_lz[j][0] = ptx::ld_global(p.z32 + gi);
               if (split_units) {
-                ring_ls[j][1] = __ldg(p.s32 + gi + 1);
-                ring_lz[j][1] = __ldg(p.z32 + gi + 1);
+                ring_ls[j][1] = ptx::ld_global(p.s32 + gi + 1);
+                ring_lz[j][1] = ptx::ld_global(p.z32 + gi + 1);
               }
             }
           } else if (valid) {
@@ -733,7 +733,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
               // the run's 32 bytes are one sector of the packed row when the matrix itself starts on a 32-byte
               // boundary (row pitch and unit offsets are multiples of 32); otherwise two 16-byte loads
               if (p.wq_sectors) {
-                ptx::ldg_256(code_ptr, reinterpret_cast<uint32_t(&)[8]>(ring_w[j][0][0]));
+                ptx::ld_global_256(code_ptr, reinterpret_cast<uint32_t(&)[8]>(ring_w[j][0][0]));
               } else {
                 load_codes64<BITS>(code_ptr, ring_w[j][0]);
                 load_codes64<BITS>(code_ptr + 8 * BITS, ring_w[j][1]);
@@ -859,19 +859,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
 
 // E2E-QP with one group per row: adds up the column tiles' partial sums in a fixed order.
 //   ds[o] = sum_n part[0][n][o],   dz[o] = -s[o] * sum_n part[1][n][o]
-__global__ void finish_row_sums_kernel(const float* __restrict__ partial, int num_n, int out_features,
-                                       const eqat_fp16* __restrict__ s16, float* __restrict__ ds, float* __restrict__ dz) {
+__global__ void finish_row_sums_kernel(const float* partial, int num_n, int out_features,
+                                       const eqat_fp16* s16, float* __restrict__ ds, float* __restrict__ dz) {
   const int o = (int)(blockIdx.x * blockDim.x + threadIdx.x);
   ptx::grid_dependents_launch();
   ptx::grid_dependency_wait();
   if (o >= out_features) return;
   float a = 0.0f, b = 0.0f;
   for (int n = 0; n < num_n; ++n) {
-    a += partial[(size_t)n * out_features + o];
-    b += partial[(size_t)(num_n + n) * out_features + o];
+    a += ptx::ld_global(partial + (size_t)n * out_features + o);
+    b += ptx::ld_global(partial + (size_t)(num_n + n) * out_features + o);
   }
   ds[o] = a;
-  if (dz != nullptr) dz[o] = -__half2float(__ushort_as_half(__ldg(s16 + o))) * b;
+  if (dz != nullptr) dz[o] = -__half2float(__ushort_as_half(ptx::ld_global(s16 + o))) * b;
 }
 
 // One warp waits, with a short limit, on an mbarrier that nothing ever arrives at: the give-up path of

@@ -224,8 +224,8 @@ __host__ __device__ constexpr float tc_bias(int j) {
 
 template <int BITS, int PARAM_MODE, bool ZF16>
 __global__ void __launch_bounds__(kTcThreads, 1)
-packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16* __restrict__ X,
-                      const eqat_fp16* __restrict__ s16, const void* __restrict__ zq, eqat_bf16* __restrict__ Y,
+packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16* X,
+                      const eqat_fp16* s16, const void* zq, eqat_bf16* __restrict__ Y,
                       int out_features, int in_features, int group_shift, int groups_per_row, int T, int stages) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = ptx::smem_addr(smem_raw);
@@ -279,7 +279,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
   uint4 x_first[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
   if (warp < kTcWarps && (int)threadIdx.x < units) {
     const uint4* src = unit_src(threadIdx.x);
-    if (src != nullptr) { x_first[0] = __ldg(src); x_first[1] = __ldg(src + 1); }
+    if (src != nullptr) { x_first[0] = ptx::ld_global(src); x_first[1] = ptx::ld_global(src + 1); }
   }
 
   const int g = lane >> 2, q = lane & 3;
@@ -302,42 +302,42 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
     if (task < n_tasks && cg0 < chunks) {
       const size_t p_lo = (size_t)(task * kTcRows + g) * groups_per_row, p_hi = p_lo + (size_t)8 * groups_per_row;
       if constexpr (PARAM_MODE == 1) {                    // the row has a multiple of four groups: all four exist
-        sp.s_lo = __ldg(reinterpret_cast<const uint2*>(s16 + p_lo + cg0));
-        sp.s_hi = __ldg(reinterpret_cast<const uint2*>(s16 + p_hi + cg0));
+        sp.s_lo = ptx::ld_global(reinterpret_cast<const uint2*>(s16 + p_lo + cg0));
+        sp.s_hi = ptx::ld_global(reinterpret_cast<const uint2*>(s16 + p_hi + cg0));
         if constexpr (ZF16) {
-          sp.z_lo = __ldg(reinterpret_cast<const uint2*>(z16 + p_lo + cg0));
-          sp.z_hi = __ldg(reinterpret_cast<const uint2*>(z16 + p_hi + cg0));
+          sp.z_lo = ptx::ld_global(reinterpret_cast<const uint2*>(z16 + p_lo + cg0));
+          sp.z_hi = ptx::ld_global(reinterpret_cast<const uint2*>(z16 + p_hi + cg0));
         } else {
-          sp.z_lo.x = __ldg(reinterpret_cast<const uint32_t*>(z8 + p_lo + cg0));
-          sp.z_hi.x = __ldg(reinterpret_cast<const uint32_t*>(z8 + p_hi + cg0));
+          sp.z_lo.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(z8 + p_lo + cg0));
+          sp.z_hi.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(z8 + p_hi + cg0));
         }
       } else if constexpr (PARAM_MODE == 2) {             // an even number of groups per row: both exist
         const int g0 = cg0 >> 1;
-        sp.s_lo.x = __ldg(reinterpret_cast<const uint32_t*>(s16 + p_lo + g0));
-        sp.s_hi.x = __ldg(reinterpret_cast<const uint32_t*>(s16 + p_hi + g0));
+        sp.s_lo.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(s16 + p_lo + g0));
+        sp.s_hi.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(s16 + p_hi + g0));
         if constexpr (ZF16) {
-          sp.z_lo.x = __ldg(reinterpret_cast<const uint32_t*>(z16 + p_lo + g0));
-          sp.z_hi.x = __ldg(reinterpret_cast<const uint32_t*>(z16 + p_hi + g0));
+          sp.z_lo.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(z16 + p_lo + g0));
+          sp.z_hi.x = ptx::ld_global(reinterpret_cast<const uint32_t*>(z16 + p_hi + g0));
         } else {
-          sp.z_lo.x = __ldg(reinterpret_cast<const uint16_t*>(z8 + p_lo + g0));
-          sp.z_hi.x = __ldg(reinterpret_cast<const uint16_t*>(z8 + p_hi + g0));
+          sp.z_lo.x = ptx::ld_global(reinterpret_cast<const uint16_t*>(z8 + p_lo + g0));
+          sp.z_hi.x = ptx::ld_global(reinterpret_cast<const uint16_t*>(z8 + p_hi + g0));
         }
       } else if constexpr (PARAM_MODE == 3) {
         const int grp = (cg0 << 6) >> group_shift;
-        sp.s_lo.x = __ldg(s16 + p_lo + grp);
-        sp.s_hi.x = __ldg(s16 + p_hi + grp);
-        sp.z_lo.x = ZF16 ? (uint32_t)__ldg(z16 + p_lo + grp) : (uint32_t)__ldg(z8 + p_lo + grp);
-        sp.z_hi.x = ZF16 ? (uint32_t)__ldg(z16 + p_hi + grp) : (uint32_t)__ldg(z8 + p_hi + grp);
+        sp.s_lo.x = ptx::ld_global(s16 + p_lo + grp);
+        sp.s_hi.x = ptx::ld_global(s16 + p_hi + grp);
+        sp.z_lo.x = ZF16 ? (uint32_t)ptx::ld_global(z16 + p_lo + grp) : (uint32_t)ptx::ld_global(z8 + p_lo + grp);
+        sp.z_hi.x = ZF16 ? (uint32_t)ptx::ld_global(z16 + p_hi + grp) : (uint32_t)ptx::ld_global(z8 + p_hi + grp);
       } else {
         uint32_t sl[4] = {0u, 0u, 0u, 0u}, sh[4] = {0u, 0u, 0u, 0u}, zl[4] = {0u, 0u, 0u, 0u}, zh[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
         for (int c = 0; c < kChunksPerWarp; ++c) {
           if (cg0 + c < chunks) {
             const int grp = ((cg0 + c) << 6) >> group_shift;
-            sl[c] = __ldg(s16 + p_lo + grp);
-            sh[c] = __ldg(s16 + p_hi + grp);
-            zl[c] = ZF16 ? (uint32_t)__ldg(z16 + p_lo + grp) : (uint32_t)__ldg(z8 + p_lo + grp);
-            zh[c] = ZF16 ? (uint32_t)__ldg(z16 + p_hi + grp) : (uint32_t)__ldg(z8 + p_hi + grp);
+            sl[c] = ptx::ld_global(s16 + p_lo + grp);
+            sh[c] = ptx::ld_global(s16 + p_hi + grp);
+            zl[c] = ZF16 ? (uint32_t)ptx::ld_global(z16 + p_lo + grp) : (uint32_t)ptx::ld_global(z8 + p_lo + grp);
+            zh[c] = ZF16 ? (uint32_t)ptx::ld_global(z16 + p_hi + grp) : (uint32_t)ptx::ld_global(z8 + p_hi + grp);
           }
         }
         sp.s_lo = make_uint2(sl[0] | (sl[1] << 16), sl[2] | (sl[3] << 16));
@@ -424,7 +424,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
       for (int i = 0; i < kZAhead; ++i) {
         z_next[i] = make_uint4(0u, 0u, 0u, 0u);
         if (task < n_tasks && lane + 32 * i < groups_per_row)
-          z_next[i] = __ldg(z_pieces + (size_t)task * groups_per_row + lane + 32 * i);
+          z_next[i] = ptx::ld_global(z_pieces + (size_t)task * groups_per_row + lane + 32 * i);
       }
     };
     auto eighth_bits = [&](int row, int n) {               // -128 s xs over the groups of a row whose zero point has it
@@ -432,12 +432,12 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
 #pragma unroll 1
       for (int cg = 0; cg < chunks; ++cg) {
         const size_t grp = (size_t)row * groups_per_row + ((cg << 6) >> group_shift);
-        if ((__ldg(z8 + grp) & 0x80u) == 0u) continue;
+        if ((ptx::ld_global(z8 + grp) & 0x80u) == 0u) continue;
         // the three parts of xs: the last value of quad lane 0's correction item, the first two of lane 1's
         const uint2* item = xb + ((size_t)cg * 4 * T + n) * kTcItems + 4;
         const uint32_t p0 = item[0].y, p12 = item[(size_t)T * kTcItems].x;
         const float xs = (__uint_as_float(p0 & 0xFFFF0000u) + __uint_as_float(p12 << 16)) + __uint_as_float(p12 & 0xFFFF0000u);
-        v = fmaf(-128.0f * __half2float(__ushort_as_half(__ldg(s16 + grp))), xs, v);
+        v = fmaf(-128.0f * __half2float(__ushort_as_half(ptx::ld_global(s16 + grp))), xs, v);
       }
       return v;
     };
@@ -449,7 +449,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
         for (int i = 0; i < kZAhead; ++i) z_seen |= z_next[i].x | z_next[i].y | z_next[i].z | z_next[i].w;
         z_fetch(task + gridDim.x);
         for (int i = lane + 32 * kZAhead; i < groups_per_row; i += 32) {
-          const uint4 v = __ldg(z_pieces + (size_t)task * groups_per_row + i);
+          const uint4 v = ptx::ld_global(z_pieces + (size_t)task * groups_per_row + i);
           z_seen |= v.x | v.y | v.z | v.w;
         }
       }
@@ -491,7 +491,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
           if (u0 >= kTcWarps * 32) {                                   // later rounds load here
             const uint4* src = unit_src(u);
             v0 = v1 = make_uint4(0u, 0u, 0u, 0u);
-            if (src != nullptr) { v0 = __ldg(src); v1 = __ldg(src + 1); }
+            if (src != nullptr) { v0 = ptx::ld_global(src); v1 = ptx::ld_global(src + 1); }
           }
           const uint32_t r[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
           uint32_t h[16];                                              // column j of the word as 16 bits

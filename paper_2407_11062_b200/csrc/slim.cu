@@ -383,11 +383,11 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
               const eqat_fp16* z16 = static_cast<const eqat_fp16*>(p.zq) + gi;
               const uint8_t* z8 = static_cast<const uint8_t*>(p.zq) + gi;
               if (pairs) {
-                vs[i] = __ldg(reinterpret_cast<const uint32_t*>(p.s16 + gi));
-                vz[i] = zf ? __ldg(reinterpret_cast<const uint32_t*>(z16)) : (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(z8));
+                vs[i] = ptx::ld_global(reinterpret_cast<const uint32_t*>(p.s16 + gi));
+                vz[i] = zf ? ptx::ld_global(reinterpret_cast<const uint32_t*>(z16)) : (uint32_t)ptx::ld_global(reinterpret_cast<const unsigned short*>(z8));
               } else {
-                vs[i] = (uint32_t)__ldg(p.s16 + gi);
-                vz[i] = zf ? (uint32_t)__ldg(z16) : (uint32_t)__ldg(z8);
+                vs[i] = (uint32_t)ptx::ld_global(p.s16 + gi);
+                vz[i] = zf ? (uint32_t)ptx::ld_global(z16) : (uint32_t)ptx::ld_global(z8);
               }
             }
           }

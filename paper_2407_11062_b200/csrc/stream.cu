@@ -206,13 +206,13 @@ __device__ __forceinline__ size_t group_index(size_t e0, int group) {
 
 // `group`: log2 of the group length, or (LONG) the length in units of 32 elements.
 template <bool LONG = false>
-__device__ __forceinline__ GroupParams fetch_group(const float* __restrict__ s, const float* __restrict__ z, size_t e0,
+__device__ __forceinline__ GroupParams fetch_group(const float* s, const float* z, size_t e0,
                                                    size_t n_elem, int group) {
   GroupParams p{1.0f, 0.0f};
   if (e0 < n_elem) {
     const size_t g = group_index<LONG>(e0, group);
-    p.s = __ldg(s + g);
-    p.z = __ldg(z + g);
+    p.s = ptx::ld_global(s + g);
+    p.z = ptx::ld_global(z + g);
   }
   return p;
 }
@@ -235,8 +235,8 @@ __device__ __forceinline__ void store_lane(eqat_bf16* dst, const uint4 (&o)[4], 
 // (clamp(r + z, 0, Q) - z) * s == clamp(r, -z, Q - z) * s for integer r and z.
 template <bool LONG>
 __global__ void __launch_bounds__(kThreadsS, kCtas1)
-fakequant_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* __restrict__ s,
-                        const float* __restrict__ z, eqat_bf16* __restrict__ What, size_t n_elem, int group,
+fakequant_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* s,
+                        const float* z, eqat_bf16* __restrict__ What, size_t n_elem, int group,
                         float Q, int wide) {
   const CUtensorMap* const maps[1] = {&map_w};
   stream_tiles<1, kStages1, GroupParams>(maps, n_elem,
@@ -272,7 +272,7 @@ fakequant_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* 
 template <int LPG>
 __global__ void __launch_bounds__(kThreadsS, kCtas2)
 ste_bwd_stream_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_w,
-                      const float* __restrict__ s, const float* __restrict__ z, eqat_bf16* __restrict__ dW,
+                      const float* s, const float* z, eqat_bf16* __restrict__ dW,
                       float* __restrict__ ds, float* __restrict__ dz, size_t n_elem, float Q, int dz_literal, int wide) {
   const CUtensorMap* const maps[2] = {&map_g, &map_w};
   constexpr int group_shift = LPG == 1 ? 5 : LPG == 2 ? 6 : LPG == 4 ? 7 : 8;
@@ -391,8 +391,8 @@ minmax_stream_kernel(const __grid_constant__ CUtensorMap map_w, float* __restric
 // low bits ARE the code.
 template <int BITS, bool LONG>
 __global__ void __launch_bounds__(kThreadsS, kCtas1)
-quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* __restrict__ s,
-                            const float* __restrict__ z, uint8_t* __restrict__ packed, uint8_t* __restrict__ z8,
+quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* s,
+                            const float* z, uint8_t* __restrict__ packed, uint8_t* __restrict__ z8,
                             eqat_fp16* __restrict__ s16, size_t n_elem, int group) {
   const CUtensorMap* const maps[1] = {&map_w};
   constexpr float Q = (float)((1 << BITS) - 1);
