@@ -235,7 +235,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   // A barrier that both CTAs of a pair signal lives in the first CTA: `lead(bar)` is its address there.
   auto lead = [&](uint32_t bar) -> uint32_t { return PAIR ? ptx::map_to_cta(bar, 0) : bar; };
 
-  ptx::grid_dependents_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
       ptx::mbar_init(ptx::smem_addr(&ctl->full[s]), C::kCtas);
@@ -258,6 +257,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
     ptx::tma_prefetch_desc(&tmap_a);
     if (!PACKED || LATENT) ptx::tma_prefetch_desc(&tmap_b);
   }
+  if (PAIR) {                                                      // the other CTA runs, and its barriers exist, from here on
+    __syncthreads();
+    ptx::cluster_arrive();
+    ptx::cluster_wait();
+  }
+  // An operation of the pair: not before the other CTA is known to run.  And the launch after this one may start only once
+  // the columns are taken: a CTA of it that got them first would wait for this grid to end, and this grid for the columns.
   if (warp == 1) {
     if (PAIR) {
       ptx::tmem_alloc_pair(ptx::smem_addr(&ctl->tmem_base), C::kTmemCols);
@@ -269,11 +275,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   }
   ptx::tc_fence_before();
   __syncthreads();
-  if (PAIR) {                                                      // the other CTA's barriers exist from here on
-    ptx::cluster_arrive();
-    ptx::cluster_wait();
-  }
   ptx::tc_fence_after();
+  ptx::grid_dependents_launch();
   const uint32_t tmem_base = ctl->tmem_base;
   ptx::grid_dependency_wait();                                     // nothing above touches global memory
 
@@ -854,6 +857,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
     ptx::tc_fence_after();
     if (PAIR) ptx::tmem_dealloc_pair(tmem_base, C::kTmemCols);
     else ptx::tmem_dealloc(tmem_base, C::kTmemCols);
+  }
+  if (PAIR) {
+    // The release is an operation of the pair too: an SM whose CTA is gone may already hold a CTA of the next launch, with
+    // columns of its own.
+    __syncwarp();
+    ptx::cluster_arrive_relaxed();
+    ptx::cluster_wait();
   }
 }
 

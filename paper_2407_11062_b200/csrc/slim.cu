@@ -248,7 +248,6 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   slice_of(p.runs, p.split_log2, rank, run0, nruns);
   const int ngroups = slice_groups(run0, nruns, p.group_shift, group0);
 
-  ptx::grid_dependents_launch();
   // The codes, step sizes and zero points of this CTA's slice are asked into L2 before the wait for the launches before
   // this one: a prefetch changes nothing that can be observed, and it takes the DRAM latency out of the loop below.
   if (warp == 0 && ptx::elect_one()) {
@@ -291,6 +290,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
+  ptx::grid_dependents_launch();                           // once the columns are taken (see gemm.cu)
   ptx::cluster_arrive_relaxed();                           // waited for before the first store to another CTA
   ptx::grid_dependency_wait();
 

@@ -114,7 +114,6 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   // barriers that both CTAs of a pair signal live in its first CTA
   auto lead = [&](const void* bar) { return ptx::map_to_cta(ptx::smem_addr(bar), (uint32_t)(2 * ks)); };
 
-  ptx::grid_dependents_launch();
   if (warp == 0 && m0 < p.out_features && ptx::elect_one()) {   // into L2 before the wait for the launches before this one
     for (int r = 0; r < nruns; ++r) ptx::tma_prefetch_2d(&map_w, (run0 + r) * code_bytes(BITS), m0);
   }
@@ -143,6 +142,7 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
+  ptx::grid_dependents_launch();                           // once the columns are taken (see gemm.cu)
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer

@@ -25,6 +25,26 @@ def test_no_operand_is_read_through_the_read_only_path():
     assert not found
 
 
+def test_tensor_memory_of_overlapped_and_paired_launches():
+    """Read in the sources: a kernel takes its tensor memory before it lets the next launch start (a CTA of that launch that
+    took the columns first would wait for this grid, and this grid for the columns); a pair takes its columns when both CTAs
+    are known to run and no CTA leaves before both have given theirs back."""
+    checked = 0
+    for name, text in sources():
+        for kernel in re.split(r"__global__", text)[1:]:
+            alloc = [m.start() for m in re.finditer(r"tmem_alloc(?:_pair)?\(", kernel)]
+            if not alloc:
+                continue
+            checked += 1
+            starts = [m.start() for m in re.finditer(r"grid_dependents_launch\(", kernel)]
+            assert len(starts) == 1 and starts[0] > max(alloc), name
+            if "tmem_alloc_pair(" in kernel:
+                waits = [m.start() for m in re.finditer(r"cluster_wait\(", kernel)]
+                assert min(waits) < kernel.index("tmem_alloc_pair("), name
+                assert max(waits) > kernel.index("tmem_dealloc_pair("), name
+    assert checked == 3
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("bits,group", [(2, 64), (3, 128), (4, 512), (4, 32)])
 def test_operands_rewritten_between_overlapped_launches(bits, group):
