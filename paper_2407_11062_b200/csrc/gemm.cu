@@ -54,10 +54,9 @@
 #include "gemm.cuh"
 #include "ptx.cuh"
 #include "quant_math.cuh"
+#include "wait.cuh"
 
 namespace eqat {
-
-__device__ int g_device_status[2];   // [0] = eqat_status, [1] = WaitSite
 
 namespace {
 
@@ -67,7 +66,6 @@ constexpr int BK = 64;           // K per stage: one 128-byte swizzle span of bf
 constexpr int UMMA_K = 16;       // K per tcgen05.mma for 16-bit inputs
 constexpr int kEpiWarps = 4;       // dense kernels: warps 2-5 are the epilogue
 constexpr int kDeqWarps = 16;      // packed kernels: warps 2-17 expand codes; warps 2-5 also run the epilogue
-constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s per wait
 constexpr uint64_t kDrainLimitNs = 50000000ull;    // 50 ms per stage at teardown
 
 enum Epilogue : int { EPI_STORE = 0, EPI_DS = 1, EPI_STE = 2 };
@@ -129,33 +127,6 @@ struct Control {
   int abort;
 };
 static_assert(sizeof(Control) <= 512, "control block must fit its reservation");
-
-// Bounded wait on an mbarrier phase.  `sleep_ns` > 0 backs off between polls so
-// that a role with nothing to do for a long time (the epilogue during a main
-// loop, the producer on a full ring) leaves the issue slots to the warps that
-// are working; latency-critical waits pass 0.  CLUSTER: the barrier is also
-// signalled from the other CTA of a pair.
-template <bool CLUSTER = false>
-__device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, volatile int* abort, int site,
-                                             uint32_t sleep_ns = 0, uint64_t limit_ns = kWaitLimitNs) {
-  auto ready = [&] { return CLUSTER ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity); };
-  if (ready()) return true;
-  const uint64_t t0 = ptx::globaltimer_ns();
-  uint32_t n = 0;
-  while (!ready()) {
-    if (sleep_ns != 0) __nanosleep(sleep_ns);
-    if ((++n & 31u) == 0u) {
-      if (*abort) return false;
-      if (ptx::globaltimer_ns() - t0 > limit_ns) {
-        *abort = 1;
-        atomicExch(&g_device_status[1], site);
-        atomicExch(&g_device_status[0], (int)EQAT_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
-}
 
 // Shared-memory matrix descriptor, 128-byte swizzle, 8-row atoms 1024 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes) {
@@ -286,10 +257,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   const int quad = warp & 3;
   const int row_in_tile = quad * 32 + lane;
   auto epilogue_tile = [&](int m0, int n_blk, int acc, uint32_t acc_phase) -> bool {
-    // The lanes of a warp must leave together: the store epilogue below shuffles across the whole warp.
-    const bool got = wait_bounded<PAIR>(ptx::smem_addr(&ctl->acc_full[acc]), acc_phase, abort_flag, WAIT_EPI_ACC_FULL,
-                                        PACKED ? 0 : (MT == 2 ? 512 : 128));
-    if (!__all_sync(0xFFFFFFFFu, got)) return false;
+    if (!bounded_wait_warp<PAIR>(ptx::smem_addr(&ctl->acc_full[acc]), acc_phase, abort_flag, WAIT_EPI_ACC_FULL,
+                                 PACKED ? 0 : (MT == 2 ? 512 : 128)))
+      return false;
     ptx::tc_fence_after();
 #pragma unroll 1
     for (int h = 0; h < MT; ++h) {
@@ -507,8 +477,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
             if (*abort_flag) break;
             if (ptx::globaltimer_ns() - t_last > kWaitLimitNs) {
               *abort_flag = 1;
-              atomicExch(&g_device_status[1], (int)WAIT_PRODUCER_EMPTY);
-              atomicExch(&g_device_status[0], (int)EQAT_ERR_TIMEOUT);
+              atomicExch(&g_wait_status[1], (int)WAIT_PRODUCER_EMPTY);
+              atomicExch(&g_wait_status[0], (int)EQAT_ERR_TIMEOUT);
               break;
             }
           }
@@ -530,7 +500,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
         const int m0 = m_blk * C::kClusterM + rank * C::kTileM;    // this CTA's rows of A
         const int n0 = n_blk * BN + rank * C::kBRows;              // this CTA's rows of B
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!wait_bounded<PAIR>(ptx::smem_addr(&ctl->empty[stage]), phase ^ 1u, abort_flag, WAIT_PRODUCER_EMPTY, 64)) {
+          if (!bounded_wait<PAIR>(ptx::smem_addr(&ctl->empty[stage]), phase ^ 1u, abort_flag, WAIT_PRODUCER_EMPTY, 64)) {
             ok = false;
             break;
           }
@@ -576,7 +546,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
             const uint64_t t0 = ptx::globaltimer_ns();
             while (!ptx::mbar_try_wait(bar, par)) {
               if (ptx::globaltimer_ns() - t0 > kDrainLimitNs) {
-                atomicExch(&g_device_status[1], (int)WAIT_TEARDOWN);
+                atomicExch(&g_wait_status[1], (int)WAIT_TEARDOWN);
                 break;
               }
             }
@@ -603,18 +573,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
       uint32_t acc_phase = 0;
       bool ok = true;
       for (int tile = cluster_id; tile < num_tiles && ok; tile += num_clusters) {
-        if (!wait_bounded<PAIR>(ptx::smem_addr(&ctl->acc_empty[acc]), acc_phase ^ 1u, abort_flag, WAIT_MMA_ACC_EMPTY, 64)) break;
+        const bool room = bounded_wait<PAIR>(ptx::smem_addr(&ctl->acc_empty[acc]), acc_phase ^ 1u, abort_flag, WAIT_MMA_ACC_EMPTY, 64);
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * MT * BN);
         for (int kb = 0; kb < num_kb; ++kb) {
-          if (!wait_bounded<PAIR>(ptx::smem_addr(&ctl->full[stage]), phase, abort_flag, WAIT_MMA_FULL, PACKED ? 32 : 0) ||
-              (PACKED &&
-               !wait_bounded<PAIR>(ptx::smem_addr(&ctl->full_b[stage_b]), phase_b, abort_flag, WAIT_MMA_FULL, 32))) {
-            ok = false;
-            break;
-          }
+          bool got = room && bounded_wait<PAIR>(ptx::smem_addr(&ctl->full[stage]), phase, abort_flag, WAIT_MMA_FULL, PACKED ? 32 : 0);
+          if (PACKED && got)
+            got = bounded_wait<PAIR>(ptx::smem_addr(&ctl->full_b[stage_b]), phase_b, abort_flag, WAIT_MMA_FULL, 32);
           ptx::tc_fence_after();
-          if (ptx::elect_one()) {
+          if (ptx::elect_one() && got) {
             const uint32_t a_addr = smem_base + C::a_offset(stage);
             const uint32_t b_addr = smem_base + C::b_offset(PACKED ? stage_b : stage);
 #pragma unroll
@@ -630,7 +597,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
             commit_both(ptx::smem_addr(&ctl->empty[stage]));
             if (PACKED) commit_both(ptx::smem_addr(&ctl->empty_b[stage_b]));
           }
-          __syncwarp();
+          ok = warp_agrees(got);
+          if (!ok) break;
           if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
           if (PACKED) {
             if (++stage_b == C::kStagesB) { stage_b = 0; phase_b ^= 1u; }
@@ -648,7 +616,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
         else ptx::mma_commit(ptx::smem_addr(&ctl->drain));
       }
       __syncwarp();
-      wait_bounded(ptx::smem_addr(&ctl->drain), 0u, abort_flag, WAIT_TEARDOWN, 64, kDrainLimitNs * 4);
+      bounded_wait(ptx::smem_addr(&ctl->drain), 0u, abort_flag, WAIT_TEARDOWN, 64, kDrainLimitNs * 4);
     }
   } else if (!PACKED) {
     // ------------------------------------------------------------ epilogue warps (dense kernels)
@@ -761,15 +729,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
               const uint32_t phase = (uint32_t)(((gk + kb) / C::kStagesB) & 1);
               // packed codes: the stage must have been released by the tensor core; latent weights: the raw tile
               // must have landed in it
-              bool free_stage = LATENT ? wait_bounded(ptx::smem_addr(&ctl->raw_b[stage]), phase, abort_flag, WAIT_DEQ_OPERAND_EMPTY)
-                                       : wait_bounded<PAIR>(ptx::smem_addr(&ctl->empty_b[stage]), phase ^ 1u, abort_flag,
-                                                            WAIT_DEQ_OPERAND_EMPTY);
-              if (R == 2 && free_stage)
-                free_stage = wait_bounded<PAIR>(ptx::smem_addr(&ctl->empty_b[stage + 1]), phase ^ 1u, abort_flag,
+              bool free_stage;
+              if (LATENT)
+                free_stage = bounded_wait(ptx::smem_addr(&ctl->raw_b[stage]), phase, abort_flag, WAIT_DEQ_OPERAND_EMPTY);
+              else
+                free_stage = bounded_wait<PAIR>(ptx::smem_addr(&ctl->empty_b[stage]), phase ^ 1u, abort_flag,
                                                 WAIT_DEQ_OPERAND_EMPTY);
-              if (!free_stage) {
-                ok = false;
-              } else {
+              if (R == 2 && free_stage)
+                free_stage = bounded_wait<PAIR>(ptx::smem_addr(&ctl->empty_b[stage + 1]), phase ^ 1u, abort_flag,
+                                                WAIT_DEQ_OPERAND_EMPTY);
+              if (free_stage) {
                 // Both K blocks of a run are one straight-line piece of code (their two stages belong to this group
                 // and share a phase): twice the independent work for the scheduler to interleave, one fence and one
                 // warp synchronisation for the two stages.
@@ -824,20 +793,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
                 }
                 if (kb + 2 * kStep < num_kb) fetch(j, kb + 2 * kStep);
                 ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
+              }
+              ok = warp_agrees(free_stage);
+              if (ok && lane == 0) {
 #pragma unroll
-                  for (int u = 0; u < R; ++u) {
-                    if (PAIR) ptx::mbar_arrive_cluster(full_b_lead + (uint32_t)(stage + u) * 8u);
-                    else ptx::mbar_arrive(ptx::smem_addr(&ctl->full_b[stage + u]));
-                  }
+                for (int u = 0; u < R; ++u) {
+                  if (PAIR) ptx::mbar_arrive_cluster(full_b_lead + (uint32_t)(stage + u) * 8u);
+                  else ptx::mbar_arrive(ptx::smem_addr(&ctl->full_b[stage + u]));
                 }
               }
             }
           }
         }
         gk += num_kb;
-        ok = __all_sync(0xFFFFFFFFu, ok);                          // a warp gives up as a whole
         if (warp < 2 + kEpiWarps && ok) {
           ok = epilogue_tile(m_blk * C::kClusterM + rank * C::kTileM, n_blk, acc, acc_phase);
           if (++acc == C::kAccSets) { acc = 0; acc_phase ^= 1u; }
@@ -882,20 +850,6 @@ __global__ void finish_row_sums_kernel(const float* partial, int num_n, int out_
   }
   ds[o] = a;
   if (dz != nullptr) dz[o] = -__half2float(__ushort_as_half(ptx::ld_global(s16 + o))) * b;
-}
-
-// One warp waits, with a short limit, on an mbarrier that nothing ever arrives at: the give-up path of
-// wait_bounded (abort flag, status word, normal return) without any copy or tensor-memory state around it.
-__global__ void wait_expiry_kernel(uint64_t limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_word;
-  if (threadIdx.x == 0) {
-    ptx::mbar_init(ptx::smem_addr(&bar), 1);
-    abort_word = 0;
-    ptx::fence_mbar_init();
-  }
-  __syncthreads();
-  (void)wait_bounded(ptx::smem_addr(&bar), 0u, &abort_word, WAIT_SELFTEST, 0, limit_ns);
 }
 
 // ------------------------------------------------------------------ host side
@@ -1192,20 +1146,7 @@ int launch_packed_ds(const eqat_desc& d, const eqat_bf16* X, const eqat_bf16* dY
                            d.out_features, s16, ds, dz);
 }
 
-int launch_wait_expiry_gemm(cudaStream_t st) {
-  wait_expiry_kernel<<<1, 32, 0, st>>>(1000000ull);   // 1 ms
-  return launch_status();
-}
-
-int read_device_status(int* status, int* detail) {
-  int h[2] = {0, 0};
-  if (cudaDeviceSynchronize() != cudaSuccess) return EQAT_ERR_CUDA;
-  if (cudaMemcpyFromSymbol(h, g_device_status, sizeof(h)) != cudaSuccess) return EQAT_ERR_CUDA;
-  const int zero[2] = {0, 0};
-  if (cudaMemcpyToSymbol(g_device_status, zero, sizeof(zero)) != cudaSuccess) return EQAT_ERR_CUDA;
-  *status = h[0];
-  if (detail != nullptr) *detail = h[1];
-  return EQAT_OK;
-}
+int launch_wait_expiry_gemm(cudaStream_t st) { return launch_wait_expiry(st); }
+int read_device_status(int* status, int* detail) { return read_wait_status(status, detail); }
 
 }  // namespace eqat

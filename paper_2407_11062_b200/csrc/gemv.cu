@@ -14,6 +14,7 @@
 #include "gemm.cuh"
 #include "gemv.cuh"
 #include "ptx.cuh"
+#include "wait.cuh"
 
 namespace eqat {
 namespace {
@@ -82,7 +83,6 @@ constexpr int kTcAhead = 3;                            // stages of lead of the 
 constexpr int kTcItems = 5;                            // instructions per chunk: four on codes, one correction
 constexpr int kTcMaxStages = 8;
 __host__ __device__ constexpr int tc_min_stages(int bits) { return bits == 2 ? 3 : 2; }   // at least 48 KB in flight
-constexpr uint64_t kTcWaitLimitNs = 2000000000ull;
 constexpr size_t kTcSmemBudget = 227 * 1024;             // the most a CTA can be given (eight tokens of 8192 columns need 225.2 KB)
 
 struct TcCtl {
@@ -117,28 +117,6 @@ inline int tc_stages_that_fit(int T, int in_features, int bits) {
   for (int st = kTcMaxStages; st >= tc_min_stages(bits); --st)
     if (tc_layout(T, in_features, st, bits).total <= kTcSmemBudget) return st;
   return 0;
-}
-
-__device__ int g_gemv_status[2];   // [0] = eqat_status, [1] = WaitSite
-
-__device__ __forceinline__ bool tc_wait(uint32_t bar, uint32_t parity, volatile int* abort, int site, uint32_t sleep_ns,
-                                        uint64_t limit_ns = kTcWaitLimitNs) {
-  if (ptx::mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = ptx::globaltimer_ns();
-  uint32_t n = 0;
-  while (!ptx::mbar_try_wait(bar, parity)) {
-    if (sleep_ns != 0) __nanosleep(sleep_ns);
-    if ((++n & 31u) == 0u) {
-      if (*abort) return false;
-      if (ptx::globaltimer_ns() - t0 > limit_ns) {
-        *abort = 1;
-        atomicExch(&g_gemv_status[1], site);
-        atomicExch(&g_gemv_status[0], (int)EQAT_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
 }
 
 // (t & mask) | magic on both halves of a register.
@@ -377,7 +355,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
       bool ok = true;
       for (int task = blockIdx.x; task < n_tasks && ok; task += gridDim.x) {
         for (int k = 0; k < task_stages; ++k) {
-          if (!tc_wait(ptx::smem_addr(&ctl->empty[slot]), phase ^ 1u, abort_flag, WAIT_STREAM_EMPTY, 32)) {
+          if (!bounded_wait(ptx::smem_addr(&ctl->empty[slot]), phase ^ 1u, abort_flag, WAIT_STREAM_EMPTY, 32)) {
             ok = false;
             break;
           }
@@ -401,7 +379,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
           const uint64_t t0 = ptx::globaltimer_ns();
           while (!ptx::mbar_try_wait(bar, par)) {
             if (ptx::globaltimer_ns() - t0 > 50000000ull) {
-              atomicExch(&g_gemv_status[1], (int)WAIT_TEARDOWN);
+              atomicExch(&g_wait_status[1], (int)WAIT_TEARDOWN);
               break;
             }
           }
@@ -453,8 +431,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
           z_seen |= v.x | v.y | v.z | v.w;
         }
       }
-      const bool got = tc_wait(ptx::smem_addr(&ctl->part_ready[buf]), ready_phase[buf], abort_flag, WAIT_EPI_ACC_FULL, 0);
-      if (!__all_sync(0xFFFFFFFFu, got)) break;
+      if (!bounded_wait_warp(ptx::smem_addr(&ctl->part_ready[buf]), ready_phase[buf], abort_flag, WAIT_EPI_ACC_FULL)) break;
       if (!ZF16 && __any_sync(0xFFFFFFFFu, (z_seen & 0x80808080u) != 0u)) {      // into the first warp's sums
 #pragma unroll 1
         for (int idx = lane; idx < kTcRows * T; idx += 32) {
@@ -562,8 +539,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
         for (int i = 0; i + 1 < kTcAhead; ++i) nx[i] = nx[i + 1];
         nx[kTcAhead - 1] = fetch(pf_task, pf_k);
         advance();
-        const bool got = tc_wait(ptx::smem_addr(&ctl->full[slot]), phase, abort_flag, WAIT_STREAM_FULL, 0);
-        if (!__all_sync(0xFFFFFFFFu, got)) { alive = false; break; }
+        if (!bounded_wait_warp(ptx::smem_addr(&ctl->full[slot]), phase, abort_flag, WAIT_STREAM_FULL)) { alive = false; break; }
         // a lane's 16 codes per row and chunk
         uint32_t w_lo[kChunksPerWarp][tc_words_per_lane(BITS)], w_hi[kChunksPerWarp][tc_words_per_lane(BITS)];
         if (have) {
@@ -657,9 +633,7 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
         }
       }
       if (!alive) break;
-      const bool free_ok = tc_wait(ptx::smem_addr(&ctl->part_free[buf]), free_phase[buf] ^ 1u, abort_flag,
-                                   WAIT_MMA_ACC_EMPTY, 0);
-      if (!__all_sync(0xFFFFFFFFu, free_ok)) break;
+      if (!bounded_wait_warp(ptx::smem_addr(&ctl->part_free[buf]), free_phase[buf] ^ 1u, abort_flag, WAIT_MMA_ACC_EMPTY)) break;
       float* pw = part + (size_t)((buf * kTcWarps + warp) * kTcRows) * kTcMaxTokens;
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
@@ -675,19 +649,6 @@ packed_gemv_tc_kernel(const __grid_constant__ CUtensorMap map_w, const eqat_bf16
       buf ^= 1;
     }
   }
-}
-
-// The give-up path of tc_wait alone: one warp, a barrier nothing signals, a short limit.
-__global__ void tc_wait_expiry_kernel(uint64_t limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_word;
-  if (threadIdx.x == 0) {
-    ptx::mbar_init(ptx::smem_addr(&bar), 1);
-    abort_word = 0;
-    ptx::fence_mbar_init();
-  }
-  __syncthreads();
-  (void)tc_wait(ptx::smem_addr(&bar), 0u, &abort_word, WAIT_SELFTEST, 0, limit_ns);
 }
 
 template <int BITS, int PARAM_MODE, bool ZF16>
@@ -803,20 +764,7 @@ int launch_packed_gemv(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq
   return EQAT_ERR_UNSUPPORTED;                           // not reached for a problem packed_gemv_applies() accepted
 }
 
-int launch_wait_expiry_gemv(cudaStream_t st) {
-  tc_wait_expiry_kernel<<<1, 32, 0, st>>>(1000000ull);   // 1 ms
-  return launch_status();
-}
-
-int read_gemv_status(int* status, int* detail) {
-  int h[2] = {0, 0};
-  if (cudaDeviceSynchronize() != cudaSuccess) return EQAT_ERR_CUDA;
-  if (cudaMemcpyFromSymbol(h, g_gemv_status, sizeof(h)) != cudaSuccess) return EQAT_ERR_CUDA;
-  const int zero[2] = {0, 0};
-  if (cudaMemcpyToSymbol(g_gemv_status, zero, sizeof(zero)) != cudaSuccess) return EQAT_ERR_CUDA;
-  *status = h[0];
-  *detail = h[1];
-  return EQAT_OK;
-}
+int launch_wait_expiry_gemv(cudaStream_t st) { return launch_wait_expiry(st); }
+int read_gemv_status(int* status, int* detail) { return read_wait_status(status, detail); }
 
 }  // namespace eqat

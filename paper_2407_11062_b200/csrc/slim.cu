@@ -37,6 +37,7 @@
 #include "gemv.cuh"
 #include "ptx.cuh"
 #include "slim.cuh"
+#include "wait.cuh"
 
 namespace eqat {
 namespace {
@@ -46,9 +47,6 @@ constexpr int kRun = 128;              // codes of a row per run
 constexpr int kSlimMaxTokens = 64;
 constexpr int kMaxSplit = 8;           // CTAs of a cluster (portable limit)
 constexpr int kMaxSmem = 232448;
-constexpr uint64_t kSlimWaitLimitNs = 2000000000ull;
-
-__device__ int g_slim_status[2];       // [0] = eqat_status, [1] = WaitSite
 
 struct SlimParams : PackedWeight {
   eqat_bf16* Y;                        // [T, out]
@@ -110,28 +108,6 @@ struct Slim {
     return need > least ? need : least;
   }
 };
-
-__device__ __forceinline__ bool slim_wait(uint32_t bar, uint32_t parity, volatile int* abort, int site, uint32_t sleep_ns,
-                                          uint64_t limit_ns = kSlimWaitLimitNs) {
-  if (ptx::mbar_try_wait(bar, parity)) return true;
-  uint64_t t0 = 0;
-  uint32_t n = 0;
-  while (!ptx::mbar_try_wait(bar, parity)) {
-    if (sleep_ns != 0) __nanosleep(sleep_ns);
-    if ((++n & 31u) == 0u) {
-      if (*abort) return false;
-      const uint64_t t = ptx::globaltimer_ns();
-      if (t0 == 0) t0 = t;                               // the clock is read only by waits that turn out long
-      if (t - t0 > limit_ns) {
-        *abort = 1;
-        atomicExch(&g_slim_status[1], site);
-        atomicExch(&g_slim_status[0], (int)EQAT_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
-}
 
 // Shared-memory matrix descriptor, K-major, 128-byte swizzle, 8-row atoms 1024 bytes apart.
 __device__ __forceinline__ uint64_t k_major_desc(uint32_t addr) {
@@ -305,7 +281,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       int st = 0;
       uint32_t ph = 1u;
       for (int b = 0; b < nboxes; ++b) {
-        if (!slim_wait(ptx::smem_addr(&ctl->empty[st]), ph, abort_flag, WAIT_PRODUCER_EMPTY, 32)) break;
+        if (!bounded_wait(ptx::smem_addr(&ctl->empty[st]), ph, abort_flag, WAIT_PRODUCER_EMPTY, 32)) break;
         ptx::fence_proxy_async_smem();                     // the row threads' reads of this stage before the copies' writes
         const uint32_t full = ptx::smem_addr(&ctl->full[st]), dst = ring_addr + st * C::kStage;
         const int run = run0 + b * kBoxRuns;
@@ -326,11 +302,10 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     uint32_t ph = 0, aph = 0;
     for (int r = 0; r < nruns; ++r) {
       const int in_box = r & (kBoxRuns - 1);
-      if ((in_box == 0 && !slim_wait(ptx::smem_addr(&ctl->full[st]), ph, abort_flag, WAIT_MMA_FULL, 0)) ||
-          !slim_wait(ptx::smem_addr(&ctl->a_full[g]), aph, abort_flag, WAIT_MMA_FULL, 0))
-        break;
+      bool got = in_box != 0 || bounded_wait(ptx::smem_addr(&ctl->full[st]), ph, abort_flag, WAIT_MMA_FULL);
+      if (got) got = bounded_wait(ptx::smem_addr(&ctl->a_full[g]), aph, abort_flag, WAIT_MMA_FULL);
       ptx::tc_fence_after();
-      if (ptx::elect_one()) {
+      if (ptx::elect_one() && got) {
         const uint32_t a = tmem + (uint32_t)(g * 64);
         const uint32_t d = tmem + (uint32_t)(C::kTmemA + g * ND * C::kTn);
         const uint64_t b = k_major_desc(ring_addr + st * C::kStage + C::kCodes + in_box * 2 * C::kBlock);
@@ -346,7 +321,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         ptx::mma_commit(ptx::smem_addr(&ctl->d_ready[g]));
         if (in_box == kBoxRuns - 1) ptx::mma_commit(ptx::smem_addr(&ctl->empty[st]));
       }
-      __syncwarp();
+      if (!__all_sync(0xFFFFFFFFu, got)) break;            // the warp gives up as a whole; off the path of the issue
       if (++g == kGroups) { g = 0; aph ^= 1u; }
       if (in_box == kBoxRuns - 1 && ++st == C::kStages) { st = 0; ph ^= 1u; }
     }
@@ -414,9 +389,8 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     uint32_t ph = 0;
     float s_run[ND], sz_run[ND];                           // step sizes of the run in flight (and -s z, fp16 zero points)
     auto collect = [&]() -> bool {                         // adds the accumulators of the run in flight
-      const bool got = slim_wait(ptx::smem_addr(&ctl->d_ready[g]), ph, abort_flag, WAIT_EPI_ACC_FULL, 0);
+      if (!bounded_wait_warp(ptx::smem_addr(&ctl->d_ready[g]), ph, abort_flag, WAIT_EPI_ACC_FULL)) return false;
       ph ^= 1u;
-      if (!__all_sync(0xFFFFFFFFu, got)) return false;
       ptx::tc_fence_after();
 #pragma unroll
       for (int i = 0; i < ND; ++i) {
@@ -467,8 +441,10 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       // With three a group skips boxes, and the box that used the stage last may be one of them: the group's run before is
       // collected first, since its MMAs come after those of that box.
       if (kGroups > 2 && r != g && !(ok = collect())) break;
-      const bool got = slim_wait(ptx::smem_addr(&ctl->full[st]), (uint32_t)(box / C::kStages) & 1u, abort_flag, WAIT_STREAM_FULL, 0);
-      if (!__all_sync(0xFFFFFFFFu, got)) { ok = false; break; }
+      if (!bounded_wait_warp(ptx::smem_addr(&ctl->full[st]), (uint32_t)(box / C::kStages) & 1u, abort_flag, WAIT_STREAM_FULL)) {
+        ok = false;
+        break;
+      }
       uint32_t w[4 * BITS], gp[ND];                        // codes of the run, parameters of its groups
       load_run<BITS>(ring_addr + st * C::kStage, box_row, r & (kBoxRuns - 1), w);
       const uint32_t* pw = params + ((((run0 + r) * kRun) >> p.group_shift) - group0) * kParamPitch + box_row;
@@ -544,19 +520,6 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem, tmem_cols);
   }
-}
-
-// The give-up path of slim_wait alone: one warp, a barrier nothing signals, a short limit.
-__global__ void slim_wait_expiry_kernel(uint64_t limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_word;
-  if (threadIdx.x == 0) {
-    ptx::mbar_init(ptx::smem_addr(&bar), 1);
-    abort_word = 0;
-    ptx::fence_mbar_init();
-  }
-  __syncthreads();
-  (void)slim_wait(ptx::smem_addr(&bar), 0u, &abort_word, WAIT_SELFTEST, 0, limit_ns);
 }
 
 template <int BITS, int NT, int ND>
@@ -697,20 +660,7 @@ int launch_slim_fwd(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, c
   }
 }
 
-int launch_wait_expiry_slim(cudaStream_t st) {
-  slim_wait_expiry_kernel<<<1, 32, 0, st>>>(1000000ull);   // 1 ms
-  return launch_status();
-}
-
-int read_slim_status(int* status, int* detail) {
-  int h[2] = {0, 0};
-  if (cudaDeviceSynchronize() != cudaSuccess) return EQAT_ERR_CUDA;
-  if (cudaMemcpyFromSymbol(h, g_slim_status, sizeof(h)) != cudaSuccess) return EQAT_ERR_CUDA;
-  const int zero[2] = {0, 0};
-  if (cudaMemcpyToSymbol(g_slim_status, zero, sizeof(zero)) != cudaSuccess) return EQAT_ERR_CUDA;
-  *status = h[0];
-  *detail = h[1];
-  return EQAT_OK;
-}
+int launch_wait_expiry_slim(cudaStream_t st) { return launch_wait_expiry(st); }
+int read_slim_status(int* status, int* detail) { return read_wait_status(status, detail); }
 
 }  // namespace eqat

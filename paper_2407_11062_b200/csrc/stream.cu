@@ -31,10 +31,9 @@
 #include "gemm.cuh"
 #include "ptx.cuh"
 #include "quant_math.cuh"
+#include "wait.cuh"
 
 namespace eqat {
-
-__device__ int g_stream_status[2];   // [0] = eqat_status, [1] = WaitSite
 
 namespace {
 
@@ -44,7 +43,6 @@ constexpr int kLaneElems = 32;                       // consecutive elements per
 constexpr int kTileRows = kConsumers / 2;            // 128-byte rows per tile (two lanes per row)
 constexpr int kTileElems = kConsumers * kLaneElems;  // 8192
 constexpr int kTileBytes = kTileElems * 2;           // 16 KB per input stream
-constexpr uint64_t kStreamWaitLimitNs = 2000000000ull;
 // Ring depth and CTAs per SM.  The stage a consumer works on is released as soon as its vectors are in
 // registers, so a few stages are enough to keep the copy engine busy.
 #ifndef EQAT_STREAM_CTAS1
@@ -67,26 +65,6 @@ struct RingCtl {
   int abort;
 };
 static_assert(sizeof(RingCtl) <= 256, "ring control block must fit its reservation");
-
-__device__ __forceinline__ bool ring_wait(uint32_t bar, uint32_t parity, volatile int* abort, int site,
-                                          uint32_t sleep_ns, uint64_t limit_ns = kStreamWaitLimitNs) {
-  if (ptx::mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = ptx::globaltimer_ns();
-  uint32_t n = 0;
-  while (!ptx::mbar_try_wait(bar, parity)) {
-    if (sleep_ns != 0) __nanosleep(sleep_ns);
-    if ((++n & 31u) == 0u) {
-      if (*abort) return false;
-      if (ptx::globaltimer_ns() - t0 > limit_ns) {
-        *abort = 1;
-        atomicExch(&g_stream_status[1], site);
-        atomicExch(&g_stream_status[0], (int)EQAT_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
-}
 
 // Runs `body(e0, raw, params)` on every consumer lane for every tile this CTA
 // owns: e0 is the index of the lane's first element, raw[i][u] the lane's
@@ -130,7 +108,7 @@ __device__ __forceinline__ void stream_tiles(const CUtensorMap* const (&maps)[NI
       size_t issued = 0;
       bool ok = true;
       for (size_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        if (!ring_wait(ptx::smem_addr(&ctl->empty[stage]), phase ^ 1u, abort_flag, WAIT_STREAM_EMPTY, 32)) {
+        if (!bounded_wait(ptx::smem_addr(&ctl->empty[stage]), phase ^ 1u, abort_flag, WAIT_STREAM_EMPTY, 32)) {
           ok = false;
           break;
         }
@@ -152,7 +130,7 @@ __device__ __forceinline__ void stream_tiles(const CUtensorMap* const (&maps)[NI
           const uint64_t t0 = ptx::globaltimer_ns();
           while (!ptx::mbar_try_wait(bar, par)) {
             if (ptx::globaltimer_ns() - t0 > 50000000ull) {
-              atomicExch(&g_stream_status[1], (int)WAIT_TEARDOWN);
+              atomicExch(&g_wait_status[1], (int)WAIT_TEARDOWN);
               break;
             }
           }
@@ -170,9 +148,7 @@ __device__ __forceinline__ void stream_tiles(const CUtensorMap* const (&maps)[NI
     for (size_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
       const Params cur = next;
       if (tile + gridDim.x < n_tiles) next = fetch((tile + gridDim.x) * kTileElems + (size_t)threadIdx.x * kLaneElems);
-      // the lanes of a warp leave together: the bodies shuffle across the whole warp
-      const bool got = ring_wait(ptx::smem_addr(&ctl->full[stage]), phase, abort_flag, WAIT_STREAM_FULL, 0);
-      if (!__all_sync(0xFFFFFFFFu, got)) break;
+      if (!bounded_wait_warp(ptx::smem_addr(&ctl->full[stage]), phase, abort_flag, WAIT_STREAM_FULL)) break;
       uint4 raw[NIN][4];
       const uint32_t st = smem_base + stage * R::kStageBytes + row_off;
 #pragma unroll
@@ -459,19 +435,6 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
   });
 }
 
-// The give-up path of ring_wait alone: one warp, a barrier nothing signals, a short limit.
-__global__ void ring_wait_expiry_kernel(uint64_t limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_word;
-  if (threadIdx.x == 0) {
-    ptx::mbar_init(ptx::smem_addr(&bar), 1);
-    abort_word = 0;
-    ptx::fence_mbar_init();
-  }
-  __syncthreads();
-  (void)ring_wait(ptx::smem_addr(&bar), 0u, &abort_word, WAIT_SELFTEST, 0, limit_ns);
-}
-
 // The flattened [out, in] weight as rows of 64 elements, one tile of kTileRows rows per copy.
 inline bool weight_map(CUtensorMap* tm, const eqat_bf16* p, size_t n_elem) {
   return make_tmap_bf16(tm, p, 64, n_elem / 64, kTileRows);
@@ -573,20 +536,7 @@ int launch_quantize_pack(const eqat_desc& d, const eqat_bf16* W, const float* s,
   }
 }
 
-int launch_wait_expiry_stream(cudaStream_t st) {
-  ring_wait_expiry_kernel<<<1, 32, 0, st>>>(1000000ull);   // 1 ms
-  return launch_status();
-}
-
-int read_stream_status(int* status, int* detail) {
-  int h[2] = {0, 0};
-  if (cudaDeviceSynchronize() != cudaSuccess) return EQAT_ERR_CUDA;
-  if (cudaMemcpyFromSymbol(h, g_stream_status, sizeof(h)) != cudaSuccess) return EQAT_ERR_CUDA;
-  const int zero[2] = {0, 0};
-  if (cudaMemcpyToSymbol(g_stream_status, zero, sizeof(zero)) != cudaSuccess) return EQAT_ERR_CUDA;
-  *status = h[0];
-  *detail = h[1];
-  return EQAT_OK;
-}
+int launch_wait_expiry_stream(cudaStream_t st) { return launch_wait_expiry(st); }
+int read_stream_status(int* status, int* detail) { return read_wait_status(status, detail); }
 
 }  // namespace eqat

@@ -20,6 +20,7 @@
 #include "gemm.cuh"
 #include "ptx.cuh"
 #include "wide.cuh"
+#include "wait.cuh"
 
 namespace eqat {
 namespace {
@@ -31,9 +32,6 @@ constexpr int kThreads = (2 + 4 * kGroups) * 32;
 constexpr int kMaxTn = 256;
 constexpr int kTmemA = kGroups * 64;   // columns of the A operand; the accumulators follow
 constexpr int kMaxSmem = 232448;
-constexpr uint64_t kWideWaitLimitNs = 2000000000ull;
-
-__device__ int g_wide_status[2];       // [0] = eqat_status, [1] = WaitSite
 
 struct WideParams : PackedWeight {
   eqat_bf16* Y;                        // [T, out]
@@ -54,28 +52,6 @@ struct WideCtl {
 
 __host__ __device__ constexpr int code_bytes(int bits) { return 16 * bits; }             // of a row per run
 __host__ __device__ inline int stage_bytes(int bits, int tn) { return kRows * code_bytes(bits) + tn * 128; }
-
-__device__ __forceinline__ bool wide_wait(uint32_t bar, uint32_t parity, volatile int* abort, int site, uint32_t sleep_ns,
-                                          uint64_t limit_ns = kWideWaitLimitNs) {
-  if (ptx::mbar_try_wait(bar, parity)) return true;
-  uint64_t t0 = 0;
-  uint32_t n = 0;
-  while (!ptx::mbar_try_wait(bar, parity)) {
-    if (sleep_ns != 0) __nanosleep(sleep_ns);
-    if ((++n & 31u) == 0u) {
-      if (*abort) return false;
-      const uint64_t t = ptx::globaltimer_ns();
-      if (t0 == 0) t0 = t;                               // the clock is read only by waits that turn out long
-      if (t - t0 > limit_ns) {
-        *abort = 1;
-        atomicExch(&g_wide_status[1], site);
-        atomicExch(&g_wide_status[0], (int)EQAT_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
-}
 
 // Shared-memory matrix descriptor, K-major, 128-byte swizzle, 8-row atoms 1024 bytes apart.
 __device__ __forceinline__ uint64_t k_major_desc(uint32_t addr) {
@@ -150,7 +126,7 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       int st = 0;
       uint32_t ph = 1u;
       for (int r = 0; r < nruns; ++r) {
-        if (!wide_wait(ptx::smem_addr(&ctl->empty[st]), ph, abort_flag, WAIT_PRODUCER_EMPTY, 32)) break;
+        if (!bounded_wait(ptx::smem_addr(&ctl->empty[st]), ph, abort_flag, WAIT_PRODUCER_EMPTY, 32)) break;
         ptx::fence_proxy_async_smem();                     // the row threads' reads of this stage before the copies' writes
         const uint32_t dst = ring_addr + st * stage_size, full_c = ptx::smem_addr(&ctl->full_c[st]);
         const uint32_t full_x = lead(&ctl->full_x[st]);
@@ -174,13 +150,10 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       uint32_t ph = 0, aph = 0;
       bool ok = true;
       for (int r = 0; r < nruns; ++r) {
-        if (!wide_wait(ptx::smem_addr(&ctl->full_x[st]), ph, abort_flag, WAIT_MMA_FULL, 0) ||
-            !wide_wait(ptx::smem_addr(&ctl->a_full[g]), aph, abort_flag, WAIT_MMA_FULL, 0)) {
-          ok = false;
-          break;
-        }
+        bool got = bounded_wait(ptx::smem_addr(&ctl->full_x[st]), ph, abort_flag, WAIT_MMA_FULL);
+        if (got) got = bounded_wait(ptx::smem_addr(&ctl->a_full[g]), aph, abort_flag, WAIT_MMA_FULL);
         ptx::tc_fence_after();
-        if (ptx::elect_one()) {
+        if (ptx::elect_one() && got) {
           const uint32_t a = tmem + (uint32_t)(g * 64);
           const uint64_t b = k_major_desc(ring_addr + st * stage_size);
 #pragma unroll
@@ -189,7 +162,8 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                                   (r | kk) != 0 ? 1u : 0u);
           ptx::mma_commit_pair_mask(ptx::smem_addr(&ctl->empty[st]), both);
         }
-        __syncwarp();
+        ok = __all_sync(0xFFFFFFFFu, got);                 // the warp gives up as a whole; off the path of the issue
+        if (!ok) break;
         if (++g == kGroups) { g = 0; aph ^= 1u; }
         if (++st == stages) { st = 0; ph ^= 1u; }
       }
@@ -217,14 +191,13 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       // that run is not after the group's run before, whose MMAs are done.
       if (r != g) {
         const int before = r - kGroups;
-        const bool fr = wide_wait(ptx::smem_addr(&ctl->empty[before % stages]), (uint32_t)(before / stages) & 1u, abort_flag,
-                                  WAIT_DEQ_OPERAND_EMPTY, 0);
-        if (!__all_sync(0xFFFFFFFFu, fr)) break;
+        if (!bounded_wait_warp(ptx::smem_addr(&ctl->empty[before % stages]), (uint32_t)(before / stages) & 1u, abort_flag,
+                               WAIT_DEQ_OPERAND_EMPTY))
+          break;
         ptx::tc_fence_after();
       }
       const int st = r % stages;
-      const bool got = wide_wait(ptx::smem_addr(&ctl->full_c[st]), (uint32_t)(r / stages) & 1u, abort_flag, WAIT_STREAM_FULL, 0);
-      if (!__all_sync(0xFFFFFFFFu, got)) break;
+      if (!bounded_wait_warp(ptx::smem_addr(&ctl->full_c[st]), (uint32_t)(r / stages) & 1u, abort_flag, WAIT_STREAM_FULL)) break;
       uint32_t w[4 * BITS];
       load_run<BITS>(ring_addr + st * stage_size + p.tn * 128, box_row, w);
       ptx::fence_proxy_async_smem();                       // the codes are in registers
@@ -258,8 +231,7 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   // CTA ks of a row tile owns token columns [ks, ks + 1) * tn / split of the tile.  The ring is free once every CTA's
   // MMAs are done: the sums go over it, [source][column / 4][row][column % 4] fp32.
   __syncwarp();
-  const bool done = wide_wait(ptx::smem_addr(&ctl->acc_full), 0u, abort_flag, WAIT_EPI_ACC_FULL, 64);
-  const bool all_done = __all_sync(0xFFFFFFFFu, done);
+  const bool all_done = bounded_wait_warp(ptx::smem_addr(&ctl->acc_full), 0u, abort_flag, WAIT_EPI_ACC_FULL, 64);
   ptx::tc_fence_after();
   ptx::cluster_arrive();
   ptx::cluster_wait();
@@ -330,19 +302,6 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   }
   __syncwarp();
   ptx::cluster_wait();
-}
-
-// The give-up path of wide_wait alone: one warp, a barrier nothing signals, a short limit.
-__global__ void wide_wait_expiry_kernel(uint64_t limit_ns) {
-  __shared__ uint64_t bar;
-  __shared__ int abort_word;
-  if (threadIdx.x == 0) {
-    ptx::mbar_init(ptx::smem_addr(&bar), 1);
-    abort_word = 0;
-    ptx::fence_mbar_init();
-  }
-  __syncthreads();
-  (void)wide_wait(ptx::smem_addr(&bar), 0u, &abort_word, WAIT_SELFTEST, 0, limit_ns);
 }
 
 int stages_that_fit(int bits, int tn) {                    // at least five (256 tokens, 4-bit codes)
@@ -480,20 +439,7 @@ int launch_wide_fwd(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, c
   }
 }
 
-int launch_wait_expiry_wide(cudaStream_t st) {
-  wide_wait_expiry_kernel<<<1, 32, 0, st>>>(1000000ull);   // 1 ms
-  return launch_status();
-}
-
-int read_wide_status(int* status, int* detail) {
-  int h[2] = {0, 0};
-  if (cudaDeviceSynchronize() != cudaSuccess) return EQAT_ERR_CUDA;
-  if (cudaMemcpyFromSymbol(h, g_wide_status, sizeof(h)) != cudaSuccess) return EQAT_ERR_CUDA;
-  const int zero[2] = {0, 0};
-  if (cudaMemcpyToSymbol(g_wide_status, zero, sizeof(zero)) != cudaSuccess) return EQAT_ERR_CUDA;
-  *status = h[0];
-  *detail = h[1];
-  return EQAT_OK;
-}
+int launch_wait_expiry_wide(cudaStream_t st) { return launch_wait_expiry(st); }
+int read_wide_status(int* status, int* detail) { return read_wait_status(status, detail); }
 
 }  // namespace eqat

@@ -45,6 +45,24 @@ def test_tensor_memory_of_overlapped_and_paired_launches():
     assert checked == 3
 
 
+def test_warps_give_up_a_wait_together():
+    """Read in the sources: only waits of a single lane (producers, teardown) are decided lane by lane.  What a whole warp
+    waits for goes through the form that votes, or its result is voted on before the warp goes on, since elect.sync,
+    shuffles and tensor-core instructions follow."""
+    one_lane, waits, alone = {"WAIT_PRODUCER_EMPTY", "WAIT_STREAM_EMPTY", "WAIT_TEARDOWN"}, 0, []
+    for name, text in sources():
+        for m in re.finditer(r"([^;{}]*?)(\w+)(?:<\w+>)?\(\s*ptx::smem_addr\(&ctl->[^;{]*?abort_flag,\s*(WAIT_\w+)", text):
+            waits += 1
+            before, function, site = m.groups()
+            result = re.search(r"(\w+) = [^;]*$", before)
+            rest = text[m.end():m.end() + 6000]
+            into = result and re.search(r"(\w+) = %s &&" % result.group(1), rest)          # or with the wait that follows
+            voted = result and any(re.search(r"(?:warp_agrees\(|__all_sync\(0xFFFFFFFFu, )%s\)" % v.group(1), rest) for v in (result, into) if v)
+            if site not in one_lane and function != "bounded_wait_warp" and not voted:
+                alone.append((name, function, site))
+    assert waits >= 20 and not alone
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("bits,group", [(2, 64), (3, 128), (4, 512), (4, 32)])
 def test_operands_rewritten_between_overlapped_launches(bits, group):
