@@ -231,10 +231,26 @@ int eqat_unpack_zeros(const eqat_desc* desc, const uint8_t* z_packed, uint8_t* z
  * multiply fp32 sums, so (W_int - z) * s is not rounded to bf16: a matrix-vector
  * kernel of up to eight tokens per launch for the smallest batches (groups of at
  * least 64; a token's result does not depend on how the tokens were sliced into
- * launches), a kernel on tiles of 128 weight rows otherwise.
+ * launches), a kernel on tiles of 128 weight rows otherwise.  (Rows of more than
+ * 57344 columns may not fit either; they are then treated like larger batches,
+ * where (W_int - z) * s is rounded to bf16.)
  *   X [T,in] bf16, Wq_packed, s16, z (in)   Y [T,out] bf16 (out) */
 int qlinear_packed_fwd(const eqat_desc* desc, const eqat_bf16* X, const uint8_t* Wq_packed,
                        const eqat_fp16* s16, const void* z, eqat_bf16* Y, void* stream);
+
+/* Which kernel qlinear_packed_fwd takes for a problem, decided on the host from
+ * the descriptor alone (a diagnostic; no counterpart in the paper).  `sms`: the
+ * number of SMs to decide for, 0 for the current device.  Returns one of the
+ * EQAT_ROUTE_* values or a negative eqat_status.  h_plan (may be NULL) receives
+ * three numbers: launches or token tiles, tokens of each, and the split of K
+ * over a cluster (0, 0, 1 for the tiled kernel). */
+enum {
+  EQAT_ROUTE_MATRIX_VECTOR = 1,     /* a few tokens: up to eight per pass over the weight   */
+  EQAT_ROUTE_WEIGHT_ROWS = 2,       /* up to 64 tokens: tiles of 128 weight rows            */
+  EQAT_ROUTE_WEIGHT_ROW_PAIRS = 3,  /* prompts: tiles of 256 weight rows                    */
+  EQAT_ROUTE_TILED = 4              /* large batches: tiles of 512 or 256 tokens            */
+};
+int eqat_packed_fwd_route(const eqat_desc* desc, int sms, int* h_plan);
 
 /* dX = dY * ((W_int - z) * s).
  *   dY [T,out] bf16, Wq_packed, s16, z (in)   dX [T,in] bf16 (out) */

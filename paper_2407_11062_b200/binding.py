@@ -21,6 +21,7 @@ EQAT_ERR_NULL, EQAT_ERR_SHAPE, EQAT_ERR_ALIGN, EQAT_ERR_UNSUPPORTED = -1, -2, -3
 EQAT_ERR_WORKSPACE, EQAT_ERR_CUDA, EQAT_ERR_TIMEOUT = -5, -6, -7
 EQAT_OP_FAKEQUANT_BWD, EQAT_OP_PACKED_BWD_DS = 1, 2
 EQAT_ZP_U8, EQAT_ZP_FP16 = 0, 1
+EQAT_ROUTE_MATRIX_VECTOR, EQAT_ROUTE_WEIGHT_ROWS, EQAT_ROUTE_WEIGHT_ROW_PAIRS, EQAT_ROUTE_TILED = 1, 2, 3, 4
 
 
 class EqatError(RuntimeError):
@@ -70,6 +71,7 @@ def _load():
         "eqat_pack_zeros": (c_int, [D, P, P, P]),
         "eqat_unpack_zeros": (c_int, [D, P, P, P]),
         "qlinear_packed_fwd": (c_int, [D, P, P, P, P, P, P]),
+        "eqat_packed_fwd_route": (c_int, [D, c_int, POINTER(c_int)]),
         "qlinear_packed_bwd_dx": (c_int, [D, P, P, P, P, P, P]),
         "qlinear_packed_bwd_ds": (c_int, [D, P, P, P, P, P, P, P, P, c_size_t, P]),
         "eqat_block_ap_step": (c_int, [POINTER(eqat_block_ap_linear), c_int, POINTER(c_int), P]),
@@ -199,6 +201,15 @@ def eqat_unpack_zeros(desc, z_packed, z8):
 def qlinear_packed_fwd(desc, X, Wq_packed, s16, z8, Y):
     _check(lib.qlinear_packed_fwd(ctypes.byref(desc), _ptr(X), _ptr(Wq_packed), _ptr(s16), _ptr(z8), _ptr(Y),
                                   _stream()), "qlinear_packed_fwd")
+
+
+def eqat_packed_fwd_route(desc, sms=0):
+    """The kernel qlinear_packed_fwd takes (EQAT_ROUTE_*), and its plan: launches or token tiles, tokens of each, split of K."""
+    plan = (c_int * 3)()
+    kernel = lib.eqat_packed_fwd_route(ctypes.byref(desc), int(sms), plan)
+    if kernel < 0:
+        raise EqatError(kernel, "eqat_packed_fwd_route")
+    return kernel, tuple(plan)
 
 
 def qlinear_packed_bwd_dx(desc, dY, Wq_packed, s16, z8, dX):

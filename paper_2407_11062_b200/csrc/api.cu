@@ -111,6 +111,24 @@ int v_packed_bwd_ds(const eqat_desc* d, const eqat_bf16* X, const eqat_bf16* dY,
   return EQAT_OK;
 }
 
+// The kernel that takes a packed forward.
+struct PackedRoute {
+  int kernel;                            // EQAT_ROUTE_*
+  SlimPlan slim;
+  WidePlan wide;
+};
+
+// On the current device (sms = 0), or as on a device of `sms` SMs.
+PackedRoute packed_route(const eqat_desc& d, int sms) {
+  PackedRoute r{};
+  if (slim_fwd_applies(d, sms > 0 ? sms : sm_count(), r.slim)) r.kernel = EQAT_ROUTE_WEIGHT_ROWS;
+  // a handful of tokens (decoding): one pass over the packed weight instead of near-empty tensor-core tiles
+  else if (packed_gemv_applies(d)) r.kernel = EQAT_ROUTE_MATRIX_VECTOR;
+  else if (wide_fwd_applies(d, sms, r.wide)) r.kernel = EQAT_ROUTE_WEIGHT_ROW_PAIRS;
+  else r.kernel = EQAT_ROUTE_TILED;
+  return r;
+}
+
 #define EQAT_TRY(expr)            \
   do {                            \
     const int rc__ = (expr);      \
@@ -258,13 +276,28 @@ int eqat_unpack_zeros(const eqat_desc* d, const uint8_t* z_packed, uint8_t* z8, 
 int qlinear_packed_fwd(const eqat_desc* d, const eqat_bf16* X, const uint8_t* Wq_packed, const eqat_fp16* s16,
                        const void* z, eqat_bf16* Y, void* stream) {
   EQAT_TRY(v_packed_fwd(d, X, Wq_packed, s16, z, Y));
-  SlimPlan plan;
-  if (slim_fwd_applies(*d, plan)) return launch_slim_fwd(*d, X, Wq_packed, s16, z, Y, plan, as_stream(stream));
-  // a handful of tokens (decoding): one pass over the packed weight instead of near-empty tensor-core tiles
-  if (packed_gemv_applies(*d)) return launch_packed_gemv(*d, X, Wq_packed, s16, z, Y, as_stream(stream));
-  WidePlan wide;
-  if (wide_fwd_applies(*d, wide)) return launch_wide_fwd(*d, X, Wq_packed, s16, z, Y, wide, as_stream(stream));
-  return launch_packed_fwd(*d, X, Wq_packed, s16, z, Y, as_stream(stream));
+  const PackedRoute r = packed_route(*d, 0);
+  switch (r.kernel) {
+    case EQAT_ROUTE_WEIGHT_ROWS: return launch_slim_fwd(*d, X, Wq_packed, s16, z, Y, r.slim, as_stream(stream));
+    case EQAT_ROUTE_MATRIX_VECTOR: return launch_packed_gemv(*d, X, Wq_packed, s16, z, Y, as_stream(stream));
+    case EQAT_ROUTE_WEIGHT_ROW_PAIRS: return launch_wide_fwd(*d, X, Wq_packed, s16, z, Y, r.wide, as_stream(stream));
+    default: return launch_packed_fwd(*d, X, Wq_packed, s16, z, Y, as_stream(stream));
+  }
+}
+
+int eqat_packed_fwd_route(const eqat_desc* d, int sms, int* h_plan) {
+  EQAT_TRY(check_gemm_desc(d, true));
+  if (sms < 0) return EQAT_ERR_SHAPE;
+  const PackedRoute r = packed_route(*d, sms);
+  if (h_plan != nullptr) {
+    const FewTokenPlan gemv = packed_gemv_plan(*d);
+    const bool mv = r.kernel == EQAT_ROUTE_MATRIX_VECTOR, rows = r.kernel == EQAT_ROUTE_WEIGHT_ROWS;
+    const bool pairs = r.kernel == EQAT_ROUTE_WEIGHT_ROW_PAIRS;
+    h_plan[0] = mv ? gemv.launches : (rows ? r.slim.token_tiles : (pairs ? r.wide.token_tiles : 0));
+    h_plan[1] = mv ? gemv.slice : (rows ? 16 * r.slim.nt : (pairs ? r.wide.tn : 0));
+    h_plan[2] = rows ? r.slim.split : (pairs ? r.wide.split : 1);
+  }
+  return r.kernel;
 }
 
 int qlinear_packed_bwd_dx(const eqat_desc* d, const eqat_bf16* dY, const uint8_t* Wq_packed, const eqat_fp16* s16,

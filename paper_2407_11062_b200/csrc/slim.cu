@@ -577,34 +577,38 @@ int smem_for(int nt, int nd, bool zf, int groups) {
 // outside its runs (start, exchange) and 0.06 us per group of parameters, a run 0.38 us alone on its SM and 0.34 us per
 // SM where two CTAs share it (a quarter more with more than 16 token columns); behind the first two, a CTA's fixed part
 // is mostly hidden by its neighbour's runs, and clusters of eight leave SMs of a GPC empty.
-SlimPlan slim_plan(const eqat_desc& d) {
+SlimPlan slim_plan(const eqat_desc& d, int sms) {
   SlimPlan best{};
   const bool zf = d.zero_point_format == EQAT_ZP_FP16;
-  const int T = (int)d.tokens, sms = sm_count();
+  const int T = (int)d.tokens;
   if (sms <= 0) return best;
   const int nd = d.group == 32 ? 4 : (d.group == 64 ? 2 : 1);
   // 16-column accumulators that fit tensor memory beside the A operand (fp16 zero points need the column sums as well)
   const int cap = nd == 4 ? 1 : (nd == 2 ? (zf ? 2 : 3) : (zf ? 3 : 4));
-  const int token_tiles = (T + 16 * cap - 1) / (16 * cap);
-  const int nt = ((T + token_tiles - 1) / token_tiles + 15) / 16;
-  const int tiles = ((d.out_features + kRows - 1) / kRows) * token_tiles, runs = d.in_features / kRun;
+  const int runs = d.in_features / kRun;
   const int boxes = (runs + kBoxRuns - 1) / kBoxRuns, shift = d.group <= 256 ? log2_exact(d.group) : 31;
-  for (int lg = 0; (1 << lg) <= kMaxSplit && (1 << lg) <= boxes; ++lg) {
-    const int split = 1 << lg;
-    // the longest slice, and the groups it touches (it starts at a multiple of 256 columns)
-    const int most = min(runs, ((boxes + split - 1) >> lg) * kBoxRuns);
-    const int groups = ((most * kRun - 1) >> shift) + 1;
-    const int smem = d.bits == 2   ? smem_for<2>(nt, nd, zf, groups)
-                     : d.bits == 3 ? smem_for<3>(nt, nd, zf, groups)
-                                   : smem_for<4>(nt, nd, zf, groups);
-    if (smem > kMaxSmem) continue;
-    const bool two = nt <= 2 && smem <= 113 * 1024;
-    const int n = (tiles * split + sms - 1) / sms;         // CTAs of the busiest SM
-    const double wide = nt == 1 ? 1.0 : 1.25, fixed = 4.0 + 0.06 * groups;
-    double us = two ? fixed + n * most * (n == 1 ? 0.38 : 0.34) * wide + (n > 2 ? (n - 2) * 0.7 : 0.0)
-                    : n * (fixed + most * 0.36 * wide);
-    if (split == 8 && n > 2) us *= 1.15;
-    if (best.us == 0.0 || us < best.us) best = SlimPlan{nt, nd, token_tiles, split, groups, us};
+  // The fewest token tiles that fit: a tile's parameters and partial sums share a CTA's shared memory, and on very long rows
+  // (49152 columns, 3-bit codes, groups of 64, 40 tokens: 235 KB) only narrower tiles leave room for them.
+  for (int token_tiles = (T + 16 * cap - 1) / (16 * cap); best.us == 0.0 && token_tiles <= (T + 15) / 16; ++token_tiles) {
+    const int nt = ((T + token_tiles - 1) / token_tiles + 15) / 16;
+    const int tiles = ((d.out_features + kRows - 1) / kRows) * token_tiles;
+    for (int lg = 0; (1 << lg) <= kMaxSplit && (1 << lg) <= boxes; ++lg) {
+      const int split = 1 << lg;
+      // the longest slice, and the groups it touches (it starts at a multiple of 256 columns)
+      const int most = min(runs, ((boxes + split - 1) >> lg) * kBoxRuns);
+      const int groups = ((most * kRun - 1) >> shift) + 1;
+      const int smem = d.bits == 2   ? smem_for<2>(nt, nd, zf, groups)
+                       : d.bits == 3 ? smem_for<3>(nt, nd, zf, groups)
+                                     : smem_for<4>(nt, nd, zf, groups);
+      if (smem > kMaxSmem) continue;
+      const bool two = nt <= 2 && smem <= 113 * 1024;
+      const int n = (tiles * split + sms - 1) / sms;         // CTAs of the busiest SM
+      const double wide = nt == 1 ? 1.0 : 1.25, fixed = 4.0 + 0.06 * groups;
+      double us = two ? fixed + n * most * (n == 1 ? 0.38 : 0.34) * wide + (n > 2 ? (n - 2) * 0.7 : 0.0)
+                      : n * (fixed + most * 0.36 * wide);
+      if (split == 8 && n > 2) us *= 1.15;
+      if (best.us == 0.0 || us < best.us) best = SlimPlan{nt, nd, token_tiles, split, groups, us};
+    }
   }
   return best;
 }
@@ -631,11 +635,11 @@ int launch_bits(const SlimPlan& pl, const SlimParams& p, const eqat_bf16* X, dim
 // so this one has to be a quarter better (13824 x 5120, 4-bit codes, 6 tokens: estimated 15.5 against 18.7 us, measured
 // 21.2 against 18.3 us).  Weights under 3 MB keep the matrix-vector kernel while it needs at most two launches, so that
 // for them a token gives the same bits alone and in any batch of up to eight or sixteen.
-bool slim_fwd_applies(const eqat_desc& d, SlimPlan& pl) {
+bool slim_fwd_applies(const eqat_desc& d, int sms, SlimPlan& pl) {
   if (d.tokens > kSlimMaxTokens) return false;
   const FewTokenPlan gemv = packed_gemv_plan(d);
   if (gemv.launches == 1 && d.tokens <= 2) return false;   // the matrix-vector kernel on every shape measured
-  pl = slim_plan(d);
+  pl = slim_plan(d, sms);
   if (pl.us == 0.0) return false;
   if (!packed_gemv_applies(d)) return true;
   const double weight_bytes = (double)d.out_features * d.in_features * d.bits / 8.0;

@@ -12,8 +12,8 @@ struct SlimPlan {
   int groups;                // quantisation groups of a row, the most that one CTA's slice touches
   double us;                 // 0: the problem does not fit
 };
-// True when the weight-row kernel is the one to take for this packed forward, and how.
-bool slim_fwd_applies(const eqat_desc& d, SlimPlan& plan);
+// True when the weight-row kernel is the one to take for this packed forward on a device of `sms` SMs, and how.
+bool slim_fwd_applies(const eqat_desc& d, int sms, SlimPlan& plan);
 // Y[T,out] = X[T,in] * dequant(Wq)^T
 int launch_slim_fwd(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16, const void* zq,
                     eqat_bf16* Y, const SlimPlan& plan, cudaStream_t st);

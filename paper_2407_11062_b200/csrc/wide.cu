@@ -389,16 +389,16 @@ int launch_bits(const WideParams& p, const eqat_bf16* X, dim3 ctas, cudaStream_t
 // loading.  There: 8 us and 0.65 / 0.72 / 0.67 us per tile and 64 input columns, a tenth more with most SMs at work, or,
 // for at most 256 tokens, 0.88 / 1.13 / 1.15 us on one CTA.  4096 x 4096, 2 bits: 128 tokens 64.2 -> 13.2 us, 333 tokens
 // 49.4 -> 16.2 us, 1024 tokens 49.8 -> 29 us; at 2048 tokens the tiled kernel is ahead (51 against 58 us).
-bool wide_fwd_applies(const eqat_desc& d, WidePlan& best) {
+bool wide_fwd_applies(const eqat_desc& d, int given_sms, WidePlan& best) {
   best = WidePlan{0, 0, 0, 0.0};
-  const int sms = sm_count();
+  const int sms = given_sms > 0 ? given_sms : sm_count();
   if (d.tokens > 4096 || sms < 2) return false;
   const int T = (int)d.tokens, runs = d.in_features / kRun, pairs = (d.out_features + 2 * kRows - 1) / (2 * kRows);
   const int least = (T + kMaxTn - 1) / kMaxTn;
   for (int tt = least; tt <= least + 3; ++tt) {
     const int tn = ((T + tt - 1) / tt + 31) / 32 * 32;
     for (int lg = 0; (1 << lg) <= kMaxSplit && (1 << lg) <= runs; ++lg) {
-      const int clusters = pairs * tt, resident = max_clusters(d.bits, lg);
+      const int clusters = pairs * tt, resident = given_sms > 0 ? sms / (2 << lg) : max_clusters(d.bits, lg);
       if (resident <= 0) continue;
       const int rounds = (clusters + resident - 1) / resident;
       const double expand = d.bits == 3 ? 0.62 : 0.41, mma = 0.0021 * tn;

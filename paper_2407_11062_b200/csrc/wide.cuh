@@ -10,8 +10,9 @@ struct WidePlan {
   int split;                 // pairs of CTAs per cluster, over K
   double us;                 // expected time; 0: the problem does not fit
 };
-// True when the kernel is the one to take for this packed forward, and how.
-bool wide_fwd_applies(const eqat_desc& d, WidePlan& plan);
+// True when the kernel is the one to take for this packed forward, and how: on the current device (sms = 0), or on one of
+// `sms` SMs all of which make up clusters.
+bool wide_fwd_applies(const eqat_desc& d, int sms, WidePlan& plan);
 // Y[T,out] = X[T,in] * dequant(Wq)^T
 int launch_wide_fwd(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16, const void* zq,
                     eqat_bf16* Y, const WidePlan& plan, cudaStream_t st);

@@ -684,6 +684,8 @@ def test_few_token_forwards_back_to_back_keep_their_order(eqat, bits, group, tok
     (9472, 1024, 24, 4, 256, True),  # more CTAs than fit at a time, groups of two runs
     (2048, 8192, 8, 4, 128, False),  # eight tokens: cheaper than the matrix-vector kernel's two launches
     (64, 28672, 40, 3, 64, False),   # the longest rows
+    (64, 49152, 40, 3, 64, False),   # rows whose parameters leave room for narrower token tiles only
+    (128, 53248, 64, 4, 32, False),  # four of them
 ])
 def test_packed_forward_on_weight_row_tiles(eqat, out, in_f, tokens, bits, group, real_z):
     """The kernel on tiles of 128 weight rows (up to 64 tokens): nothing is rounded on the way to the fp32 sums, so beside

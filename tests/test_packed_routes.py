@@ -1,0 +1,54 @@
+"""Which kernel a packed forward goes to (decided on the host; here for a device of 148 SMs)."""
+import random
+
+import pytest
+
+SMS = 148
+
+
+@pytest.fixture(scope="module")
+def eqat():
+    from paper_2407_11062_b200.build import build_library
+    build_library()
+    from paper_2407_11062_b200 import binding
+    return binding
+
+
+def route(eqat, out, in_f, tokens, bits, group, fp16_z=False):
+    zfmt = eqat.EQAT_ZP_FP16 if fp16_z else eqat.EQAT_ZP_U8
+    return eqat.eqat_packed_fwd_route(eqat.make_desc(bits, group, out, in_f, tokens, 0, zfmt), SMS)
+
+
+def test_few_tokens_keep_exact_codes_on_long_rows(eqat):
+    """Up to 64 tokens neither kernel that takes them rounds (q - z) * s to bf16.  A token tile that does not fit shared
+    memory is no reason to leave them: narrower tiles do (here 49152 and 53248 columns, among a grid of shapes)."""
+    few = (eqat.EQAT_ROUTE_MATRIX_VECTOR, eqat.EQAT_ROUTE_WEIGHT_ROWS)
+    assert route(eqat, 2048, 49152, 40, 3, 64) == (eqat.EQAT_ROUTE_WEIGHT_ROWS, (2, 32, 4))
+    for in_f in (128, 384, 1024, 4096, 8192, 11008, 28672, 49152, 53248, 57344):
+        for out in (64, 1024, 2048, 28672):
+            for bits in (2, 3, 4):
+                for group in {32, 64, 128, min(in_f, 32768)} | ({256} if in_f % 256 == 0 else set()):
+                    if in_f % group or (group > 256 and group != in_f):
+                        continue
+                    for tokens in (1, 3, 8, 9, 13, 16, 17, 31, 33, 40, 48, 49, 64):
+                        for fp16_z in (False, True):
+                            assert route(eqat, out, in_f, tokens, bits, group, fp16_z)[0] in few, (out, in_f, bits, group, tokens)
+
+
+def test_plans_cover_all_tokens(eqat):
+    rng = random.Random(3)
+    for _ in range(3000):
+        in_f, out = 128 * rng.randint(1, 224), 64 * rng.randint(1, 448)
+        tokens, bits = int(4096 ** rng.random()) or 1, rng.choice([2, 3, 4])
+        kernel, (parts, each, split) = route(eqat, out, in_f, tokens, bits, rng.choice([32, 64, 128, in_f]))
+        if kernel == eqat.EQAT_ROUTE_TILED:
+            assert (parts, each, split) == (0, 0, 1)
+        else:
+            assert (parts - 1) * each < tokens <= parts * each and split in (1, 2, 4, 8)
+
+
+def test_the_query_checks_its_descriptor(eqat):
+    with pytest.raises(eqat.EqatError):
+        eqat.eqat_packed_fwd_route(eqat.make_desc(2, 64, 96, 512, 4), SMS)
+    with pytest.raises(eqat.EqatError):
+        eqat.eqat_packed_fwd_route(eqat.make_desc(2, 64, 512, 512, 4), -1)
