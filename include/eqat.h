@@ -234,6 +234,15 @@ int eqat_unpack_zeros(const eqat_desc* desc, const uint8_t* z_packed, uint8_t* z
  * launches), a kernel on tiles of 128 weight rows otherwise.  (Rows of more than
  * 57344 columns may not fit either; they are then treated like larger batches,
  * where (W_int - z) * s is rounded to bf16.)
+ *
+ * Repeated calls give the same bits on one device.  The bits of a token may
+ * depend on the batch around it: which kernel runs, and in which order it adds up
+ * K, follow the number of tokens, and above 64 tokens also the number of thread
+ * block clusters that the device keeps resident, so a token can differ in the
+ * last bits between batches of 7 and 8 tokens, between prefill chunks of 256 and
+ * 512, and between devices.  They do not depend on it where every batch of up to
+ * 16 tokens takes the matrix-vector kernel: weights of less than 3,000,000 bytes
+ * of codes (out*in*N/8), in_features from 1024 to 4096, groups of at least 64.
  *   X [T,in] bf16, Wq_packed, s16, z (in)   Y [T,out] bf16 (out) */
 int qlinear_packed_fwd(const eqat_desc* desc, const eqat_bf16* X, const uint8_t* Wq_packed,
                        const eqat_fp16* s16, const void* z, eqat_bf16* Y, void* stream);

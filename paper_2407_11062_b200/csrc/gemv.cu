@@ -731,9 +731,19 @@ FewTokenPlan packed_gemv_plan(const eqat_desc& d) {
   return FewTokenPlan{launches, slice, us};
 }
 
+// The range is a promise and not a matter of speed: from nine tokens on, which take two launches here, the weight-row kernel
+// is faster (1024 x 1024, 2 bits, 9 tokens 5.8 against 4.2 us; 1280 x 4096, 13 tokens 12.5 against 7.2 us).  It is kept where
+// that costs little.  16 tokens of 1024 x 8192 took 27.9 against 7.8 us, 9 tokens of 512 x 384 6.5 against 4.0 us: longer and
+// shorter rows go by time.  3 MB holds the linears of models of up to 2048 hidden units.
+bool packed_gemv_keeps_bits(const eqat_desc& d) {
+  return d.tokens <= 2 * kTcMaxTokens && d.in_features >= 1024 && d.in_features <= 4096 &&
+         (int64_t)d.out_features * d.in_features * d.bits < (int64_t)8 * 3000000 && packed_gemv_plan(d).launches > 0;
+}
+
 bool packed_gemv_applies(const eqat_desc& d) {
   const FewTokenPlan plan = packed_gemv_plan(d);
   if (plan.launches <= 1) return plan.launches == 1;
+  if (packed_gemv_keeps_bits(d)) return true;
   // several launches only while clearly cheaper than the tiled kernel, which takes about 1 / 1.45 / 1.2 us per 64 input
   // columns for any token count below a full row-tile, because the K loop of a tile is serial
   return plan.us < 0.8 * (d.in_features / 64.0 * (d.bits == 2 ? 1.0 : (d.bits == 3 ? 1.45 : 1.2)));

@@ -633,17 +633,15 @@ int launch_bits(const SlimPlan& pl, const SlimParams& p, const eqat_bf16* X, dim
 // one token of 4096 x 4096, 2-bit codes) but pays for every token and holds at most eight; this one costs the same for
 // any number up to 16 (7.1 us against 10.0 us at 8 tokens, 19.8 us in two launches at 16).  Two estimates are compared,
 // so this one has to be a quarter better (13824 x 5120, 4-bit codes, 6 tokens: estimated 15.5 against 18.7 us, measured
-// 21.2 against 18.3 us).  Weights under 3 MB keep the matrix-vector kernel while it needs at most two launches, so that
-// for them a token gives the same bits alone and in any batch of up to eight or sixteen.
+// 21.2 against 18.3 us).  Small weights keep the matrix-vector kernel for the sake of their bits (packed_gemv_keeps_bits).
 bool slim_fwd_applies(const eqat_desc& d, int sms, SlimPlan& pl) {
   if (d.tokens > kSlimMaxTokens) return false;
   const FewTokenPlan gemv = packed_gemv_plan(d);
   if (gemv.launches == 1 && d.tokens <= 2) return false;   // the matrix-vector kernel on every shape measured
+  if (packed_gemv_keeps_bits(d)) return false;
   pl = slim_plan(d, sms);
   if (pl.us == 0.0) return false;
   if (!packed_gemv_applies(d)) return true;
-  const double weight_bytes = (double)d.out_features * d.in_features * d.bits / 8.0;
-  if (gemv.launches <= 2 && weight_bytes < 3.0e6) return false;
   return gemv.launches > 1 || pl.us * 1.25 < gemv.us;
 }
 

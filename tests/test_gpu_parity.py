@@ -647,6 +647,30 @@ def test_few_token_forward_does_not_depend_on_the_slicing(eqat, bits, group):
     assert rel_err(torch_to_f64(Y), O.linear_fwd(torch_to_f64(X), What_o)) <= TOL
 
 
+@pytest.mark.parametrize("out,in_f,bits,group", [
+    (64, 1024, 2, 64),       # the shortest rows
+    (2880, 4096, 2, 64),     # 2.95 MB of codes, the most
+    (3904, 2048, 3, 2048),
+    (320, 1152, 4, 128),
+])
+def test_small_weights_give_a_token_the_same_bits_in_any_batch_of_up_to_sixteen(eqat, out, in_f, bits, group):
+    P, z8, s16, X = few_token_problem(out, in_f, 16, 23, bits, group)
+
+    def forward(x):
+        y = torch.empty(x.shape[0], out, dtype=torch.bfloat16, device="cuda")
+        eqat.qlinear_packed_fwd(eqat.make_desc(bits, group, out, in_f, x.shape[0]), x.contiguous(), P, s16, z8, y)
+        return y.view(torch.int16)
+
+    Y = forward(X)
+    for t in range(16):
+        assert torch.equal(forward(X[t:t + 1]), Y[t:t + 1]), t
+    for tokens in (2, 3, 8, 9, 13):
+        assert torch.equal(forward(X[:tokens]), Y[:tokens]), tokens
+    q = O.unpack_rows(P.cpu().numpy(), bits, in_f)
+    What_o = O.dequantize(q, s16.cpu().numpy().astype(np.float32), z8.cpu().numpy(), group)
+    assert rel_err(torch_to_f64(Y.view(torch.bfloat16)), O.linear_fwd(torch_to_f64(X), What_o)) <= TOL
+
+
 @pytest.mark.parametrize("bits,group,tokens", [(2, 64, 1), (2, 64, 8), (2, 64, 12), (3, 128, 5), (4, 128, 3), (4, 128, 12)])
 def test_few_token_forwards_back_to_back_keep_their_order(eqat, bits, group, tokens):
     """Twelve layers in a row, each reading what the one before wrote, issued without a pause (the launches may

@@ -35,6 +35,28 @@ def test_few_tokens_keep_exact_codes_on_long_rows(eqat):
                             assert route(eqat, out, in_f, tokens, bits, group, fp16_z)[0] in few, (out, in_f, bits, group, tokens)
 
 
+def test_small_weights_take_one_kernel_up_to_sixteen_tokens(eqat):
+    """The range over which a token's bits do not depend on its batch, and both sides of its boundary."""
+    def kernels(out, in_f, bits, group, tokens):
+        return {route(eqat, out, in_f, t, bits, group)[0] for t in tokens}
+
+    inside = {eqat.EQAT_ROUTE_MATRIX_VECTOR}
+    for in_f in (1024, 1152, 1408, 2048, 2944, 3072, 4096):
+        for bits in (2, 3, 4):
+            for group in {64, 128, in_f}:
+                largest = (8 * 3000000 - 1) // (in_f * bits) // 64 * 64
+                for out in {64, 192, 512, largest} if in_f % group == 0 else ():
+                    assert kernels(out, in_f, bits, group, range(1, 17)) == inside, (out, in_f, bits, group)
+                    assert kernels(out, in_f, bits, group, range(17, 65)) == {eqat.EQAT_ROUTE_WEIGHT_ROWS}
+    # outside: larger weights, longer and shorter rows and groups of 32 go by time
+    assert kernels(512, 384, 2, 64, range(9, 17)) == {eqat.EQAT_ROUTE_WEIGHT_ROWS}
+    assert kernels(2944, 4096, 2, 64, (1, 2)) == inside                     # 3,014,656 bytes
+    assert kernels(2944, 4096, 2, 64, range(9, 17)) == {eqat.EQAT_ROUTE_WEIGHT_ROWS}
+    assert kernels(1024, 5120, 2, 64, range(9, 17)) == {eqat.EQAT_ROUTE_WEIGHT_ROWS}
+    assert kernels(1024, 8192, 2, 64, (8, 16)) == {eqat.EQAT_ROUTE_WEIGHT_ROWS}
+    assert kernels(1024, 2048, 2, 32, range(1, 17)) == {eqat.EQAT_ROUTE_WEIGHT_ROWS}
+
+
 def test_plans_cover_all_tokens(eqat):
     rng = random.Random(3)
     for _ in range(3000):
