@@ -573,7 +573,7 @@ int smem_for(int nt, int nd, bool zf, int groups) {
 }
 
 // The split of K (CTAs per cluster) with the least expected time.  The terms are fits to timings of every split on the
-// 7B, 13B and 70B shapes, 2 to 4 bits (within 15 %, but for an odd number of CTAs per SM): a CTA costs about 4 us
+// 7B, 13B and 70B shapes, 2 to 4 bits (within 15 %): a CTA costs about 4 us
 // outside its runs (start, exchange) and 0.06 us per group of parameters, a run 0.38 us alone on its SM and 0.34 us per
 // SM where two CTAs share it (a quarter more with more than 16 token columns); behind the first two, a CTA's fixed part
 // is mostly hidden by its neighbour's runs, and clusters of eight leave SMs of a GPC empty.
@@ -606,6 +606,11 @@ SlimPlan slim_plan(const eqat_desc& d, int sms) {
       const double wide = nt == 1 ? 1.0 : 1.25, fixed = 4.0 + 0.06 * groups;
       double us = two ? fixed + n * most * (n == 1 ? 0.38 : 0.34) * wide + (n > 2 ? (n - 2) * 0.7 : 0.0)
                       : n * (fixed + most * 0.36 * wide);
+      // Two CTAs share an SM, so the last of an odd number runs by itself: a fixed part more where most SMs have it (three on
+      // 136 of 148 SMs, 13824 x 5120: estimated 15.5 without it, 19.8 with it, measured 21.5 us).  Where few have it the
+      // next launch fills in (12288 x 6144, 88 SMs: 17.7 us without, measured 19.5 us).
+      const int last = (tiles * split) % sms;
+      if (two && n > 2 && (n & 1) != 0 && 5 * last > 3 * sms) us += fixed * last / sms;
       if (split == 8 && n > 2) us *= 1.15;
       if (best.us == 0.0 || us < best.us) best = SlimPlan{nt, nd, token_tiles, split, groups, us};
     }
@@ -632,8 +637,8 @@ int launch_bits(const SlimPlan& pl, const SlimParams& p, const eqat_bf16* X, dim
 // Which kernel takes few tokens.  The matrix-vector kernel streams the weight with less start-up (5.1 against 6.8 us for
 // one token of 4096 x 4096, 2-bit codes) but pays for every token and holds at most eight; this one costs the same for
 // any number up to 16 (7.1 us against 10.0 us at 8 tokens, 19.8 us in two launches at 16).  Two estimates are compared,
-// so this one has to be a quarter better (13824 x 5120, 4-bit codes, 6 tokens: estimated 15.5 against 18.7 us, measured
-// 21.2 against 18.3 us).  Small weights keep the matrix-vector kernel for the sake of their bits (packed_gemv_keeps_bits).
+// so this one has to be a quarter better (11008 x 4096, 4-bit codes, 8 tokens: estimated 13.3 against 15.0 us, measured
+// 14.8 against 15.1 us).  Small weights keep the matrix-vector kernel for the sake of their bits (packed_gemv_keeps_bits).
 bool slim_fwd_applies(const eqat_desc& d, int sms, SlimPlan& pl) {
   if (d.tokens > kSlimMaxTokens) return false;
   const FewTokenPlan gemv = packed_gemv_plan(d);

@@ -57,6 +57,16 @@ def test_small_weights_take_one_kernel_up_to_sixteen_tokens(eqat):
     assert kernels(1024, 2048, 2, 32, range(1, 17)) == {eqat.EQAT_ROUTE_WEIGHT_ROWS}
 
 
+def test_an_odd_number_of_ctas_per_sm_is_not_taken_for_free(eqat):
+    """Three CTAs on nearly every SM, of which two run at a time: 13824 x 5120 at seven and eight tokens was estimated at 15.5
+    us, took 21.5, and the matrix-vector kernel 18.9 to 20.8 us."""
+    for bits in (3, 4):
+        for tokens in (7, 8):
+            assert route(eqat, 13824, 5120, tokens, bits, 128)[0] == eqat.EQAT_ROUTE_MATRIX_VECTOR
+    assert route(eqat, 13824, 5120, 16, 4, 128) == (eqat.EQAT_ROUTE_WEIGHT_ROWS, (1, 16, 2))
+    assert route(eqat, 12288, 6144, 8, 4, 128) == (eqat.EQAT_ROUTE_WEIGHT_ROWS, (1, 16, 4))   # on 88 of the 148 SMs only
+
+
 def test_plans_cover_all_tokens(eqat):
     rng = random.Random(3)
     for _ in range(3000):
