@@ -11,7 +11,7 @@ struct WidePlan {
   double us;                 // expected time; 0: the problem does not fit
 };
 // True when the kernel is the one to take for this packed forward, and how: on the current device (sms = 0), or on one of
-// `sms` SMs all of which make up clusters.
+// `sms` SMs that are grouped like a B200's.
 bool wide_fwd_applies(const eqat_desc& d, int sms, WidePlan& plan);
 // Y[T,out] = X[T,in] * dequant(Wq)^T
 int launch_wide_fwd(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16, const void* zq,

@@ -67,6 +67,12 @@ def test_an_odd_number_of_ctas_per_sm_is_not_taken_for_free(eqat):
     assert route(eqat, 12288, 6144, 8, 4, 128) == (eqat.EQAT_ROUTE_WEIGHT_ROWS, (1, 16, 4))   # on 88 of the 148 SMs only
 
 
+def test_large_batches_of_4_bit_codes_keep_the_tiled_kernel(eqat):
+    assert route(eqat, 8192, 28672, 2048, 4, 128)[0] == eqat.EQAT_ROUTE_TILED            # 705 to 850 against 825 to 920 us
+    assert route(eqat, 8192, 28672, 2300, 4, 128)[0] == eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS   # 1161 against 798 us
+    assert route(eqat, 4096, 4096, 333, 4, 128)[0] == eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS
+
+
 def test_plans_cover_all_tokens(eqat):
     rng = random.Random(3)
     for _ in range(3000):
