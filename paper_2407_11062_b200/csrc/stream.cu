@@ -86,7 +86,6 @@ __device__ __forceinline__ void stream_tiles(const CUtensorMap* const (&maps)[NI
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const size_t n_tiles = (n_elem + kTileElems - 1) / kTileElems;
 
-  ptx::grid_dependents_launch();
   if (threadIdx.x == 0) {
     for (int s = 0; s < R::kStages; ++s) {
       ptx::mbar_init(ptx::smem_addr(&ctl->full[s]), 1);
@@ -121,6 +120,16 @@ __device__ __forceinline__ void stream_tiles(const CUtensorMap* const (&maps)[NI
         ++issued;
         if (++stage == R::kStages) { stage = 0; phase ^= 1u; }
       }
+      // The next launch may start when this CTA is about to finish: its last tile (with two inputs) or the one before has been
+      // handed back.  Let in at once, its CTAs took the slots as they fell free, several of the low-numbered ones, which have
+      // a tile more, on one SM: the straight-through backward of 1024 x 8192 took 15.4 us, without overlap 14.8, now 14.2;
+      // of 512 x 2048 5.4, 4.9, 4.2 us; the fake quantiser of 1024 x 8192 8.9, 8.9, 8.6 us.
+      if (ok && issued > 1) {
+        const size_t last = issued - (NIN > 1 ? 1 : 2);
+        ok = bounded_wait(ptx::smem_addr(&ctl->empty[last % R::kStages]), (uint32_t)((last / R::kStages) & 1), abort_flag,
+                          WAIT_STREAM_EMPTY, 32);
+      }
+      ptx::grid_dependents_launch();
       if (!ok || *abort_flag) {
         // every copy this thread started must land before the CTA exits
         const size_t first = issued > (size_t)R::kStages ? issued - R::kStages : 0;
