@@ -66,7 +66,7 @@ namespace {
 // task go through a double-buffered shared array to a reducer warp, which adds
 // them in a fixed order and stores Y while the consumers are on the next task.
 constexpr int kTcMaxTokens = 8;                         // the instruction has eight token columns
-constexpr int kTcMaxTotalTokens = 64;                   // up to here, as several launches over slices of the tokens
+constexpr int kTcMaxTotalTokens = 64;                   // up to here a plan is made, for comparison (see packed_gemv_applies)
 constexpr int kTcWarps = 16;
 constexpr int kTcThreads = (kTcWarps + 2) * 32;        // + producer warp + reducer warp
 constexpr int kTcRows = 16;                            // weight rows per task
@@ -741,12 +741,7 @@ bool packed_gemv_keeps_bits(const eqat_desc& d) {
 }
 
 bool packed_gemv_applies(const eqat_desc& d) {
-  const FewTokenPlan plan = packed_gemv_plan(d);
-  if (plan.launches <= 1) return plan.launches == 1;
-  if (packed_gemv_keeps_bits(d)) return true;
-  // several launches only while clearly cheaper than the tiled kernel, which takes about 1 / 1.45 / 1.2 us per 64 input
-  // columns for any token count below a full row-tile, because the K loop of a tile is serial
-  return plan.us < 0.8 * (d.in_features / 64.0 * (d.bits == 2 ? 1.0 : (d.bits == 3 ? 1.45 : 1.2)));
+  return packed_gemv_plan(d).launches == 1 || packed_gemv_keeps_bits(d);
 }
 
 int launch_packed_gemv(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16,

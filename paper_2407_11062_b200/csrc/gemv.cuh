@@ -16,9 +16,9 @@ FewTokenPlan packed_gemv_plan(const eqat_desc& d);
 // True where every batch of up to sixteen tokens goes through this kernel, so that a token gives the same bits alone and in
 // any of them: weights of less than 3 MB of codes, rows of 1024 to 4096 columns, groups of at least 64.
 bool packed_gemv_keeps_bits(const eqat_desc& d);
-// True when the few-token kernel handles this problem: groups of at least 64 elements, at most 64 tokens, staged
-// activations of at least one token that fit in the shared memory of a CTA, and, where the tokens need several
-// launches, either the range above or a cost estimate below the tiled kernel's.
+// True when the few-token kernel handles this problem: groups of at least 64 elements and tokens whose staged activations
+// fit in the shared memory of a CTA, so that one launch takes them all, or the range above (two launches).  Where the tokens
+// need more launches the weight-row kernel is faster on every shape and fits wherever this one does.
 bool packed_gemv_applies(const eqat_desc& d);
 // Y[T,out] = X[T,in] * dequant(Wq)^T for a problem packed_gemv_applies() accepted
 int launch_packed_gemv(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16,
