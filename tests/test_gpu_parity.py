@@ -536,7 +536,8 @@ def check_e2e(r, group):
 def test_e2e_small(eqat, bits, group, real_z):
     """Every group size of the paper's ablation (32 .. 256) and one group per row (512 = in_features, the
     channel-wise setting of its Q-PEFT comparison), with frozen integer zero points and with trained fp16 ones.
-    600 tokens: a pair of CTAs per tile with a ragged last row-tile; 256: single CTAs."""
+    600 tokens: a pair of CTAs per tile with a ragged last row-tile; 256: single CTAs (dX and ds; the forward of both runs on
+    pairs of weight-row tiles, the tiled forward in test_packed_forward_of_large_batches)."""
     for tokens in (600, 256):
         cfg = small_cfg(f"e2e_{bits}_{group}", 512, 512, bits, group, tokens, "student_t4", 0.02, 0.01)
         check_e2e(run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z), group)
@@ -545,8 +546,8 @@ def test_e2e_small(eqat, bits, group, real_z):
 @pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("tokens", [1, 2, 3, 4, 5, 7, 8, 9])
 def test_e2e_few_tokens(eqat, bits, tokens):
-    """Decode-sized batches: up to eight tokens take a matrix-vector forward kernel, more the tiled one (rows this
-    short are not worth several launches).
+    """Decode-sized batches: up to eight tokens take a matrix-vector forward kernel, nine the kernel on weight-row tiles or
+    (rows of 1408) two launches.
     640 = 10 units of 64 columns, fewer than the sixteen warps of a CTA (some get none); 1408 = 22 (one or two each)."""
     group = 64 if bits == 2 else 128
     cfg = small_cfg(f"gemv_{bits}_{tokens}", 448, 640 if group == 64 else 1408, bits, group, tokens, "student_t4", 0.02, 0.01)
@@ -568,7 +569,8 @@ def test_e2e_few_tokens_with_trained_zero_points(eqat, bits, group, in_f, tokens
 
 
 def test_few_token_forward_agrees_with_tiled_forward(eqat):
-    """The same rows through both forward kernels (4 tokens alone, and as the first rows of a 9-token batch)."""
+    """The same rows alone (4 tokens, one launch) and as the first rows of a 9-token batch (two launches).  The kernels are
+    compared with each other in test_packed_forward_kernels_agree."""
     cfg = small_cfg("gemv_vs_gemm", 512, 1024, 2, 64, 9)
     r5 = run_e2e(eqat, cfg, cfg.linears[0], 9)
     cfg4 = small_cfg("gemv_vs_gemm", 512, 1024, 2, 64, 4)
@@ -772,7 +774,8 @@ def test_few_token_forward_takes_any_zero_point_byte(eqat, bits, group, in_f, to
     (1024, 4096, 256, 2, 256, False), # one full token tile, eight CTAs per cluster
     (1088, 8192, 257, 4, 8192, False),   # one group per row, one token more than a tile
     (4096, 1024, 700, 3, 64, True),   # several token tiles, more clusters than fit at a time
-    (11008, 512, 333, 2, 64, False),  # four runs: every group of row threads gets one
+    (4096, 512, 333, 2, 64, False),   # four runs: every group of row threads gets one, or none over a split of K
+    (11008, 512, 333, 2, 64, False),  # more weight rows: the tiled kernel is ahead
 ])
 def test_packed_forward_for_prompts(eqat, out, in_f, tokens, bits, group, real_z):
     """The kernel on pairs of weight-row tiles, against the oracle and against itself."""
@@ -782,6 +785,50 @@ def test_packed_forward_for_prompts(eqat, out, in_f, tokens, bits, group, real_z
     again = run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z)
     assert torch.equal(r["Y"].view(torch.int16), again["Y"].view(torch.int16))
     assert eqat.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("out,in_f,tokens,bits,group,real_z", [
+    (512, 512, 4100, 4, 32, False),      # 4-bit codes, two groups per 64-code unit, a last row tile of four tokens
+    (448, 1408, 4100, 4, 128, True),     # fp16 zero points, a ragged column tile
+    (512, 512, 4100, 4, 256, False),
+    (448, 1408, 4097, 4, 1408, False),   # one group per row, in_features not a power of two; one token past a tile
+    (320, 640, 4100, 3, 64, True),
+    (448, 1408, 4100, 3, 1408, False),
+    (512, 768, 4100, 2, 32, True),       # 2-bit codes: runs of two K blocks
+    (192, 512, 4352, 2, 256, False),     # half a row tile of a pair: the second CTA has no tokens
+    (25600, 512, 128, 4, 32, False),     # many weight rows, few tokens: one CTA per tile
+    (25600, 384, 200, 3, 128, True),
+    (25600, 512, 256, 2, 64, False),
+])
+def test_packed_forward_of_large_batches(eqat, out, in_f, tokens, bits, group, real_z):
+    """The tiled kernel: the forms that the smaller cases do not reach."""
+    cfg = small_cfg(f"tiled_{out}_{in_f}_{tokens}", out, in_f, bits, group, tokens, "student_t4", 0.02, 0.01)
+    zfmt = eqat.EQAT_ZP_FP16 if real_z else eqat.EQAT_ZP_U8
+    assert eqat.eqat_packed_fwd_route(eqat.make_desc(bits, group, out, in_f, tokens, 0, zfmt))[0] == eqat.EQAT_ROUTE_TILED
+    check_e2e(run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z), group)
+    assert eqat.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("bits,group", [(2, 64), (3, 128), (4, 64)])
+def test_packed_forward_kernels_agree(eqat, bits, group):
+    """The same eight tokens through all four kernels, alone and as the first of larger batches."""
+    out, in_f = 512, 1024
+    P, z8, s16, X = few_token_problem(out, in_f, 4100, 31, bits, group)
+    q = O.unpack_rows(P.cpu().numpy(), bits, in_f)
+    What_o = O.dequantize(q, s16.cpu().numpy().astype(np.float32), z8.cpu().numpy(), group)
+    want = O.linear_fwd(torch_to_f64(X[:8]), What_o)
+    first = []
+    for tokens, kernel in ((8, eqat.EQAT_ROUTE_MATRIX_VECTOR), (24, eqat.EQAT_ROUTE_WEIGHT_ROWS),
+                           (200, eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS), (4100, eqat.EQAT_ROUTE_TILED)):
+        d = eqat.make_desc(bits, group, out, in_f, tokens)
+        assert eqat.eqat_packed_fwd_route(d)[0] == kernel
+        Y = torch.full((tokens, out), float("nan"), dtype=torch.bfloat16, device="cuda")
+        eqat.qlinear_packed_fwd(d, X[:tokens].contiguous(), P, s16, z8, Y)
+        first.append(torch_to_f64(Y[:8]))
+        assert rel_err(first[-1], want) <= TOL
+    # the two kernels for few tokens round nothing but Y, the other two W_hat and Y in the same places
+    for a, b in ((0, 1), (2, 3)):
+        assert rel_err(first[a], first[b]) <= 1e-3
 
 
 @pytest.mark.parametrize("which", [3, 4])
@@ -798,31 +845,31 @@ def test_weight_row_kernels_wait_runs_out_cleanly(eqat, which):
     (1024, 256, 520, 2, 64),
     (64, 11008, 4, 2, 64),          # few-token kernel with more than 48 KB of staged activations
     (64, 28672, 2, 4, 128),         # the longest rows of the 70B block, 4-bit codes: two tokens fit one launch
-    (64, 28672, 3, 3, 128),         # 3-bit codes, the longest rows: slices of two tokens and one
+    (64, 28672, 3, 3, 128),         # 3-bit codes, the longest rows: the kernel on weight-row tiles
     (448, 1408, 700, 3, 32),        # groups of 32, nothing a multiple of a tile
     (320, 1408, 1100, 2, 1408),     # one group per row with in_features not a power of two: 5.5 column tiles
     (192, 640, 3, 4, 640),          # one group per row through the few-token kernel
-    (192, 640, 3, 2, 32),           # groups of 32 with few tokens: the tiled kernel
+    (192, 640, 3, 2, 32),           # groups of 32 with few tokens: the kernel on weight-row tiles
     (128, 1152, 3, 2, 1152),        # 2-bit codes, one group per row, few tokens: the tensor-core matrix-vector kernel
     (192, 768, 2, 2, 128),          # the same kernel with groups of 128 (two 64-column chunks per group) ...
     (80 * 16, 4608, 1, 2, 256),     # ... and of 256; 80 row-blocks of 16 over several stages of the ring, 9 boxes per row
     (64, 128, 1, 2, 64),            # rows of 32 bytes: a quarter of the copy engine's 128-byte box
     (64, 256, 8, 2, 128),           # eight tokens, the most the matrix-vector kernel takes
     (2432, 512, 4, 2, 64),          # more row-blocks than SMs: every CTA takes a second task, parameters loaded as vectors
-    (64, 11008, 8, 2, 64),          # eight tokens whose staged activations do not fit: two launches of four
-    (128, 4096, 13, 2, 64),         # more than eight tokens: slices of seven and six
-    (128, 8192, 31, 2, 128),        # five slices (7, 7, 7, 7, 3)
-    (64, 28672, 4, 2, 64),          # the longest rows of the 70B block: two tokens per launch
-    (64, 11008, 8, 4, 128),         # 4-bit codes: 43 boxes of 256 columns per row, two launches of four tokens
+    (64, 11008, 8, 2, 64),          # eight tokens whose staged activations do not fit: the kernel on weight-row tiles
+    (128, 4096, 13, 2, 64),         # more than eight tokens, small weight: slices of seven and six
+    (128, 8192, 31, 2, 128),        # thirty-one tokens: 32 columns of a weight-row tile
+    (64, 28672, 4, 2, 64),          # the longest rows of the 70B block: more tokens than staged activations fit
+    (64, 11008, 8, 4, 128),         # 4-bit codes: 86 runs of 128 codes per row
     (128, 4096, 13, 4, 64),         # 4-bit codes, groups of 64 (one group per chunk), slices of seven and six
     (80 * 16, 2304, 5, 4, 256),     # 4-bit codes, groups of 256, nine boxes per row, 80 row-blocks
     (64, 128, 2, 4, 64),            # rows of 64 bytes: half a box, two chunks, two groups
     (128, 4096, 13, 3, 128),        # 3-bit codes: boxes of 96 bytes (256 columns), slices of seven and six
     (80 * 16, 2304, 5, 3, 256),     # 3-bit codes, groups of 256, nine boxes per row, 80 row-blocks
-    (64, 11008, 8, 3, 64),          # 3-bit codes, groups of 64, 43 boxes per row, two launches of four tokens
+    (64, 11008, 8, 3, 64),          # 3-bit codes, groups of 64, 86 runs per row
     (64, 128, 1, 3, 128),           # 3-bit rows of 48 bytes: half a box, one group
-    (128, 11008, 40, 2, 64),        # forty tokens over long rows: eight launches of five
-    (128, 11008, 64, 4, 128),       # the most tokens that go out in slices: thirteen launches (twelve of five, one of four)
+    (128, 11008, 40, 2, 64),        # forty tokens over long rows
+    (128, 11008, 64, 4, 128),       # the most tokens of the kernel on weight-row tiles
 ])
 def test_e2e_ragged(eqat, out, in_f, tokens, bits, group):
     cfg = small_cfg(f"e2er_{out}_{in_f}_{tokens}", out, in_f, bits, group, tokens)
@@ -881,7 +928,7 @@ def test_handoff_side_outputs_against_hand_values(eqat, kind, bits):
 def test_packed_weight_aligned_to_16_bytes_only(eqat, bits, tokens):
     """The packed matrix (and its step sizes and zero points) 16 bytes past a 256-byte boundary: 16-byte alignment is
     all the interface asks for, so the kernels must not fetch whole 32-byte sectors from it.  Same bits as the
-    aligned run, through the matrix-vector kernel (1 and 4 tokens) and the tiled one."""
+    aligned run, through the matrix-vector kernel (1 and 4 tokens) and the one on pairs of weight-row tiles."""
     group = 64 if bits == 2 else 128
     cfg = small_cfg(f"wq16_{bits}", 320, 512, bits, group, tokens, "student_t4", 0.02, 0.01)
     lin = cfg.linears[0]

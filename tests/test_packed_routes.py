@@ -90,3 +90,29 @@ def test_the_query_checks_its_descriptor(eqat):
         eqat.eqat_packed_fwd_route(eqat.make_desc(2, 64, 96, 512, 4), SMS)
     with pytest.raises(eqat.EqatError):
         eqat.eqat_packed_fwd_route(eqat.make_desc(2, 64, 512, 512, 4), -1)
+
+
+def test_the_gpu_tests_reach_the_kernels_they_name(eqat):
+    """The sizes of the GPU tests, by the kernel that each test is about."""
+    import test_gpu_parity as gpu
+
+    def sizes(test):
+        return next(m.args[1] for m in test.pytestmark if m.name == "parametrize")
+
+    for out, in_f, tokens, bits, group, real_z in sizes(gpu.test_packed_forward_on_weight_row_tiles):
+        assert route(eqat, out, in_f, tokens, bits, group, real_z)[0] == eqat.EQAT_ROUTE_WEIGHT_ROWS, (out, in_f, tokens)
+    for out, in_f, tokens, bits, group, real_z in sizes(gpu.test_packed_forward_for_prompts):
+        kernel = eqat.EQAT_ROUTE_TILED if out == 11008 else eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS
+        assert route(eqat, out, in_f, tokens, bits, group, real_z)[0] == kernel, (out, in_f, tokens)
+    for out, in_f, tokens, bits, group, real_z in sizes(gpu.test_packed_forward_of_large_batches):
+        assert route(eqat, out, in_f, tokens, bits, group, real_z)[0] == eqat.EQAT_ROUTE_TILED, (out, in_f, tokens)
+    for bits, group, in_f in next(m.args[1] for m in gpu.test_few_token_forward_takes_any_zero_point_byte.pytestmark
+                                  if m.args[0].startswith("bits")):
+        for tokens in (1, 2, 8):
+            assert route(eqat, 320, in_f, tokens, bits, group)[0] == eqat.EQAT_ROUTE_MATRIX_VECTOR
+    for bits, group, in_f, tokens in sizes(gpu.test_e2e_few_tokens_with_trained_zero_points):
+        assert route(eqat, 320, in_f, tokens, bits, group, True)[0] == eqat.EQAT_ROUTE_MATRIX_VECTOR
+    for bits, group in sizes(gpu.test_few_token_forward_does_not_depend_on_the_slicing):
+        assert route(eqat, 1280, 4096, 13, bits, group) == (eqat.EQAT_ROUTE_MATRIX_VECTOR, (2, 7, 1))
+    for out, in_f, bits, group in sizes(gpu.test_small_weights_give_a_token_the_same_bits_in_any_batch_of_up_to_sixteen):
+        assert route(eqat, out, in_f, 16, bits, group) == (eqat.EQAT_ROUTE_MATRIX_VECTOR, (2, 8, 1))
