@@ -7,13 +7,14 @@ One step = one pass of the whole path over the seven linear layers of a
 Llama-2-7B decoder block at 2 bits, group 64:
     min/max init, Block-AP forward and backward at 4096 tokens (batch 2 x 2048),
     hand-off (quantise + pack, unpack), E2E-QP forward / dX / ds at 16384 tokens.
-Prints one JSON line (rank 0).  `value` is the tensor-core throughput of the six
+Prints one JSON line of at most 2 KB on standard output (rank 0), and everything measured as one JSON object on standard
+error or, with `--detail FILE`, into that file.  `value` is the tensor-core throughput of the six
 contractions per linear (2*T*in*out flop each) over the whole step, all kernels
 included in the time; dequantisation, STE and epilogue arithmetic are not counted
 as flops.
 
-On one GPU the same run then times, outside the headline's timed region and reported under their own keys:
-the other workloads (7B w4g128 Block-AP, 13B w3g128 E2E-QP, 70B w2g64 both modes) under "configs", and the five
+On one GPU the same run then times, outside the headline's timed region and reported in the full object under their own
+keys: the other workloads (7B w4g128 Block-AP, 13B w3g128 E2E-QP, 70B w2g64 both modes) under "configs", and the five
 streaming kernels on cold data, back to back over buffer sets several times the L2, under "streaming" (once before
 the GEMM phases of the run and again after them, with the GPU's clocks read beside each).
 `--gpus N` started without a launcher spawns the N ranks itself.
@@ -743,6 +744,39 @@ def run_streaming_leg(eqat, device, peaks, bits, group, shape=(11008, 4096), min
 
 
 # ----------------------------------------------------------------------------- main
+def short(v, digits=6):
+    """The same value with its floats rounded to a few significant digits."""
+    if isinstance(v, float):
+        return float(f"{v:.{digits}g}")
+    if isinstance(v, dict):
+        return {k: short(x, digits) for k, x in v.items()}
+    return [short(x, digits) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def headline(out):
+    """The part of a result that goes to standard output: small enough to survive a truncated log."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+            "dtype", "data", "config", "pct_of_bf16_peak", "tflops_by_mode", "clocks", "e2e", "gpu_launches")
+    line = {k: out[k] for k in keys if k in out}
+    if out.get("roofline"):
+        line["roofline"] = {k: out["roofline"].get(k) for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "peak_source",
+                                                                "traffic")}
+    if "kernel_classes" in out:
+        line["frac_of_peak"] = {k: short(c["roofline"]["frac"], 3) for k, c in out["kernel_classes"].items() if "roofline" in c}
+    if "cpu_baseline" in out:
+        line["cpu_baseline"] = {k: out["cpu_baseline"].get(k) for k in ("value", "unit", "kind", "cores")}
+    return short(line)
+
+
+def report(out, detail_path):
+    if detail_path:
+        with open(detail_path, "w") as f:
+            json.dump(out, f)
+    else:
+        print(json.dumps(out), file=sys.stderr, flush=True)
+    print(json.dumps(headline(out)), flush=True)
+
+
 def spawn_ranks(args):
     """`--gpus N` without a launcher: start N copies of this script, one per GPU, with the environment
     torch.distributed's launcher would have given them; rank 0's line is the job's line."""
@@ -873,7 +907,7 @@ def run_ours(args):
                                                     "GEMM phases of this run), not part of the step"}
         if world == 1 and not args.no_cpu_baseline:
             out["cpu_baseline"] = cpu_baseline()
-        print(json.dumps(out), flush=True)
+        report(out, args.detail)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
@@ -924,7 +958,7 @@ def decode_leg(eqat, dev, peaks, iters, model="7b", bits=BITS, group=GROUP, only
     out = {"metric": "packed forward, few tokens", "unit": "us per call", "bits": bits, "group": group,
            "zero_points": "fp16" if fp16_zero_points else "uint8", "model": model, "hbm_gbs_peak": peaks["hbm_gbs"],
            "method": "CUDA graph of one call per weight copy (copies total > 2 x L2), replayed back to back; a call "
-                     "is one kernel launch for up to 8 tokens where the staged activations fit, else one per token slice",
+                     "is one kernel launch (on small weights with rows of 1024 to 4096 columns two, from 9 to 16 tokens)",
            "cases": {}}
     for lin in LINEARS[model]:
         if only_shape is not None and lin.name != only_shape:
@@ -988,6 +1022,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--detail", default=None, metavar="FILE", help="write everything measured there instead of to standard error")
     ap.add_argument("--headline-only", action="store_true", help="skip the other workloads and the streaming leg")
     args = ap.parse_args()
     if args.kernel_case:

@@ -122,3 +122,36 @@ def test_extra_configs_match_the_workload_table():
         assert {spec["t_ap"], spec["t_e2e"]} - {0} == {c.tokens}
         assert (spec["t_ap"] > 0) == ("block_ap" in c.modes) and (spec["t_e2e"] > 0) == ("e2e_qp" in c.modes)
         assert spec["w"] == (c.weight_dist, c.weight_scale, c.outlier_frac)
+
+
+def test_the_line_on_standard_output_is_short(tmp_path, capsys):
+    """The result's line holds the contract's keys in at most 2 KB, whatever else was measured; the rest goes elsewhere."""
+    third = 1.0 / 3.0
+    roof = dict(bench.tensor_roofline(1000.0 * third, bench.load_peaks(), 0.4, 1500.0), kernel="gemm_kernel (packed_bwd_dx)",
+                traffic=1e9 * third, traffic_unit="x" * 200, algorithmic_bytes=1e9 * third)
+    out = {"metric": "QLinear fwd+bwd TFLOP/s", "value": 1e3 * third, "unit": "TFLOP/s", "n_gpus": 8, "steps": 20, "warmup": 5,
+           "ms_per_step": 20 * third, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16",
+           "data": "synthetic", "config": {"workload": bench.WORKLOAD, "bits": 2, "group": 64, "tokens_block_ap": 4096,
+                                           "tokens_e2e_qp": 16384, "l2": "inputs larger than L2 (working set > 2 GB per shape, weights per linear)"},
+           "pct_of_bf16_peak": {k: 200 * third for k in ("vs_burst", "vs_sustained", "vs_nominal_dense")},
+           "tflops_by_mode": {"block_ap": 1e3 * third, "e2e_qp": 1e3 * third}, "roofline": roof,
+           "kernel_classes": {name: {"roofline": dict(roof), "ms": third} for name in
+                              ("minmax_init", "fakequant_weight", "fakequant_fwd", "fakequant_bwd", "quantize_pack", "unpack", "packed_fwd",
+                               "packed_bwd_dx", "packed_bwd_ds", "ste_bwd", "minmax_init_cold", "quantize_pack_cold", "unpack_cold")},
+           "clocks": {"sm_mhz": 1300.0 + third, "sm_max_mhz": 1965.0, "power_w_max": 1000 * third, "samples": 145,
+                      "reasons": ["hw_slowdown", "hw_thermal_slowdown", "sw_power_cap", "sw_thermal_slowdown"]},
+           "e2e": {"value": 1e3 * third, "unit": "TFLOP/s", "ms_per_step": third, "steps": 20, "h2d_bytes_per_step": 10 ** 10,
+                   "d2h_bytes_per_step": 10 ** 10}, "gpu_launches": 2940, "configs": {"x" * 50: "y" * 20000}, "streaming": ["z" * 9000],
+           "cpu_baseline": {"value": 0.03 * third, "unit": "TFLOP/s", "kind": "oracle", "cores": 224, "sample": "s" * 500}}
+    bench.report(out, str(tmp_path / "detail.json"))
+    lines = capsys.readouterr().out.strip().splitlines()
+    assert len(lines) == 1 and len(lines[0]) <= 2048
+    line = json.loads(lines[0])
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+                "dtype", "data", "config", "clocks", "e2e", "gpu_launches", "roofline"):
+        assert key in line, key
+    assert line["value"] == pytest.approx(out["value"], rel=1e-5) and line["roofline"]["traffic"] is not None
+    assert json.load(open(tmp_path / "detail.json")) == out
+    bench.report(out, None)
+    both = capsys.readouterr()
+    assert both.out.strip() == lines[0] and json.loads(both.err) == out
