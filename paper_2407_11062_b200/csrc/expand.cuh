@@ -48,7 +48,7 @@ inline void set_weight(PackedWeight& p, const eqat_desc& d, const uint8_t* Wq, c
 // constants are exact in fp32 (s is an fp16 value, 11 significant bits) and so is the result: the only rounding
 // is the final one to bf16.  With a real-valued (fp16) zero point the constant (128 + z)*s is rounded to fp32
 // first, an error of at most 2^-17 s.  4-bit codes reach byte positions with one shift+mask per 4 codes and one
-// byte permute each; 3-bit codes are shifted individually.
+// byte permute each; 3-bit codes sit at other positions (below).
 // 2-bit codes: the four possible values of a group are built once as bf16 ((q - z)*s in fp32, rounded once) and
 // each code is looked up with a byte permute: lut01 = (v0, v1), lut23 = (v2, v3); value q occupies bytes 2q, 2q+1
 // of the 8-byte pair, so the selector byte of a code is 0x10 + 0x22*q.

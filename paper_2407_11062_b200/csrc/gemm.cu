@@ -128,12 +128,6 @@ struct Control {
 };
 static_assert(sizeof(Control) <= 512, "control block must fit its reservation");
 
-// Shared-memory matrix descriptor, 128-byte swizzle, 8-row atoms 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) |
-         (1ull << 46) | (2ull << 61);
-}
-
 template <bool ROW_ORDER, int BAND>
 __device__ __forceinline__ void tile_coords(int tile, int num_m, int num_n, int& m_blk, int& n_blk) {
   if (ROW_ORDER) {
@@ -586,10 +580,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
             const uint32_t b_addr = smem_base + C::b_offset(PACKED ? stage_b : stage);
 #pragma unroll
             for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-              const uint64_t b_desc = smem_desc(b_addr + kk * b_step, b_lbo);
+              const uint64_t b_desc = ptx::smem_desc(b_addr + kk * b_step, b_lbo);
 #pragma unroll
               for (int h = 0; h < MT; ++h) {
-                const uint64_t a_desc = smem_desc(a_addr + h * a_half + kk * a_step, a_lbo);
+                const uint64_t a_desc = ptx::smem_desc(a_addr + h * a_half + kk * a_step, a_lbo);
                 if (PAIR) ptx::mma_bf16_ss_pair(d_tmem + h * BN, a_desc, b_desc, idesc, (kb | kk) != 0 ? 1u : 0u);
                 else ptx::mma_bf16_ss(d_tmem + h * BN, a_desc, b_desc, idesc, (kb | kk) != 0 ? 1u : 0u);
               }

@@ -172,6 +172,12 @@ __device__ __forceinline__ bool elect_one() {
   return ok != 0;
 }
 
+// Shared-memory matrix descriptor, 128-byte swizzle, 8-row atoms 1024 bytes apart (K-major operands: lbo 16).
+__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes = 16) {
+  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) |
+         (1ull << 46) | (2ull << 61);
+}
+
 // ---- MMA: D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate, one CTA.
 __device__ __forceinline__ void mma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                             uint32_t accumulate) {

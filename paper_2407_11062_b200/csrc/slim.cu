@@ -109,11 +109,6 @@ struct Slim {
   }
 };
 
-// Shared-memory matrix descriptor, K-major, 128-byte swizzle, 8-row atoms 1024 bytes apart.
-__device__ __forceinline__ uint64_t k_major_desc(uint32_t addr) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-
 __device__ __forceinline__ uint32_t add_bf16x2(uint32_t a, uint32_t b) {
   const __nv_bfloat162 r = __hadd2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
   return *reinterpret_cast<const uint32_t*>(&r);
@@ -308,7 +303,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
       if (ptx::elect_one() && got) {
         const uint32_t a = tmem + (uint32_t)(g * 64);
         const uint32_t d = tmem + (uint32_t)(C::kTmemA + g * ND * C::kTn);
-        const uint64_t b = k_major_desc(ring_addr + st * C::kStage + C::kCodes + in_box * 2 * C::kBlock);
+        const uint64_t b = ptx::smem_desc(ring_addr + st * C::kStage + C::kCodes + in_box * 2 * C::kBlock);
         constexpr int kPer = 8 / ND;                       // instructions (16 columns each) per accumulator
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
@@ -316,7 +311,7 @@ slim_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
           const uint64_t bk = b + (uint64_t)((kk >> 2) * (C::kBlock >> 4) + (kk & 3) * 2);
           ptx::mma_bf16_ts(d + (uint32_t)((kk / kPer) * C::kTn), a + kk * 8, bk, idesc, acc);
           if (zf)                                          // rows of ones: the sums of the activations, in every lane
-            ptx::mma_bf16_ss(d + (uint32_t)(C::kTmemD + (kk / kPer) * C::kTn), k_major_desc(ring_addr + ones_off), bk, idesc, acc);
+            ptx::mma_bf16_ss(d + (uint32_t)(C::kTmemD + (kk / kPer) * C::kTn), ptx::smem_desc(ring_addr + ones_off), bk, idesc, acc);
         }
         ptx::mma_commit(ptx::smem_addr(&ctl->d_ready[g]));
         if (in_box == kBoxRuns - 1) ptx::mma_commit(ptx::smem_addr(&ctl->empty[st]));

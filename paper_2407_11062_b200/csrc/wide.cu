@@ -53,11 +53,6 @@ struct WideCtl {
 __host__ __device__ constexpr int code_bytes(int bits) { return 16 * bits; }             // of a row per run
 __host__ __device__ inline int stage_bytes(int bits, int tn) { return kRows * code_bytes(bits) + tn * 128; }
 
-// Shared-memory matrix descriptor, K-major, 128-byte swizzle, 8-row atoms 1024 bytes apart.
-__device__ __forceinline__ uint64_t k_major_desc(uint32_t addr) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-
 // The 128 codes of box row `row`: rows of 32, 48 or 64 bytes; 16-byte piece c of row r sits at piece c ^ ((r >> 2) & 1)
 // of 32-byte rows, c ^ ((r >> 1) & 3) of 64-byte rows (the copy engine's swizzles); 48-byte rows need none.
 template <int BITS>
@@ -155,7 +150,7 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         ptx::tc_fence_after();
         if (ptx::elect_one() && got) {
           const uint32_t a = tmem + (uint32_t)(g * 64);
-          const uint64_t b = k_major_desc(ring_addr + st * stage_size);
+          const uint64_t b = ptx::smem_desc(ring_addr + st * stage_size);
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)                   // a K block's activations of this CTA: tn/2 rows of 128 bytes
             ptx::mma_bf16_ts_pair(tmem + kTmemA, a + kk * 8, b + (uint64_t)((kk >> 2) * (p.tn * 4) + (kk & 3) * 2), idesc,
