@@ -62,11 +62,11 @@ EXTRA_CONFIGS = {
 # under profiles/ give the command).  They describe the kernels whose sources hash to `sources_sha256`; once those
 # files change (comments and white space aside) the figures are stale and `roofline.traffic` is reported as null.
 NCU_TRAFFIC = {
-    "sources": ("gemm.cu", "expand.cuh", "ptx.cuh"),
-    "sources_sha256": "1f52250845d827a08b2c43516139e086747f08fee7a4ee3cebf1b839ea29aa33",
-    "packed_fwd": {"qkvo": 140.6e6 + 95.5e6, "gate_up": 163.1e6 + 314.4e6, "down": 503.7e6 + 116.0e6},
-    "packed_bwd_dx": {"qkvo": 139.6e6 + 95.7e6, "gate_up": 514.9e6 + 115.9e6, "down": 153.6e6 + 315.4e6},
-    "packed_bwd_ds": {"qkvo": 416.3e6 + 1.0e6, "gate_up": 1306.5e6 + 3.1e6, "down": 1073.3e6 + 2.9e6},
+    "sources": ("gemm.cu", "expand.cuh", "ptx.cuh", "wait.cuh"),
+    "sources_sha256": "ae0001cdddf7bbcb4fbea7a781313a8fd209ecd2f592748daa1ee4b6737c95a7",
+    "packed_fwd": {"qkvo": 140.6e6 + 98.8e6, "gate_up": 165.2e6 + 317.2e6, "down": 502.7e6 + 120.6e6},
+    "packed_bwd_dx": {"qkvo": 139.6e6 + 95.9e6, "gate_up": 513.8e6 + 115.8e6, "down": 153.4e6 + 316.7e6},
+    "packed_bwd_ds": {"qkvo": 416.4e6 + 1.0e6, "gate_up": 1325.1e6 + 2.8e6, "down": 1079.5e6 + 3.2e6},
 }
 
 

@@ -4,8 +4,8 @@
 // 512-row tensor-memory tiles of gemm.cu would be almost empty here; the work is
 // one pass over the packed weight, so the kernel is a stream over its bytes that
 // builds weight fragments for warp-level matrix instructions in registers.  It
-// takes up to eight tokens per launch (more tokens, or rows too long for the
-// staged activations, go out as several launches).  The dequantised weight is
+// takes up to eight tokens per launch (small weights take up to sixteen tokens
+// in two launches, see packed_gemv_keeps_bits).  The dequantised weight is
 // never rounded to bf16 here: the codes enter the matrix instructions as exact
 // small numbers and the step size scales fp32 accumulators.
 #include <cuda.h>

@@ -924,11 +924,11 @@ def test_handoff_side_outputs_against_hand_values(eqat, kind, bits):
 
 
 @pytest.mark.parametrize("bits", [2, 3, 4])
-@pytest.mark.parametrize("tokens", [1, 4, 300])
+@pytest.mark.parametrize("tokens", [1, 4, 20, 300])
 def test_packed_weight_aligned_to_16_bytes_only(eqat, bits, tokens):
     """The packed matrix (and its step sizes and zero points) 16 bytes past a 256-byte boundary: 16-byte alignment is
     all the interface asks for, so the kernels must not fetch whole 32-byte sectors from it.  Same bits as the
-    aligned run, through the matrix-vector kernel (1 and 4 tokens) and the one on pairs of weight-row tiles."""
+    aligned run, through the matrix-vector kernel (1 and 4 tokens), the one on weight-row tiles and the one on pairs of them."""
     group = 64 if bits == 2 else 128
     cfg = small_cfg(f"wq16_{bits}", 320, 512, bits, group, tokens, "student_t4", 0.02, 0.01)
     lin = cfg.linears[0]
