@@ -61,7 +61,7 @@ namespace eqat {
 namespace {
 
 constexpr int BM = 128;          // rows per CTA and MMA = TMEM lanes
-constexpr int BN = 256;          // columns per tile
+constexpr int kBN = 256;         // columns per tile (128 or 64 where a problem is too small to fill the chip)
 constexpr int BK = 64;           // K per stage: one 128-byte swizzle span of bf16
 constexpr int UMMA_K = 16;       // K per tcgen05.mma for 16-bit inputs
 constexpr int kEpiWarps = 4;       // dense kernels: warps 2-5 are the epilogue
@@ -85,7 +85,7 @@ struct GemmParams : PackedWeight {
   int dz_literal;            // Eq. 4 clamped branch: -1 instead of -s
 };
 
-template <int MT, bool PACKED, bool PAIR>
+template <int MT, bool PACKED, bool PAIR, int BN>
 struct Cfg {
   static constexpr int kCtas = PAIR ? 2 : 1;
   static constexpr int kTileM = MT * BM;                 // output rows per CTA
@@ -109,7 +109,8 @@ struct Cfg {
   static constexpr int kThreads = (2 + (PACKED ? kDeqWarps : kEpiWarps)) * 32;
   static constexpr int kTmemCols = kAccSets * MT * BN;
   static constexpr int kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 512 /*barriers*/;
-  static_assert(!PACKED || MT == 2, "packed kernels use 256 rows per CTA");
+  static_assert(!PACKED || MT == 2 || BN == 128, "packed kernels use 256 rows per CTA, or tiles of 128 x 128");
+  static_assert(!PAIR || BN == kBN, "pairs share tiles of 256 columns");
   static_assert(kStages <= 8 && kStagesB <= 8, "barrier arrays hold eight stages");
   static_assert(kSmemBytes <= 232448, "stage rings exceed the shared memory of one CTA");
 };
@@ -172,11 +173,11 @@ __device__ __forceinline__ void quad_transpose(uint32_t (&o)[16], int lane) {
 // codes (BITS = 2, 3, 4), or (BITS = 16, Block-AP) fetched by TMA as the latent bf16 weight and fake-quantised in
 // place, Eq. 1 then Eq. 2, before the tensor core reads it.  PAIR: the tile is computed by two CTAs sharing one
 // MMA.  BITS is used by PACKED and by EPI_DS.
-template <int MT, bool A_MN, bool B_MN, bool PACKED, int EPI, int BITS, bool PAIR>
-__global__ void __launch_bounds__(Cfg<MT, PACKED, PAIR>::kThreads, 1)
+template <int MT, bool A_MN, bool B_MN, bool PACKED, int EPI, int BITS, bool PAIR, int BN>
+__global__ void __launch_bounds__(Cfg<MT, PACKED, PAIR, BN>::kThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
             const GemmParams p) {
-  using C = Cfg<MT, PACKED, PAIR>;
+  using C = Cfg<MT, PACKED, PAIR, BN>;
   constexpr bool LATENT = PACKED && BITS == 16;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = ptx::smem_addr(smem_raw);
@@ -914,10 +915,11 @@ bool make_tmap(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t outer
   return make_tmap_bf16(tm, base, inner, outer, box_outer);
 }
 
-// How a contraction's tiles are shaped: rows per CTA (128 * mt) and whether pairs of CTAs share a tile.
+// How a contraction's tiles are shaped: rows per CTA (128 * mt), whether pairs of CTAs share a tile, and its columns.
 struct TileShape {
   int mt;
   bool pair;
+  int bn;
   int rows() const { return 128 * mt * (pair ? 2 : 1); }
 };
 
@@ -934,10 +936,10 @@ bool operand_tmap(CUtensorMap* tm, const Operand& op, int rows_per_cta) {
   return op.mn_major ? make_tmap(tm, op.base, op.rows, op.k, BK) : make_tmap(tm, op.base, op.k, op.rows, rows_per_cta);
 }
 
-template <int MT, bool A_MN, bool B_MN, bool PACKED, int EPI, int BITS, bool PAIR>
+template <int MT, bool A_MN, bool B_MN, bool PACKED, int EPI, int BITS, bool PAIR, int BN = kBN>
 int launch(const Operand& a, const Operand& b, const GemmParams& p, cudaStream_t st) {
-  using C = Cfg<MT, PACKED, PAIR>;
-  auto kern = gemm_kernel<MT, A_MN, B_MN, PACKED, EPI, BITS, PAIR>;
+  using C = Cfg<MT, PACKED, PAIR, BN>;
+  auto kern = gemm_kernel<MT, A_MN, B_MN, PACKED, EPI, BITS, PAIR, BN>;
   static SmemOptIn opt_in;
   if (!opt_in.ensure(kern, C::kSmemBytes)) return EQAT_ERR_CUDA;
   CUtensorMap ta, tb;
@@ -969,23 +971,37 @@ int launch(const Operand& a, const Operand& b, const GemmParams& p, cudaStream_t
   return launch_status();
 }
 
+// The narrowest tile of 128 rows whose tiles still fit the chip at once, at least `least` columns (a quantisation group that
+// the epilogue sums up lies in one tile); 256 when none does.  A small problem is a chain of latencies: the fill of the ring,
+// a K loop that waits for L2, an epilogue of BN / 32 steps per warp.  A K block takes a CTA about as long with 64 columns
+// (24 KB to fetch) as with 256 of a pair (32 KB), so more and smaller tiles shorten the chain as long as every SM has one.
+// 512 x 512, 256 tokens: Block-AP forward 9.0 -> 6.5 us, backward 20.1 -> 10.6 us, E2E-QP 23.7 -> 15.6 us; packed dX of
+// 2048 x 2048, 200 tokens 29.4 -> 16.4 us.
+int narrow_columns(int M, int N, int least) {
+  const long sms = sm_count(), rows = (M + 127) / 128;
+  for (int bn = least <= 64 ? 64 : 128; bn < kBN && bn >= least; bn *= 2)
+    if (rows * ((N + bn - 1) / bn) <= sms) return bn;
+  return kBN;
+}
+
 // Tile shape for a contraction with M output rows.  Pairs of CTAs are what keeps the tensor cores fed (half the
 // B traffic per flop), 256 rows per CTA run a few percent faster per flop than 128 but make tiles twice as
 // coarse; so the largest shape is taken whose last wave of tiles is still about as full as a finer shape's.
 // A problem of at most 128 rows gets single CTAs (a pair's second CTA would have nothing to do).
-TileShape choose_shape(int M, int N, bool allow_mt2) {
+TileShape choose_shape(int M, int N, int least_columns) {
   const int sms = sm_count();
-  if (M <= 128 || sms < 2) return {1, false};
+  const int narrow = narrow_columns(M, N, least_columns);
+  if (narrow < kBN) return {1, false, narrow};
+  if (M <= 128 || sms < 2) return {1, false, kBN};
   auto fill = [&](const TileShape& s) {
     const long units = sms / (s.pair ? 2 : 1);
-    const long tiles = (long)((M + s.rows() - 1) / s.rows()) * ((N + BN - 1) / BN);
+    const long tiles = (long)((M + s.rows() - 1) / s.rows()) * ((N + kBN - 1) / kBN);
     const long waves = (tiles + units - 1) / units;
     // useful rows / rows computed, times the fill of the last wave
     return ((double)M / ((double)((M + s.rows() - 1) / s.rows()) * s.rows())) * ((double)tiles / (double)(waves * units));
   };
-  const TileShape small{1, true}, large{2, true};
-  if (allow_mt2 && fill(large) * 1.04 > fill(small)) return large;
-  return small;
+  const TileShape small{1, true, kBN}, large{2, true, kBN};
+  return fill(large) * 1.04 > fill(small) ? large : small;
 }
 
 GemmParams base_params(int M, int N, int K) {
@@ -1008,7 +1024,9 @@ void set_latent(GemmParams& p, const eqat_desc& d, const eqat_bf16* W, const flo
 // Dense contraction with the plain store epilogue, over the three operand layouts.
 template <bool A_MN, bool B_MN>
 int launch_dense(const Operand& a, const Operand& b, GemmParams& p, cudaStream_t st) {
-  const TileShape s = choose_shape(p.M, p.N, true);
+  const TileShape s = choose_shape(p.M, p.N, 64);
+  if (s.bn == 64) return launch<1, A_MN, B_MN, false, EPI_STORE, 2, false, 64>(a, b, p, st);
+  if (s.bn == 128) return launch<1, A_MN, B_MN, false, EPI_STORE, 2, false, 128>(a, b, p, st);
   if (!s.pair) return launch<1, A_MN, B_MN, false, EPI_STORE, 2, false>(a, b, p, st);
   return s.mt == 2 ? launch<2, A_MN, B_MN, false, EPI_STORE, 2, true>(a, b, p, st)
                    : launch<1, A_MN, B_MN, false, EPI_STORE, 2, true>(a, b, p, st);
@@ -1016,6 +1034,7 @@ int launch_dense(const Operand& a, const Operand& b, GemmParams& p, cudaStream_t
 
 template <bool B_MN, int BITS>
 int launch_packed(const Operand& a, GemmParams& p, cudaStream_t st) {
+  if (narrow_columns(p.M, p.N, 128) == 128) return launch<1, false, B_MN, true, EPI_STORE, BITS, false, 128>(a, a, p, st);
   // 256 rows per CTA; pairs as soon as there are more rows than one CTA takes
   return p.M > 256 ? launch<2, false, B_MN, true, EPI_STORE, BITS, true>(a, a, p, st)
                    : launch<2, false, B_MN, true, EPI_STORE, BITS, false>(a, a, p, st);
@@ -1023,7 +1042,9 @@ int launch_packed(const Operand& a, GemmParams& p, cudaStream_t st) {
 
 template <int BITS>
 int launch_ds(const Operand& a, const Operand& b, GemmParams& p, cudaStream_t st) {
-  const TileShape s = choose_shape(p.M, p.N, true);
+  const TileShape s = choose_shape(p.M, p.N, p.partial != nullptr ? kBN : 1 << p.group_shift);
+  if (s.bn == 64) return launch<1, true, true, false, EPI_DS, BITS, false, 64>(a, b, p, st);
+  if (s.bn == 128) return launch<1, true, true, false, EPI_DS, BITS, false, 128>(a, b, p, st);
   if (!s.pair) return launch<1, true, true, false, EPI_DS, BITS, false>(a, b, p, st);
   return s.mt == 2 ? launch<2, true, true, false, EPI_DS, BITS, true>(a, b, p, st)
                    : launch<1, true, true, false, EPI_DS, BITS, true>(a, b, p, st);
@@ -1062,6 +1083,9 @@ int launch_dense_dw_ste(const eqat_desc& d, const eqat_bf16* dY, const eqat_bf16
   p.Q = (float)((1 << d.bits) - 1);
   p.dz_literal = d.dz_mode;
   const Operand a{dY, (uint64_t)d.out_features, (uint64_t)d.tokens, true}, b{X, (uint64_t)d.in_features, (uint64_t)d.tokens, true};
+  const int narrow = narrow_columns(p.M, p.N, d.group);
+  if (narrow == 64) return launch<1, true, true, false, EPI_STE, 2, false, 64>(a, b, p, st);
+  if (narrow == 128) return launch<1, true, true, false, EPI_STE, 2, false, 128>(a, b, p, st);
   // 128 rows per CTA: with two accumulator sets this epilogue, the longest of the three, runs under the next tile
   return p.M > 128 ? launch<1, true, true, false, EPI_STE, 2, true>(a, b, p, st)
                    : launch<1, true, true, false, EPI_STE, 2, false>(a, b, p, st);
@@ -1115,7 +1139,7 @@ int launch_packed_dx(const eqat_desc& d, const eqat_bf16* dY, const uint8_t* Wq,
 
 size_t packed_ds_workspace_bytes(const eqat_desc& d) {
   if (!(d.group == d.in_features && d.group > 256)) return 0;
-  const size_t num_n = (size_t)(d.in_features + BN - 1) / BN;
+  const size_t num_n = (size_t)(d.in_features + kBN - 1) / kBN;
   return 2 * num_n * (size_t)d.out_features * sizeof(float);
 }
 
@@ -1135,7 +1159,7 @@ int launch_packed_ds(const eqat_desc& d, const eqat_bf16* X, const eqat_bf16* dY
     default: rc = launch_ds<4>(a, b, p, st); break;
   }
   if (rc != EQAT_OK || !whole_row) return rc;
-  const int num_n = (d.in_features + BN - 1) / BN;
+  const int num_n = (d.in_features + kBN - 1) / kBN;
   return launch_overlapped(finish_row_sums_kernel, dim3((d.out_features + 255) / 256), dim3(256), 0, st, p.partial, num_n,
                            d.out_features, s16, ds, dz);
 }
