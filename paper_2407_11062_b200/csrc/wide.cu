@@ -38,6 +38,7 @@ struct WideParams : PackedWeight {
   int T, tn;                           // tokens, tokens per tile (a multiple of 32)
   int split, split_log2, runs;         // runs = in_features / 128
   int stages;
+  int tile0;                           // first row tile of the launch (an even number)
 };
 
 struct WideCtl {
@@ -80,7 +81,7 @@ wide_fwd_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 
   // grid: row tiles (an even number) x pairs of a cluster x token tiles; cluster = 2 row tiles x split
   const int half = (int)(blockIdx.x & 1u), ks = (int)blockIdx.y;
-  const int m0 = (int)blockIdx.x * kRows, t0 = (int)blockIdx.z * p.tn;
+  const int m0 = (p.tile0 + (int)blockIdx.x) * kRows, t0 = (int)blockIdx.z * p.tn;
   const int run0 = (p.runs * ks) >> p.split_log2, nruns = ((p.runs * (ks + 1)) >> p.split_log2) - run0;
   // barriers that both CTAs of a pair signal live in its first CTA
   auto lead = [&](const void* bar) { return ptx::map_to_cta(ptx::smem_addr(bar), (uint32_t)(2 * ks)); };
@@ -377,6 +378,17 @@ int launch_bits(const WideParams& p, const eqat_bf16* X, dim3 ctas, cudaStream_t
   return launch_status();
 }
 
+int launch_rows(WideParams& p, int bits, const eqat_bf16* X, int pairs, int split, int token_tiles, cudaStream_t st) {
+  p.split = split;
+  p.split_log2 = log2_exact(split);
+  const dim3 ctas((unsigned)pairs * 2u, (unsigned)split, (unsigned)token_tiles);
+  switch (bits) {
+    case 2: return launch_bits<2>(p, X, ctas, st);
+    case 3: return launch_bits<3>(p, X, ctas, st);
+    default: return launch_bits<4>(p, X, ctas, st);
+  }
+}
+
 }  // namespace
 
 // Whether this kernel is expected to beat the tiled kernel of gemm.cu (512 or 256 TOKENS x 256 weight rows per tile), and
@@ -387,21 +399,34 @@ int launch_bits(const WideParams& p, const eqat_bf16* X, dim3 ctas, cudaStream_t
 // for at most 256 tokens, 0.88 / 1.13 / 1.15 us on one CTA.  4096 x 4096, 2 bits: 128 tokens 64.2 -> 13.2 us, 333 tokens
 // 49.4 -> 16.2 us, 1024 tokens 49.8 -> 29 us; at 2048 tokens the tiled kernel is ahead (51 against 58 us).
 bool wide_fwd_applies(const eqat_desc& d, int given_sms, WidePlan& best) {
-  best = WidePlan{0, 0, 0, 0.0};
+  best = WidePlan{};
   const int sms = given_sms > 0 ? given_sms : sm_count();
   if (d.tokens > 4096 || sms < 2) return false;
   const int T = (int)d.tokens, runs = d.in_features / kRun, pairs = (d.out_features + 2 * kRows - 1) / (2 * kRows);
   const int least = (T + kMaxTn - 1) / kMaxTn;
+  auto resident = [&](int lg) { return given_sms > 0 ? sms * kResidentOf148[lg] / 148 : max_clusters(d.bits, lg); };
   for (int tt = least; tt <= least + 3; ++tt) {
     const int tn = ((T + tt - 1) / tt + 31) / 32 * 32;
-    for (int lg = 0; (1 << lg) <= kMaxSplit && (1 << lg) <= runs; ++lg) {
-      const int clusters = pairs * tt, resident = given_sms > 0 ? sms * kResidentOf148[lg] / 148 : max_clusters(d.bits, lg);
-      if (resident <= 0) continue;
-      const int rounds = (clusters + resident - 1) / resident;
+    auto round_us = [&](int lg, int clusters) {              // of clusters that are resident together
       const double expand = d.bits == 3 ? 0.62 : 0.41, mma = 0.0021 * tn;
       const double load = (clusters << lg) * 2 > 100 ? 1.25 : 1.0;
-      const double us = rounds * (5.0 + 0.018 * tn + ((runs + (1 << lg) - 1) >> lg) * (expand > mma ? expand : mma) * load);
-      if (best.us == 0.0 || us < best.us) best = WidePlan{tn, (T + tn - 1) / tn, 1 << lg, us};
+      return 5.0 + 0.018 * tn + ((runs + (1 << lg) - 1) >> lg) * (expand > mma ? expand : mma) * load;
+    };
+    for (int lg = 0; (1 << lg) <= kMaxSplit && (1 << lg) <= runs; ++lg) {
+      const int clusters = pairs * tt, fit = resident(lg);
+      if (fit <= 0) continue;
+      const double us = (clusters + fit - 1) / fit * round_us(lg, clusters);
+      if (best.us == 0.0 || us < best.us) best = WidePlan{tn, (T + tn - 1) / tn, 1 << lg, pairs, 1, us};
+      // The whole rounds as they are, and what is left over split finer: 11008 x 4096, 2 bits, 333 tokens has 86 clusters of
+      // which 74 are resident, 50.4 us in two rounds (or tiled), 37.7 us with the last twelve split four ways; 28672 x 8192,
+      // 4 bits, 333 tokens 175.9 -> 157.7 us, 4096 x 11008, 4 bits, 1531 tokens 127.6 -> 116.7 us.
+      const int whole = clusters / fit * fit / tt;           // pairs of row tiles, with all their token tiles
+      for (int lg2 = lg + 1; whole > 0 && whole < pairs && (1 << lg2) <= kMaxSplit && (1 << lg2) <= runs; ++lg2) {
+        const int rest = (pairs - whole) * tt, fit2 = resident(lg2);
+        if (fit2 <= 0) continue;
+        const double two = clusters / fit * round_us(lg, clusters) + (rest + fit2 - 1) / fit2 * round_us(lg2, rest);
+        if (two < best.us) best = WidePlan{tn, (T + tn - 1) / tn, 1 << lg, whole, 1 << lg2, two};
+      }
     }
   }
   if (best.us == 0.0) return false;
@@ -426,16 +451,15 @@ int launch_wide_fwd(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, c
   p.Y = Y;
   p.T = (int)d.tokens;
   p.tn = pl.tn;
-  p.split = pl.split;
-  p.split_log2 = log2_exact(pl.split);
   p.runs = d.in_features / kRun;
   p.stages = stages_that_fit(d.bits, pl.tn);
-  const dim3 ctas((unsigned)((d.out_features + 2 * kRows - 1) / (2 * kRows)) * 2u, (unsigned)pl.split, (unsigned)pl.token_tiles);
-  switch (d.bits) {
-    case 2: return launch_bits<2>(p, X, ctas, st);
-    case 3: return launch_bits<3>(p, X, ctas, st);
-    default: return launch_bits<4>(p, X, ctas, st);
+  const int pairs = (d.out_features + 2 * kRows - 1) / (2 * kRows);
+  int rc = launch_rows(p, d.bits, X, pl.first_pairs, pl.split, pl.token_tiles, st);
+  if (rc == EQAT_OK && pl.first_pairs < pairs) {
+    p.tile0 = 2 * pl.first_pairs;
+    rc = launch_rows(p, d.bits, X, pairs - pl.first_pairs, pl.rest_split, pl.token_tiles, st);
   }
+  return rc;
 }
 
 int launch_wait_expiry_wide(cudaStream_t st) { return launch_wait_expiry(st); }

@@ -8,6 +8,8 @@ namespace eqat {
 struct WidePlan {
   int tn, token_tiles;       // tokens per tile
   int split;                 // pairs of CTAs per cluster, over K
+  int first_pairs;           // pairs of row tiles that are computed so; the others, in a launch of their own,
+  int rest_split;            // with this split
   double us;                 // expected time; 0: the problem does not fit
 };
 // True when the kernel is the one to take for this packed forward, and how: on the current device (sms = 0), or on one of
