@@ -214,10 +214,4 @@ __device__ __forceinline__ float step_size_at(const GroupParamsRaw& r, int i) { 
 __device__ __forceinline__ float zero_point_at(const GroupParamsRaw& r, int i, int z_fp16) {
   return z_fp16 ? half_at(r.z, i) : (float)((r.z.x >> (8 * i)) & 0xFFu);
 }
-// Zero point of one group, whichever way it is stored.
-__device__ __forceinline__ float load_zero_point(const PackedWeight& p, size_t gi) {
-  return p.z_fp16 ? __half2float(__ushort_as_half(ptx::ld_global(static_cast<const eqat_fp16*>(p.zq) + gi)))
-                  : (float)ptx::ld_global(static_cast<const uint8_t*>(p.zq) + gi);
-}
-
 }  // namespace eqat

@@ -26,13 +26,13 @@
 //   warp 1      MMA issuer (first CTA of a pair only): an elected lane issues tcgen05.mma,
 //               frees stages in both CTAs with tcgen05.commit; owns the TMEM allocation
 //   warps 2-5   epilogue: tcgen05.ld the finished accumulator (one TMEM lane
-//               quadrant each)
+//               quadrant each); MT = 2: warps 6-9 do the second 128 rows
 //   warps 2-17  (packed-weight kernels only) expand N-bit codes into the bf16 B
 //               operand, (q - z) * s, rounded once to bf16.  That operand has a
 //               ring of its own; the sixteen warps form groups of as many threads
 //               as the CTA's B stage has rows (one 64-code row per thread and K
 //               block) and the groups take alternate runs of one or two K blocks,
-//               two ring stages per group.  Warps 2-5 then run the tile's epilogue.
+//               two ring stages per group.  The first of them then run the tile's epilogue.
 // The epilogue either stores the tile as bf16; or, for the E2E-QP step-size
 // gradient, multiplies each accumulator row by (q - z) of the matching packed
 // codes and reduces runs of `group` columns, so the [out,in] weight gradient
@@ -64,8 +64,7 @@ constexpr int BM = 128;          // rows per CTA and MMA = TMEM lanes
 constexpr int kBN = 256;         // columns per tile (128 or 64 where a problem is too small to fill the chip)
 constexpr int BK = 64;           // K per stage: one 128-byte swizzle span of bf16
 constexpr int UMMA_K = 16;       // K per tcgen05.mma for 16-bit inputs
-constexpr int kEpiWarps = 4;       // dense kernels: warps 2-5 are the epilogue
-constexpr int kDeqWarps = 16;      // packed kernels: warps 2-17 expand codes; warps 2-5 also run the epilogue
+constexpr int kDeqWarps = 16;      // packed kernels: warps 2-17 expand codes; the first of them also run the epilogue
 constexpr uint64_t kDrainLimitNs = 50000000ull;    // 50 ms per stage at teardown
 
 enum Epilogue : int { EPI_STORE = 0, EPI_DS = 1, EPI_STE = 2 };
@@ -106,6 +105,9 @@ struct Cfg {
   __host__ __device__ static constexpr int b_offset(int stage_b) {
     return PACKED ? kStages * kABytes + stage_b * kBBytes : stage_b * kStageBytes + kABytes;
   }
+  // Warps of the epilogue, from warp 2 on: four per 128 rows.  With 256 rows per CTA there is one accumulator set, so the
+  // tensor core waits for them: a second four take the second half of the rows.
+  static constexpr int kEpiWarps = 4 * MT;
   static constexpr int kThreads = (2 + (PACKED ? kDeqWarps : kEpiWarps)) * 32;
   static constexpr int kTmemCols = kAccSets * MT * BN;
   static constexpr int kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 512 /*barriers*/;
@@ -215,7 +217,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
     }
     for (int a = 0; a < C::kAccSets; ++a) {
       ptx::mbar_init(ptx::smem_addr(&ctl->acc_full[a]), 1);
-      ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty[a]), C::kCtas * kEpiWarps);
+      ptx::mbar_init(ptx::smem_addr(&ctl->acc_empty[a]), C::kCtas * C::kEpiWarps);
     }
     ptx::mbar_init(ptx::smem_addr(&ctl->drain), 1);
     ctl->abort = 0;
@@ -247,142 +249,171 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   ptx::grid_dependency_wait();                                     // nothing above touches global memory
 
   // ---------------------------------------------------------------- epilogue of one tile
-  // Run by four warps, one per TMEM lane quadrant (warp index mod 4).  `m0` is the first output row of this CTA's
-  // part of the tile.
+  // Run by four warps per 128 rows, one per TMEM lane quadrant (warp index mod 4).  `m0` is the first output row of this
+  // CTA's part of the tile.  What an epilogue reads from global memory it asks for a step ahead, and for the first step
+  // before the accumulators are there.
+  // (The step-size gradient of 4096 x 11008, 4 bits, 1531 tokens: 155.6 -> 126.2 us with this and the second four warps;
+  // waiting for its codes, each step of 32 columns took as long as two K blocks.)
   const int quad = warp & 3;
   const int row_in_tile = quad * 32 + lane;
   auto epilogue_tile = [&](int m0, int n_blk, int acc, uint32_t acc_phase) -> bool {
-    if (!bounded_wait_warp<PAIR>(ptx::smem_addr(&ctl->acc_full[acc]), acc_phase, abort_flag, WAIT_EPI_ACC_FULL,
-                                 PACKED ? 0 : (MT == 2 ? 512 : 128)))
-      return false;
-    ptx::tc_fence_after();
+    const int h = MT == 2 ? (warp - 2) >> 2 : 0;
+    const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)((acc * MT + h) * BN);
+    const int m = m0 + h * BM + row_in_tile;
+    auto accumulators = [&]() {
+      const bool ok = bounded_wait_warp<PAIR>(ptx::smem_addr(&ctl->acc_full[acc]), acc_phase, abort_flag, WAIT_EPI_ACC_FULL,
+                                              PACKED ? 0 : (MT == 2 ? 512 : 128));
+      ptx::tc_fence_after();
+      return ok;
+    };
+    if constexpr (EPI == EPI_STORE) {
+      if (!accumulators()) return false;
 #pragma unroll 1
-    for (int h = 0; h < MT; ++h) {
-      const uint32_t t_row = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)((acc * MT + h) * BN);
-      const int m = m0 + h * BM + row_in_tile;
-      if constexpr (EPI == EPI_STORE) {
-#pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
-          uint32_t r[32];
-          ptx::tmem_ld_32x32(t_row + c * 32, r);
-          ptx::tmem_ld_wait();
-          const int col0 = n_blk * BN + c * 32;
-          // A lane owns a row, so a plain store instruction would hit 32 different lines, and it is the stores, not
-          // the TMEM loads, that set the pace of this epilogue.  The four lanes of a quad therefore trade 16-byte
-          // pieces so that each store instruction writes 64 contiguous bytes of one row per quad: 8 lines instead
-          // of 32.  (N is a multiple of 16 for every shape the library accepts, so a piece is never ragged.)
-          uint32_t o[16];
+      for (int c = 0; c < BN / 32; ++c) {
+        uint32_t r[32];
+        ptx::tmem_ld_32x32(t_row + c * 32, r);
+        ptx::tmem_ld_wait();
+        const int col0 = n_blk * BN + c * 32;
+        // A lane owns a row, so a plain store instruction would hit 32 different lines, and it is the stores, not
+        // the TMEM loads, that set the pace of this epilogue.  The four lanes of a quad therefore trade 16-byte
+        // pieces so that each store instruction writes 64 contiguous bytes of one row per quad: 8 lines instead
+        // of 32.  (N is a multiple of 16 for every shape the library accepts, so a piece is never ragged.)
+        uint32_t o[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) o[i] = pack_bf16x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
-          quad_transpose(o, lane);
-          const int q = lane & 3;
-          if (col0 + q * 8 < p.N) {
+        for (int i = 0; i < 16; ++i) o[i] = pack_bf16x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+        quad_transpose(o, lane);
+        const int q = lane & 3;
+        if (col0 + q * 8 < p.N) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int mk = m - q + k;
-              if (mk < p.M)
-                *reinterpret_cast<uint4*>(p.D + (size_t)mk * p.N + col0 + q * 8) =
-                    make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
-            }
+          for (int k = 0; k < 4; ++k) {
+            const int mk = m - q + k;
+            if (mk < p.M)
+              *reinterpret_cast<uint4*>(p.D + (size_t)mk * p.N + col0 + q * 8) =
+                  make_uint4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
           }
         }
-      } else if constexpr (EPI == EPI_STE) {
-        // Block-AP: the accumulator row is the gradient of row m of W_hat.  Eqs. 3-5 are applied to it here,
-        // in fp32, next to the matching latent weights: dW = G where the code is in range, ds and dz are the
-        // group sums of G times the partials.  G itself is never written.
-        const int groups_per_row = p.N >> p.group_shift;
-        const int chunks_per_group = 1 << (p.group_shift - 5);
-        const eqat_bf16* wrow = p.W + (size_t)m * p.N;
-        eqat_bf16* drow = p.D + (size_t)m * p.N;
-        float acc_s = 0.0f, acc_g = 0.0f;
-#pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
-          const int col0 = n_blk * BN + c * 32;
-          const bool live = m < p.M && col0 < p.N;
-          uint4 wraw[4];
-          float sv = 1.0f, zr = 0.0f;
-          if (live) {
+      }
+    } else if constexpr (EPI == EPI_STE) {
+      // Block-AP: the accumulator row is the gradient of row m of W_hat.  Eqs. 3-5 are applied to it here,
+      // in fp32, next to the matching latent weights: dW = G where the code is in range, ds and dz are the
+      // group sums of G times the partials.  G itself is never written.
+      const int groups_per_row = p.N >> p.group_shift;
+      const int chunks_per_group = 1 << (p.group_shift - 5);
+      const eqat_bf16* wrow = p.W + (size_t)m * p.N;
+      eqat_bf16* drow = p.D + (size_t)m * p.N;
+      float acc_s = 0.0f, acc_g = 0.0f;
+      uint4 w_next[4];
+      float s_next = 1.0f, z_next = 0.0f;
+      auto fetch = [&](int c) {
+        const int col0 = n_blk * BN + c * 32;
+        if (m < p.M && col0 < p.N) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) wraw[v] = ptx::ld_global(reinterpret_cast<const uint4*>(wrow + col0) + v);
+          for (int v = 0; v < 4; ++v) w_next[v] = ptx::ld_global(reinterpret_cast<const uint4*>(wrow + col0) + v);
+          const size_t gi = (size_t)m * groups_per_row + (col0 >> p.group_shift);
+          s_next = ptx::ld_global(p.s32 + gi);
+          z_next = ptx::ld_global(p.z32 + gi);
+        }
+      };
+      fetch(0);
+      if (!accumulators()) return false;
+#pragma unroll 1
+      for (int c = 0; c < BN / 32; ++c) {
+        const int col0 = n_blk * BN + c * 32;
+        const bool live = m < p.M && col0 < p.N;
+        uint4 wraw[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) wraw[v] = w_next[v];
+        const float sv = s_next, zr = rintf(z_next);
+        if (c + 1 < BN / 32) fetch(c + 1);
+        uint32_t r32[32];
+        ptx::tmem_ld_32x32(t_row + c * 32, r32);
+        ptx::tmem_ld_wait();
+        if (live) {
+          const float rs = group_rcp(sv, zr);
+          const float lo = -zr, hi = p.Q - zr;
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            float w[8], r[8], rt[8];
+            unpack8(wraw[v], w);
+            quotient_round8(w, sv, rs, r, rt);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float gr = __uint_as_float(r32[8 * v + i]);
+              const float cl = fminf(fmaxf(r[i], lo), hi);
+              const bool inside = (cl == r[i]);
+              acc_s = fmaf(gr, inside ? rt[i] : cl, acc_s);     // Eq. 3
+              acc_g += inside ? 0.0f : gr;                      // Eq. 4
+              w[i] = inside ? gr : 0.0f;                        // Eq. 5
+            }
+            reinterpret_cast<uint4*>(drow + col0)[v] = pack8(w);
+          }
+          if (((c + 1) & (chunks_per_group - 1)) == 0) {
             const size_t gi = (size_t)m * groups_per_row + (col0 >> p.group_shift);
-            sv = ptx::ld_global(p.s32 + gi);
-            zr = rintf(ptx::ld_global(p.z32 + gi));
-          }
-          uint32_t r32[32];
-          ptx::tmem_ld_32x32(t_row + c * 32, r32);
-          ptx::tmem_ld_wait();
-          if (live) {
-            const float rs = group_rcp(sv, zr);
-            const float lo = -zr, hi = p.Q - zr;
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-              float w[8], r[8], rt[8];
-              unpack8(wraw[v], w);
-              quotient_round8(w, sv, rs, r, rt);
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const float gr = __uint_as_float(r32[8 * v + i]);
-                const float cl = fminf(fmaxf(r[i], lo), hi);
-                const bool inside = (cl == r[i]);
-                acc_s = fmaf(gr, inside ? rt[i] : cl, acc_s);     // Eq. 3
-                acc_g += inside ? 0.0f : gr;                      // Eq. 4
-                w[i] = inside ? gr : 0.0f;                        // Eq. 5
-              }
-              reinterpret_cast<uint4*>(drow + col0)[v] = pack8(w);
-            }
-            if (((c + 1) & (chunks_per_group - 1)) == 0) {
-              const size_t gi = (size_t)m * groups_per_row + (col0 >> p.group_shift);
-              p.ds[gi] = acc_s;
-              if (p.dz != nullptr) p.dz[gi] = (p.dz_literal ? -1.0f : -sv) * acc_g;
-              acc_s = 0.0f;
-              acc_g = 0.0f;
-            }
+            p.ds[gi] = acc_s;
+            if (p.dz != nullptr) p.dz[gi] = (p.dz_literal ? -1.0f : -sv) * acc_g;
+            acc_s = 0.0f;
+            acc_g = 0.0f;
           }
         }
-      } else {
-        // Row m of the tile is output row o = m of the weight; columns are input
-        // features.  ds[o,g] = sum_{j in g} G[o,j] * (q[o,j] - z[o,g]).  With one group per row the tile
-        // holds 256 of the row's columns: its sums go to the partial arrays and a second kernel adds the
-        // column tiles up in a fixed order.
-        const bool whole_row = p.partial != nullptr;
-        const int chunks_per_group = whole_row ? BN / 32 : 1 << (p.group_shift - 5);
-        const uint8_t* qrow = p.Wq + (size_t)m * ((size_t)p.in_features * BITS / 8);
-        float acc_s = 0.0f, acc_g = 0.0f;
+      }
+    } else {
+      // Row m of the tile is output row o = m of the weight; columns are input
+      // features.  ds[o,g] = sum_{j in g} G[o,j] * (q[o,j] - z[o,g]).  With one group per row the tile
+      // holds 256 of the row's columns: its sums go to the partial arrays and a second kernel adds the
+      // column tiles up in a fixed order.
+      const bool whole_row = p.partial != nullptr, wants_s = p.dz != nullptr && !whole_row;
+      const int chunks_per_group = whole_row ? BN / 32 : 1 << (p.group_shift - 5);
+      const uint8_t* qrow = p.Wq + (size_t)m * ((size_t)p.in_features * BITS / 8);
+      float acc_s = 0.0f, acc_g = 0.0f;
+      uint32_t w_next[BITS], z_next = 0u, s_next = 0u;                 // zero point (byte or fp16) and step size as stored
+      auto fetch = [&](int c) {
+        const int col0 = n_blk * BN + c * 32;
+        if (m < p.M && col0 < p.N) {
+          const uint32_t* src = reinterpret_cast<const uint32_t*>(qrow) + (size_t)(col0 >> 5) * BITS;
+#pragma unroll
+          for (int i = 0; i < BITS; ++i) w_next[i] = ptx::ld_global(src + i);
+          const size_t gi = (size_t)m * p.groups_per_row + (col0 >> p.group_shift);
+          z_next = p.z_fp16 ? (uint32_t)ptx::ld_global(static_cast<const eqat_fp16*>(p.zq) + gi)
+                            : ptx::ld_global(static_cast<const uint8_t*>(p.zq) + gi);
+          if (wants_s) s_next = (uint32_t)ptx::ld_global(p.s16 + gi);
+        }
+      };
+      fetch(0);
+      if (!accumulators()) return false;
 #pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
-          uint32_t r[32];
-          ptx::tmem_ld_32x32(t_row + c * 32, r);
-          ptx::tmem_ld_wait();
-          const int col0 = n_blk * BN + c * 32;
-          if (m < p.M) {
-            if (col0 < p.N) {
-              uint32_t words[BITS];
-              const uint32_t* src = reinterpret_cast<const uint32_t*>(qrow) + (size_t)(col0 >> 5) * BITS;
+      for (int c = 0; c < BN / 32; ++c) {
+        uint32_t words[BITS];
 #pragma unroll
-              for (int i = 0; i < BITS; ++i) words[i] = ptx::ld_global(src + i);
-              uint32_t codes[32];
-              unpack32<BITS>(words, codes);
+        for (int i = 0; i < BITS; ++i) words[i] = w_next[i];
+        const uint32_t z_raw = z_next, s_raw = s_next;
+        if (c + 1 < BN / 32) fetch(c + 1);
+        uint32_t r[32];
+        ptx::tmem_ld_32x32(t_row + c * 32, r);
+        ptx::tmem_ld_wait();
+        const int col0 = n_blk * BN + c * 32;
+        if (m < p.M) {
+          if (col0 < p.N) {
+            uint32_t codes[32];
+            unpack32<BITS>(words, codes);
+            const float zf = p.z_fp16 ? __half2float(__ushort_as_half((unsigned short)z_raw)) : (float)z_raw;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              const float gv = __uint_as_float(r[i]);
+              acc_s = fmaf(gv, (float)codes[i] - zf, acc_s);
+              acc_g += gv;
+            }
+          }
+          if (((c + 1) & (chunks_per_group - 1)) == 0) {
+            if (whole_row) {
+              p.partial[(size_t)n_blk * p.M + m] = acc_s;
+              p.partial[(size_t)(num_n + n_blk) * p.M + m] = acc_g;
+            } else if (col0 < p.N) {
               const size_t gi = (size_t)m * p.groups_per_row + (col0 >> p.group_shift);
-              const float zf = load_zero_point(p, gi);
-#pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                const float gv = __uint_as_float(r[i]);
-                acc_s = fmaf(gv, (float)codes[i] - zf, acc_s);
-                acc_g += gv;
-              }
+              p.ds[gi] = acc_s;
+              if (p.dz != nullptr) p.dz[gi] = -__half2float(__ushort_as_half((unsigned short)s_raw)) * acc_g;
             }
-            if (((c + 1) & (chunks_per_group - 1)) == 0) {
-              if (whole_row) {
-                p.partial[(size_t)n_blk * p.M + m] = acc_s;
-                p.partial[(size_t)(num_n + n_blk) * p.M + m] = acc_g;
-              } else if (col0 < p.N) {
-                const size_t gi = (size_t)m * p.groups_per_row + (col0 >> p.group_shift);
-                p.ds[gi] = acc_s;
-                if (p.dz != nullptr) p.dz[gi] = -__half2float(__ushort_as_half(ptx::ld_global(p.s16 + gi))) * acc_g;
-              }
-              acc_s = 0.0f;
-              acc_g = 0.0f;
-            }
+            acc_s = 0.0f;
+            acc_g = 0.0f;
           }
         }
       }
@@ -801,7 +832,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
           }
         }
         gk += num_kb;
-        if (warp < 2 + kEpiWarps && ok) {
+        if (warp < 2 + C::kEpiWarps && ok) {
           ok = epilogue_tile(m_blk * C::kClusterM + rank * C::kTileM, n_blk, acc, acc_phase);
           if (++acc == C::kAccSets) { acc = 0; acc_phase ^= 1u; }
         }
