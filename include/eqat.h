@@ -252,7 +252,8 @@ int qlinear_packed_fwd(const eqat_desc* desc, const eqat_bf16* X, const uint8_t*
  * number of SMs to decide for, 0 for the current device.  Returns one of the
  * EQAT_ROUTE_* values or a negative eqat_status.  h_plan (may be NULL) receives
  * three numbers: launches or token tiles, tokens of each, and the split of K
- * over a cluster (0, 0, 1 for the tiled kernel). */
+ * over a cluster (0, 0, 1 for the tiled kernel).  Where a prompt goes out as two
+ * launches the split is the first one's (eqat_packed_fwd_rest has the other). */
 enum {
   EQAT_ROUTE_MATRIX_VECTOR = 1,     /* a few tokens: up to eight per pass over the weight   */
   EQAT_ROUTE_WEIGHT_ROWS = 2,       /* up to 64 tokens: tiles of 128 weight rows            */
@@ -260,6 +261,13 @@ enum {
   EQAT_ROUTE_TILED = 4              /* large batches: tiles of 512 or 256 tokens            */
 };
 int eqat_packed_fwd_route(const eqat_desc* desc, int sms, int* h_plan);
+
+/* The second launch of a prompt on pairs of weight-row tiles: its weight rows, the
+ * last ones of the weight, whose K is split over larger clusters than that of the
+ * rows before them.  The token tiles are the same.  Same arguments as above (a
+ * diagnostic); h_rest receives the number of those rows and their split, or 0 and 0
+ * where one launch takes all rows. */
+int eqat_packed_fwd_rest(const eqat_desc* desc, int sms, int* h_rest);
 
 /* dX = dY * ((W_int - z) * s).
  *   dY [T,out] bf16, Wq_packed, s16, z (in)   dX [T,in] bf16 (out) */

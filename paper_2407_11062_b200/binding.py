@@ -72,6 +72,7 @@ def _load():
         "eqat_unpack_zeros": (c_int, [D, P, P, P]),
         "qlinear_packed_fwd": (c_int, [D, P, P, P, P, P, P]),
         "eqat_packed_fwd_route": (c_int, [D, c_int, POINTER(c_int)]),
+        "eqat_packed_fwd_rest": (c_int, [D, c_int, POINTER(c_int)]),
         "qlinear_packed_bwd_dx": (c_int, [D, P, P, P, P, P, P]),
         "qlinear_packed_bwd_ds": (c_int, [D, P, P, P, P, P, P, P, P, c_size_t, P]),
         "eqat_block_ap_step": (c_int, [POINTER(eqat_block_ap_linear), c_int, POINTER(c_int), P]),
@@ -210,6 +211,13 @@ def eqat_packed_fwd_route(desc, sms=0):
     if kernel < 0:
         raise EqatError(kernel, "eqat_packed_fwd_route")
     return kernel, tuple(plan)
+
+
+def eqat_packed_fwd_rest(desc, sms=0):
+    """Weight rows of the second launch of a prompt on pairs of weight-row tiles, and its split of K; (0, 0) if there is none."""
+    rest = (c_int * 2)()
+    _check(lib.eqat_packed_fwd_rest(ctypes.byref(desc), int(sms), rest), "eqat_packed_fwd_rest")
+    return tuple(rest)
 
 
 def qlinear_packed_bwd_dx(desc, dY, Wq_packed, s16, z8, dX):

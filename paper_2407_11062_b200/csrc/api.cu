@@ -300,6 +300,17 @@ int eqat_packed_fwd_route(const eqat_desc* d, int sms, int* h_plan) {
   return r.kernel;
 }
 
+int eqat_packed_fwd_rest(const eqat_desc* d, int sms, int* h_rest) {
+  EQAT_TRY(check_gemm_desc(d, true));
+  if (h_rest == nullptr) return EQAT_ERR_NULL;
+  if (sms < 0) return EQAT_ERR_SHAPE;
+  const PackedRoute r = packed_route(*d, sms);
+  const int rows = r.kernel == EQAT_ROUTE_WEIGHT_ROW_PAIRS ? d->out_features - 256 * r.wide.first_pairs : 0;
+  h_rest[0] = rows > 0 ? rows : 0;
+  h_rest[1] = rows > 0 ? r.wide.rest_split : 0;
+  return EQAT_OK;
+}
+
 int qlinear_packed_bwd_dx(const eqat_desc* d, const eqat_bf16* dY, const uint8_t* Wq_packed, const eqat_fp16* s16,
                           const void* z, eqat_bf16* dX, void* stream) {
   EQAT_TRY(v_packed_fwd(d, dY, Wq_packed, s16, z, dX));          // same shape of check: one activation in, one out

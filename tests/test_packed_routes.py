@@ -85,6 +85,27 @@ def test_plans_cover_all_tokens(eqat):
             assert (parts - 1) * each < tokens <= parts * each and split in (1, 2, 4, 8)
 
 
+def test_the_rest_of_a_prompt_is_told(eqat):
+    """Where a prompt goes out as two launches, the second one's rows and its split of K."""
+    def rest(out, in_f, tokens, bits, group, fp16_z=False):
+        zfmt = eqat.EQAT_ZP_FP16 if fp16_z else eqat.EQAT_ZP_U8
+        return eqat.eqat_packed_fwd_rest(eqat.make_desc(bits, group, out, in_f, tokens, 0, zfmt), SMS)
+
+    assert route(eqat, 11008, 4096, 333, 2, 64) == (eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS, (2, 192, 1))
+    assert rest(11008, 4096, 333, 2, 64) == (1536, 4)           # 86 clusters, 74 resident: the last six pairs of row tiles
+    assert rest(4096, 11008, 1531, 4, 64, True) == (1024, 2)
+    assert rest(4096, 4096, 333, 2, 64) == (0, 0)               # one round
+    assert rest(512, 512, 4, 2, 64) == (0, 0)                   # another kernel
+    import test_gpu_weight_row_forward as gpu
+    for problem, tiles, split in gpu.REST:
+        kernel, (token_tiles, _, first) = route(eqat, *problem)
+        assert (kernel, token_tiles, first) == (eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS, tiles, 1), problem
+        rows, second = rest(*problem)
+        assert 0 < rows < problem[0] and second == split, problem
+    with pytest.raises(eqat.EqatError):
+        eqat.eqat_packed_fwd_rest(eqat.make_desc(2, 64, 512, 512, 4), -1)
+
+
 def test_the_query_checks_its_descriptor(eqat):
     with pytest.raises(eqat.EqatError):
         eqat.eqat_packed_fwd_route(eqat.make_desc(2, 64, 96, 512, 4), SMS)
