@@ -111,7 +111,7 @@ minmax_long_group_kernel(const eqat_bf16* W, float* __restrict__ s, float* __res
   ptx::grid_dependents_launch();
   ptx::grid_dependency_wait();
   __shared__ float red_mx[kThreads / 32], red_mn[kThreads / 32];
-  const size_t g = blockIdx.x;
+  const size_t g = gridDim.x - 1 - blockIdx.x;      // from the end of the weight, as in stream.cu
   float mx = -INFINITY, mn = INFINITY;
   for (int k = threadIdx.x; k < vec_per_group; k += kThreads) {
     const Vec8 w = load_bf16x8(W, g * (size_t)vec_per_group + k);
