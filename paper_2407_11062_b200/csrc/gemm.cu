@@ -946,14 +946,6 @@ bool make_tmap(CUtensorMap* tm, const void* base, uint64_t inner, uint64_t outer
   return make_tmap_bf16(tm, base, inner, outer, box_outer);
 }
 
-// How a contraction's tiles are shaped: rows per CTA (128 * mt), whether pairs of CTAs share a tile, and its columns.
-struct TileShape {
-  int mt;
-  bool pair;
-  int bn;
-  int rows() const { return 128 * mt * (pair ? 2 : 1); }
-};
-
 // One operand of a contraction: a bf16 matrix and which way it is walked.
 //   K-major : [rows, K] row-major, tiled in boxes of 64 K x `rows per CTA`
 //   MN-major: [K, rows] row-major, tiled in boxes of 64 rows x 64 K
@@ -1008,8 +1000,8 @@ int launch(const Operand& a, const Operand& b, const GemmParams& p, cudaStream_t
 // (24 KB to fetch) as with 256 of a pair (32 KB), so more and smaller tiles shorten the chain as long as every SM has one.
 // 512 x 512, 256 tokens: Block-AP forward 9.0 -> 6.5 us, backward 20.1 -> 10.6 us, E2E-QP 23.7 -> 15.6 us; packed dX of
 // 2048 x 2048, 200 tokens 29.4 -> 16.4 us.
-int narrow_columns(int M, int N, int least) {
-  const long sms = sm_count(), rows = (M + 127) / 128;
+int narrow_columns(int M, int N, int least, int sms) {
+  const long rows = (M + 127) / 128;
   for (int bn = least <= 64 ? 64 : 128; bn < kBN && bn >= least; bn *= 2)
     if (rows * ((N + bn - 1) / bn) <= sms) return bn;
   return kBN;
@@ -1019,9 +1011,8 @@ int narrow_columns(int M, int N, int least) {
 // B traffic per flop), 256 rows per CTA run a few percent faster per flop than 128 but make tiles twice as
 // coarse; so the largest shape is taken whose last wave of tiles is still about as full as a finer shape's.
 // A problem of at most 128 rows gets single CTAs (a pair's second CTA would have nothing to do).
-TileShape choose_shape(int M, int N, int least_columns) {
-  const int sms = sm_count();
-  const int narrow = narrow_columns(M, N, least_columns);
+TileShape choose_shape(int M, int N, int least_columns, int sms) {
+  const int narrow = narrow_columns(M, N, least_columns, sms);
   if (narrow < kBN) return {1, false, narrow};
   if (M <= 128 || sms < 2) return {1, false, kBN};
   auto fill = [&](const TileShape& s) {
@@ -1034,6 +1025,24 @@ TileShape choose_shape(int M, int N, int least_columns) {
   const TileShape small{1, true, kBN}, large{2, true, kBN};
   return fill(large) * 1.04 > fill(small) ? large : small;
 }
+
+// Eqs. 3-5 in the epilogue.  128 rows per CTA: with two accumulator sets this epilogue, the longest of the three, runs under
+// the next tile.
+TileShape ste_shape(int M, int N, int group, int sms) {
+  const int bn = narrow_columns(M, N, group, sms);
+  return {1, bn == kBN && M > 128, bn};
+}
+
+}  // namespace
+
+// Packed codes: 256 rows per CTA, pairs as soon as there are more rows than one CTA takes.  (128 columns are the least that
+// the expansion's threads work on.)
+TileShape packed_shape(int M, int N, int sms) {
+  if (narrow_columns(M, N, 128, sms) == 128) return {1, false, 128};
+  return {2, M > 256, kBN};
+}
+
+namespace {
 
 GemmParams base_params(int M, int N, int K) {
   GemmParams p{};
@@ -1055,7 +1064,7 @@ void set_latent(GemmParams& p, const eqat_desc& d, const eqat_bf16* W, const flo
 // Dense contraction with the plain store epilogue, over the three operand layouts.
 template <bool A_MN, bool B_MN>
 int launch_dense(const Operand& a, const Operand& b, GemmParams& p, cudaStream_t st) {
-  const TileShape s = choose_shape(p.M, p.N, 64);
+  const TileShape s = choose_shape(p.M, p.N, 64, sm_count());
   if (s.bn == 64) return launch<1, A_MN, B_MN, false, EPI_STORE, 2, false, 64>(a, b, p, st);
   if (s.bn == 128) return launch<1, A_MN, B_MN, false, EPI_STORE, 2, false, 128>(a, b, p, st);
   if (!s.pair) return launch<1, A_MN, B_MN, false, EPI_STORE, 2, false>(a, b, p, st);
@@ -1065,15 +1074,15 @@ int launch_dense(const Operand& a, const Operand& b, GemmParams& p, cudaStream_t
 
 template <bool B_MN, int BITS>
 int launch_packed(const Operand& a, GemmParams& p, cudaStream_t st) {
-  if (narrow_columns(p.M, p.N, 128) == 128) return launch<1, false, B_MN, true, EPI_STORE, BITS, false, 128>(a, a, p, st);
-  // 256 rows per CTA; pairs as soon as there are more rows than one CTA takes
-  return p.M > 256 ? launch<2, false, B_MN, true, EPI_STORE, BITS, true>(a, a, p, st)
-                   : launch<2, false, B_MN, true, EPI_STORE, BITS, false>(a, a, p, st);
+  const TileShape s = packed_shape(p.M, p.N, sm_count());
+  if (s.bn == 128) return launch<1, false, B_MN, true, EPI_STORE, BITS, false, 128>(a, a, p, st);
+  return s.pair ? launch<2, false, B_MN, true, EPI_STORE, BITS, true>(a, a, p, st)
+                : launch<2, false, B_MN, true, EPI_STORE, BITS, false>(a, a, p, st);
 }
 
 template <int BITS>
 int launch_ds(const Operand& a, const Operand& b, GemmParams& p, cudaStream_t st) {
-  const TileShape s = choose_shape(p.M, p.N, p.partial != nullptr ? kBN : 1 << p.group_shift);
+  const TileShape s = choose_shape(p.M, p.N, p.partial != nullptr ? kBN : 1 << p.group_shift, sm_count());
   if (s.bn == 64) return launch<1, true, true, false, EPI_DS, BITS, false, 64>(a, b, p, st);
   if (s.bn == 128) return launch<1, true, true, false, EPI_DS, BITS, false, 128>(a, b, p, st);
   if (!s.pair) return launch<1, true, true, false, EPI_DS, BITS, false>(a, b, p, st);
@@ -1114,12 +1123,11 @@ int launch_dense_dw_ste(const eqat_desc& d, const eqat_bf16* dY, const eqat_bf16
   p.Q = (float)((1 << d.bits) - 1);
   p.dz_literal = d.dz_mode;
   const Operand a{dY, (uint64_t)d.out_features, (uint64_t)d.tokens, true}, b{X, (uint64_t)d.in_features, (uint64_t)d.tokens, true};
-  const int narrow = narrow_columns(p.M, p.N, d.group);
-  if (narrow == 64) return launch<1, true, true, false, EPI_STE, 2, false, 64>(a, b, p, st);
-  if (narrow == 128) return launch<1, true, true, false, EPI_STE, 2, false, 128>(a, b, p, st);
-  // 128 rows per CTA: with two accumulator sets this epilogue, the longest of the three, runs under the next tile
-  return p.M > 128 ? launch<1, true, true, false, EPI_STE, 2, true>(a, b, p, st)
-                   : launch<1, true, true, false, EPI_STE, 2, false>(a, b, p, st);
+  const TileShape shape = ste_shape(p.M, p.N, d.group, sm_count());
+  if (shape.bn == 64) return launch<1, true, true, false, EPI_STE, 2, false, 64>(a, b, p, st);
+  if (shape.bn == 128) return launch<1, true, true, false, EPI_STE, 2, false, 128>(a, b, p, st);
+  return shape.pair ? launch<1, true, true, false, EPI_STE, 2, true>(a, b, p, st)
+                : launch<1, true, true, false, EPI_STE, 2, false>(a, b, p, st);
 }
 
 int launch_latent_fwd(const eqat_desc& d, const eqat_bf16* X, const eqat_bf16* W, const float* s, const float* z,

@@ -19,6 +19,16 @@ bool make_tmap_blocks_bf16(CUtensorMap* tm, const void* base, uint64_t inner, ui
 bool make_tmap_u8(CUtensorMap* tm, const void* base, uint64_t inner_bytes, uint64_t outer, uint32_t box_bytes,
                   uint32_t box_outer, uint32_t swizzle_bytes);
 
+// How a contraction is cut into output tiles: rows per CTA (128 * mt), whether pairs of CTAs share a tile, and its columns.
+struct TileShape {
+  int mt;
+  bool pair;
+  int bn;
+  int rows() const { return 128 * mt * (pair ? 2 : 1); }
+};
+// Of the packed contractions Y and dX: M x N results, on a device of `sms` SMs.
+TileShape packed_shape(int M, int N, int sms);
+
 // Y[T,out] = X[T,in] * What[out,in]^T
 int launch_dense_fwd(const eqat_desc& d, const eqat_bf16* X, const eqat_bf16* What, eqat_bf16* Y, cudaStream_t st);
 // dX[T,in] = dY[T,out] * What[out,in]

@@ -391,13 +391,17 @@ int launch_rows(WideParams& p, int bits, const eqat_bf16* X, int pairs, int spli
 
 }  // namespace
 
-// Whether this kernel is expected to beat the tiled kernel of gemm.cu (512 or 256 TOKENS x 256 weight rows per tile), and
-// with which token tiles and split of K.  The terms are fits to timings on the 7B, 13B and 70B shapes from 65 to 2048
-// tokens (within 15 %).  Here: a CTA costs 5 us plus 0.018 us per token column outside its runs, a run 0.41 / 0.62 / 0.41
-// us (2 / 3 / 4-bit codes: its expansion) or 0.0021 us per token column (its MMAs), a quarter more when most SMs are
-// loading.  There: 8 us and 0.65 / 0.72 / 0.67 us per tile and 64 input columns, a tenth more with most SMs at work, or,
-// for at most 256 tokens, 0.88 / 1.13 / 1.15 us on one CTA.  4096 x 4096, 2 bits: 128 tokens 64.2 -> 13.2 us, 333 tokens
-// 49.4 -> 16.2 us, 1024 tokens 49.8 -> 29 us; at 2048 tokens the tiled kernel is ahead (51 against 58 us).
+// Whether this kernel is expected to beat the tiled kernel of gemm.cu (512 or 256 TOKENS x 256 weight rows per tile, or 128 x
+// 128 where all of those fit the chip at once), and with which token tiles and split of K.  The terms are fits to timings on
+// the 7B, 13B and 70B shapes from 65 to 2048 tokens (within 15 %).  Here: a CTA costs 5 us plus 0.018 us per token column
+// outside its runs, a run 0.41 / 0.62 / 0.41 us (2 / 3 / 4-bit codes: its expansion) or 0.0021 us per token column (its MMAs),
+// a quarter more when most SMs are loading.  There: 8 us and 0.65 / 0.72 / 0.67 us per tile and 64 input columns, a tenth more
+// with most SMs at work, or, for at most 256 tokens, 0.88 / 1.13 / 1.15 us on one CTA.  4096 x 4096, 2 bits: 128 tokens 64.2 ->
+// 13.2 us, 333 tokens 49.4 -> 16.2 us, 1024 tokens 49.8 -> 29 us; at 2048 tokens the tiled kernel is ahead (51 against 58 us).
+// Tiles of 128 x 128 take 3.6 us and 0.42 / 0.49 / 0.47 us per 64 input columns; the line that picks the faster kernel is a
+// little above that, because the estimate here is 10 to 15 % high for problems of that size.  Over 1024 of them (65 to 4096
+// tokens, 128 to 16384 columns) the kernel picked takes 0.15 % more than the faster one; by the price of 256-column tiles,
+// 2.7 % (1022 tokens of 64 x 128, 3 bits: 5.8 against 3.8 us; 1536 of 1536 x 512, 2 bits: 9.0 against 8.0 us).
 bool wide_fwd_applies(const eqat_desc& d, int given_sms, WidePlan& best) {
   best = WidePlan{};
   const int sms = given_sms > 0 ? given_sms : sm_count();
@@ -432,6 +436,8 @@ bool wide_fwd_applies(const eqat_desc& d, int given_sms, WidePlan& best) {
   if (best.us == 0.0) return false;
   const int cols = (d.out_features + 255) / 256, kb = d.in_features / 64;
   double tiled;
+  if (packed_shape(T, d.out_features, sms).bn == 128)
+    return best.us < 5.0 + kb * (d.bits == 2 ? 0.48 : (d.bits == 3 ? 0.58 : 0.52));
   if (T <= 256) {
     tiled = 8.0 + ((cols + sms - 1) / sms) * kb * (d.bits == 2 ? 0.88 : (d.bits == 3 ? 1.13 : 1.15));
   } else {

@@ -73,6 +73,19 @@ def test_large_batches_of_4_bit_codes_keep_the_tiled_kernel(eqat):
     assert route(eqat, 4096, 4096, 333, 4, 128)[0] == eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS
 
 
+def test_the_tiled_kernel_is_priced_by_the_tiles_it_takes(eqat):
+    """128 x 128 where all of them fit the chip at once: with few columns those are ahead of the weight-row pairs."""
+    for out, in_f, tokens, bits in ((64, 128, 1022, 3),           # 3.8 against 5.8 us
+                                    (640, 256, 1816, 2),          # 5.4 against 7.5
+                                    (1536, 512, 1536, 2),         # 8.0 against 9.0
+                                    (128, 384, 3938, 3)):         # 7.0 against 9.7
+        assert route(eqat, out, in_f, tokens, bits, 64)[0] == eqat.EQAT_ROUTE_TILED, (out, in_f, tokens)
+    for out, in_f, tokens, bits in ((1536, 1024, 1536, 2),        # 11.1 against 12.0
+                                    (256, 512, 256, 4),           # 4.9 against 7.5
+                                    (3392, 1024, 417, 4)):        # 10.2 against 12.4
+        assert route(eqat, out, in_f, tokens, bits, 64)[0] == eqat.EQAT_ROUTE_WEIGHT_ROW_PAIRS, (out, in_f, tokens)
+
+
 def test_plans_cover_all_tokens(eqat):
     rng = random.Random(3)
     for _ in range(3000):
