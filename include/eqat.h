@@ -269,6 +269,23 @@ int eqat_packed_fwd_route(const eqat_desc* desc, int sms, int* h_plan);
  * where one launch takes all rows. */
 int eqat_packed_fwd_rest(const eqat_desc* desc, int sms, int* h_rest);
 
+/* The output tiles of a contraction, decided on the host from the descriptor alone
+ * (a diagnostic; no counterpart in the paper).  `sms` as in eqat_packed_fwd_route;
+ * h_tile receives three numbers: rows of a tile per CTA, its columns, and the CTAs
+ * that share it (1 or 2; two CTAs have rows of their own).  EQAT_GEMM_PACKED_Y is
+ * the tiled kernel, whether or not qlinear_packed_fwd takes it. */
+enum {
+  EQAT_GEMM_Y = 0,                  /* qlinear_fakequant_fwd, W_hat stored                  */
+  EQAT_GEMM_DX = 1,                 /* qlinear_fakequant_bwd: dX, W_hat stored              */
+  EQAT_GEMM_DW = 2,                 /* qlinear_fakequant_bwd: the weight gradient           */
+  EQAT_GEMM_LATENT_Y = 3,           /* as 0 and 1 with W_hat == NULL                        */
+  EQAT_GEMM_LATENT_DX = 4,
+  EQAT_GEMM_PACKED_Y = 5,           /* qlinear_packed_fwd, bwd_dx and bwd_ds                */
+  EQAT_GEMM_PACKED_DX = 6,
+  EQAT_GEMM_PACKED_DS = 7
+};
+int eqat_gemm_tile(const eqat_desc* desc, int contraction, int sms, int* h_tile);
+
 /* dX = dY * ((W_int - z) * s).
  *   dY [T,out] bf16, Wq_packed, s16, z (in)   dX [T,in] bf16 (out) */
 int qlinear_packed_bwd_dx(const eqat_desc* desc, const eqat_bf16* dY, const uint8_t* Wq_packed,

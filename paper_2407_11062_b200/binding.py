@@ -22,6 +22,8 @@ EQAT_ERR_WORKSPACE, EQAT_ERR_CUDA, EQAT_ERR_TIMEOUT = -5, -6, -7
 EQAT_OP_FAKEQUANT_BWD, EQAT_OP_PACKED_BWD_DS = 1, 2
 EQAT_ZP_U8, EQAT_ZP_FP16 = 0, 1
 EQAT_ROUTE_MATRIX_VECTOR, EQAT_ROUTE_WEIGHT_ROWS, EQAT_ROUTE_WEIGHT_ROW_PAIRS, EQAT_ROUTE_TILED = 1, 2, 3, 4
+EQAT_GEMM_Y, EQAT_GEMM_DX, EQAT_GEMM_DW, EQAT_GEMM_LATENT_Y, EQAT_GEMM_LATENT_DX = 0, 1, 2, 3, 4
+EQAT_GEMM_PACKED_Y, EQAT_GEMM_PACKED_DX, EQAT_GEMM_PACKED_DS = 5, 6, 7
 
 
 class EqatError(RuntimeError):
@@ -73,6 +75,7 @@ def _load():
         "qlinear_packed_fwd": (c_int, [D, P, P, P, P, P, P]),
         "eqat_packed_fwd_route": (c_int, [D, c_int, POINTER(c_int)]),
         "eqat_packed_fwd_rest": (c_int, [D, c_int, POINTER(c_int)]),
+        "eqat_gemm_tile": (c_int, [D, c_int, c_int, POINTER(c_int)]),
         "qlinear_packed_bwd_dx": (c_int, [D, P, P, P, P, P, P]),
         "qlinear_packed_bwd_ds": (c_int, [D, P, P, P, P, P, P, P, P, c_size_t, P]),
         "eqat_block_ap_step": (c_int, [POINTER(eqat_block_ap_linear), c_int, POINTER(c_int), P]),
@@ -218,6 +221,13 @@ def eqat_packed_fwd_rest(desc, sms=0):
     rest = (c_int * 2)()
     _check(lib.eqat_packed_fwd_rest(ctypes.byref(desc), int(sms), rest), "eqat_packed_fwd_rest")
     return tuple(rest)
+
+
+def eqat_gemm_tile(desc, contraction, sms=0):
+    """The output tiles of a contraction (EQAT_GEMM_*): rows per CTA, columns, CTAs that share a tile."""
+    tile = (c_int * 3)()
+    _check(lib.eqat_gemm_tile(ctypes.byref(desc), int(contraction), int(sms), tile), "eqat_gemm_tile")
+    return tuple(tile)
 
 
 def qlinear_packed_bwd_dx(desc, dY, Wq_packed, s16, z8, dX):

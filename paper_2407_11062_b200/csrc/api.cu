@@ -311,6 +311,18 @@ int eqat_packed_fwd_rest(const eqat_desc* d, int sms, int* h_rest) {
   return EQAT_OK;
 }
 
+int eqat_gemm_tile(const eqat_desc* d, int contraction, int sms, int* h_tile) {
+  if (contraction < EQAT_GEMM_Y || contraction > EQAT_GEMM_PACKED_DS) return EQAT_ERR_UNSUPPORTED;
+  EQAT_TRY(check_gemm_desc(d, contraction >= EQAT_GEMM_PACKED_Y));
+  if (h_tile == nullptr) return EQAT_ERR_NULL;
+  if (sms < 0) return EQAT_ERR_SHAPE;
+  const TileShape t = contraction_shape(*d, contraction, sms > 0 ? sms : sm_count());
+  h_tile[0] = 128 * t.mt;
+  h_tile[1] = t.bn;
+  h_tile[2] = t.pair ? 2 : 1;
+  return EQAT_OK;
+}
+
 int qlinear_packed_bwd_dx(const eqat_desc* d, const eqat_bf16* dY, const uint8_t* Wq_packed, const eqat_fp16* s16,
                           const void* z, eqat_bf16* dX, void* stream) {
   EQAT_TRY(v_packed_fwd(d, dY, Wq_packed, s16, z, dX));          // same shape of check: one activation in, one out

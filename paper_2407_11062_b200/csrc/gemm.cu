@@ -1033,6 +1033,12 @@ TileShape ste_shape(int M, int N, int group, int sms) {
   return {1, bn == kBN && M > 128, bn};
 }
 
+// The step-size gradient: a group lies in a tile, or the sums of 256 columns go to memory.
+TileShape ds_shape(int M, int N, int group, int sms) { return choose_shape(M, N, group < kBN ? group : kBN, sms); }
+
+// The latent weight, fake-quantised in shared memory.
+TileShape latent_shape(int M) { return {2, M > 256, kBN}; }
+
 }  // namespace
 
 // Packed codes: 256 rows per CTA, pairs as soon as there are more rows than one CTA takes.  (128 columns are the least that
@@ -1040,6 +1046,20 @@ TileShape ste_shape(int M, int N, int group, int sms) {
 TileShape packed_shape(int M, int N, int sms) {
   if (narrow_columns(M, N, 128, sms) == 128) return {1, false, 128};
   return {2, M > 256, kBN};
+}
+
+TileShape contraction_shape(const eqat_desc& d, int contraction, int sms) {
+  const int T = (int)d.tokens, out = d.out_features, in = d.in_features;
+  switch (contraction) {
+    case EQAT_GEMM_Y: return choose_shape(T, out, 64, sms);
+    case EQAT_GEMM_DX: return choose_shape(T, in, 64, sms);
+    case EQAT_GEMM_DW: return d.group <= kBN ? ste_shape(out, in, d.group, sms) : choose_shape(out, in, 64, sms);
+    case EQAT_GEMM_LATENT_Y:
+    case EQAT_GEMM_LATENT_DX: return latent_shape(T);
+    case EQAT_GEMM_PACKED_Y: return packed_shape(T, out, sms);
+    case EQAT_GEMM_PACKED_DX: return packed_shape(T, in, sms);
+    default: return ds_shape(out, in, d.group, sms);
+  }
 }
 
 namespace {
@@ -1082,7 +1102,7 @@ int launch_packed(const Operand& a, GemmParams& p, cudaStream_t st) {
 
 template <int BITS>
 int launch_ds(const Operand& a, const Operand& b, GemmParams& p, cudaStream_t st) {
-  const TileShape s = choose_shape(p.M, p.N, p.partial != nullptr ? kBN : 1 << p.group_shift, sm_count());
+  const TileShape s = ds_shape(p.M, p.N, p.partial != nullptr ? kBN : 1 << p.group_shift, sm_count());
   if (s.bn == 64) return launch<1, true, true, false, EPI_DS, BITS, false, 64>(a, b, p, st);
   if (s.bn == 128) return launch<1, true, true, false, EPI_DS, BITS, false, 128>(a, b, p, st);
   if (!s.pair) return launch<1, true, true, false, EPI_DS, BITS, false>(a, b, p, st);
@@ -1136,8 +1156,8 @@ int launch_latent_fwd(const eqat_desc& d, const eqat_bf16* X, const eqat_bf16* W
   p.D = Y;
   set_latent(p, d, W, s, z);
   const Operand a{X, (uint64_t)d.tokens, (uint64_t)d.in_features, false}, b{W, (uint64_t)d.out_features, (uint64_t)d.in_features, false};
-  return p.M > 256 ? launch<2, false, false, true, EPI_STORE, 16, true>(a, b, p, st)
-                   : launch<2, false, false, true, EPI_STORE, 16, false>(a, b, p, st);
+  return latent_shape(p.M).pair ? launch<2, false, false, true, EPI_STORE, 16, true>(a, b, p, st)
+                               : launch<2, false, false, true, EPI_STORE, 16, false>(a, b, p, st);
 }
 
 int launch_latent_dx(const eqat_desc& d, const eqat_bf16* dY, const eqat_bf16* W, const float* s, const float* z,
@@ -1146,8 +1166,8 @@ int launch_latent_dx(const eqat_desc& d, const eqat_bf16* dY, const eqat_bf16* W
   p.D = dX;
   set_latent(p, d, W, s, z);
   const Operand a{dY, (uint64_t)d.tokens, (uint64_t)d.out_features, false}, b{W, (uint64_t)d.in_features, (uint64_t)d.out_features, true};
-  return p.M > 256 ? launch<2, false, true, true, EPI_STORE, 16, true>(a, b, p, st)
-                   : launch<2, false, true, true, EPI_STORE, 16, false>(a, b, p, st);
+  return latent_shape(p.M).pair ? launch<2, false, true, true, EPI_STORE, 16, true>(a, b, p, st)
+                               : launch<2, false, true, true, EPI_STORE, 16, false>(a, b, p, st);
 }
 
 int launch_packed_fwd(const eqat_desc& d, const eqat_bf16* X, const uint8_t* Wq, const eqat_fp16* s16,

@@ -28,6 +28,8 @@ struct TileShape {
 };
 // Of the packed contractions Y and dX: M x N results, on a device of `sms` SMs.
 TileShape packed_shape(int M, int N, int sms);
+// Of one of the contractions EQAT_GEMM_*.
+TileShape contraction_shape(const eqat_desc& d, int contraction, int sms);
 
 // Y[T,out] = X[T,in] * What[out,in]^T
 int launch_dense_fwd(const eqat_desc& d, const eqat_bf16* X, const eqat_bf16* What, eqat_bf16* Y, cudaStream_t st);

@@ -400,7 +400,7 @@ int launch_rows(WideParams& p, int bits, const eqat_bf16* X, int pairs, int spli
 // 13.2 us, 333 tokens 49.4 -> 16.2 us, 1024 tokens 49.8 -> 29 us; at 2048 tokens the tiled kernel is ahead (51 against 58 us).
 // Tiles of 128 x 128 take 3.6 us and 0.42 / 0.49 / 0.47 us per 64 input columns; the line that picks the faster kernel is a
 // little above that, because the estimate here is 10 to 15 % high for problems of that size.  Over 1024 of them (65 to 4096
-// tokens, 128 to 16384 columns) the kernel picked takes 0.15 % more than the faster one; by the price of 256-column tiles,
+// tokens, 128 to 16384 columns) the kernel picked takes 0.13 % more than the faster one; by the price of 256-column tiles,
 // 2.7 % (1022 tokens of 64 x 128, 3 bits: 5.8 against 3.8 us; 1536 of 1536 x 512, 2 bits: 9.0 against 8.0 us).
 bool wide_fwd_applies(const eqat_desc& d, int given_sms, WidePlan& best) {
   best = WidePlan{};

@@ -427,7 +427,7 @@ def test_block_ap_ragged(eqat, out, in_f, tokens, bits, group):
 
 @pytest.mark.parametrize("out,in_f,tokens,bits,group", [
     (512, 512, 256, 2, 64),         # the first workload's shape: single CTAs
-    (512, 512, 700, 4, 128),        # pairs of CTAs, ragged last row-tile
+    (512, 512, 700, 4, 128),        # pairs of CTAs, ragged last row-tile (with a stored W_hat single ones of 64 columns)
     (192, 384, 300, 3, 32),         # two groups per 64-column unit, ragged in every dimension
     (320, 768, 1030, 2, 256),
     (192, 1408, 600, 4, 1408),      # one group per row, in_features not a power of two
@@ -536,8 +536,8 @@ def check_e2e(r, group):
 def test_e2e_small(eqat, bits, group, real_z):
     """Every group size of the paper's ablation (32 .. 256) and one group per row (512 = in_features, the
     channel-wise setting of its Q-PEFT comparison), with frozen integer zero points and with trained fp16 ones.
-    600 tokens: a pair of CTAs per tile with a ragged last row-tile; 256: single CTAs (dX and ds; the forward of both runs on
-    pairs of weight-row tiles, the tiled forward in test_packed_forward_of_large_batches)."""
+    600 tokens: a ragged last row-tile.  (Tiles of 64 or 128 columns for dX and, where a group fits one, ds; the other tiles
+    in test_tile_shapes.py.  The forward runs on pairs of weight-row tiles, the tiled one in the tests of large batches.)"""
     for tokens in (600, 256):
         cfg = small_cfg(f"e2e_{bits}_{group}", 512, 512, bits, group, tokens, "student_t4", 0.02, 0.01)
         check_e2e(run_e2e(eqat, cfg, cfg.linears[0], tokens, real_z=real_z), group)
@@ -795,13 +795,13 @@ def test_packed_forward_for_prompts(eqat, out, in_f, tokens, bits, group, real_z
     (320, 640, 4100, 3, 64, True),
     (448, 1408, 4100, 3, 1408, False),
     (512, 768, 4100, 2, 32, True),       # 2-bit codes: runs of two K blocks
-    (192, 512, 4352, 2, 256, False),     # half a row tile of a pair: the second CTA has no tokens
+    (192, 512, 4352, 2, 256, False),     # whole row tiles
     (25600, 512, 128, 4, 32, False),     # many weight rows, few tokens: one CTA per tile
     (25600, 384, 200, 3, 128, True),
     (25600, 512, 256, 2, 64, False),
 ])
 def test_packed_forward_of_large_batches(eqat, out, in_f, tokens, bits, group, real_z):
-    """The tiled kernel: the forms that the smaller cases do not reach."""
+    """The tiled kernel: tiles of 128 x 128, and with 25600 weight rows of 256 x 256.  (Pairs of CTAs in test_tile_shapes.py.)"""
     cfg = small_cfg(f"tiled_{out}_{in_f}_{tokens}", out, in_f, bits, group, tokens, "student_t4", 0.02, 0.01)
     zfmt = eqat.EQAT_ZP_FP16 if real_z else eqat.EQAT_ZP_U8
     assert eqat.eqat_packed_fwd_route(eqat.make_desc(bits, group, out, in_f, tokens, 0, zfmt))[0] == eqat.EQAT_ROUTE_TILED
