@@ -447,12 +447,18 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
     const float sv = gp.s;
     const float zr = rintf(gp.z);
     const float rs = group_rcp(sv, zr);                 // NaN: the whole group takes the defining sequence
-    const size_t g = group_index<LONG>(e0, group);
-    if (e0 == (LONG ? g * (size_t)group << 5 : g << group)) {          // the group's first lane
-      z8[g] = (uint8_t)(__float_as_uint(fminf(fmaxf(zr, 0.0f), Q) + 8388608.0f) & 0xFFu);
-      s16[g] = __half_as_ushort(__float2half_rn(sv));
-    }
     uint32_t* dst = reinterpret_cast<uint32_t*>(packed) + (e0 >> 5) * BITS;
+    // Zero point and step size, by the group's first lane: before the comparisons (28672 x 8192, groups of 64: 105.9 against 109.2
+    // us with it after them), after everything else (3 bits 111.8 against 114.5 us, 4 bits 120.8 against 124.0 us).
+    auto hand_over = [&] {
+      const size_t g = group_index<LONG>(e0, group);
+      if (e0 == (LONG ? g * (size_t)group << 5 : g << group)) {
+        z8[g] = (uint8_t)(__float_as_uint(fminf(fmaxf(zr, 0.0f), Q) + 8388608.0f) & 0xFFu);
+        s16[g] = __half_as_ushort(__float2half_rn(sv));
+      }
+    };
+    constexpr bool kFirst = BITS == 2 && !LONG;
+    if constexpr (kFirst) hand_over();
     if constexpr (BITS == 2) {
       if (Thresholds2::apply(sv, rs)) {
         // Codes j and j + 8 of a word are decided as a pair: bit 0 is set where one or all three of the comparisons hold,
@@ -471,6 +477,7 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
             word[h] |= m1 & (0x00020002u << (2 * j));
           }
         }
+        if constexpr (!kFirst) hand_over();
         *reinterpret_cast<uint2*>(dst) = make_uint2(word[0], word[1]);
         return;
       }
@@ -510,6 +517,7 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
         acc = (acc << BITS) + __float_as_uint(fminf(fmaxf(t[i], kTwo23), kTwo23 + Q));
       piece[u] = acc - kBias;
     }
+    if constexpr (!kFirst) hand_over();
     if constexpr (BITS == 2) {
       *reinterpret_cast<uint2*>(dst) = make_uint2(piece[0] | (piece[1] << 16), piece[2] | (piece[3] << 16));
     } else if constexpr (BITS == 3) {
