@@ -409,31 +409,46 @@ bool wide_fwd_applies(const eqat_desc& d, int given_sms, WidePlan& best) {
   const int T = (int)d.tokens, runs = d.in_features / kRun, pairs = (d.out_features + 2 * kRows - 1) / (2 * kRows);
   const int least = (T + kMaxTn - 1) / kMaxTn;
   auto resident = [&](int lg) { return given_sms > 0 ? sms * kResidentOf148[lg] / 148 : max_clusters(d.bits, lg); };
+  auto columns = [&](int tt) { return ((T + tt - 1) / tt + 31) / 32 * 32; };                // of each of tt token tiles
+  auto round_us = [&](int tn, int lg, int clusters) {        // of clusters that are resident together
+    const double expand = d.bits == 3 ? 0.62 : 0.41, mma = 0.0021 * tn;
+    const double load = (clusters << lg) * 2 > 100 ? 1.25 : 1.0;
+    return 5.0 + 0.018 * tn + ((runs + (1 << lg) - 1) >> lg) * (expand > mma ? expand : mma) * load;
+  };
+  const int splits = runs >= kMaxSplit ? 3 : (runs >= 2 ? 2 : 1);
+  static_assert(kMaxSplit == 4, "splits of 1, 2 and 4");
   for (int tt = least; tt <= least + 3; ++tt) {
-    const int tn = ((T + tt - 1) / tt + 31) / 32 * 32;
-    auto round_us = [&](int lg, int clusters) {              // of clusters that are resident together
-      const double expand = d.bits == 3 ? 0.62 : 0.41, mma = 0.0021 * tn;
-      const double load = (clusters << lg) * 2 > 100 ? 1.25 : 1.0;
-      return 5.0 + 0.018 * tn + ((runs + (1 << lg) - 1) >> lg) * (expand > mma ? expand : mma) * load;
-    };
-    for (int lg = 0; (1 << lg) <= kMaxSplit && (1 << lg) <= runs; ++lg) {
+    const int tn = columns(tt);
+    for (int lg = 0; lg < splits; ++lg) {
       const int clusters = pairs * tt, fit = resident(lg);
       if (fit <= 0) continue;
-      const double us = (clusters + fit - 1) / fit * round_us(lg, clusters);
+      const double us = (clusters + fit - 1) / fit * round_us(tn, lg, clusters);
       if (best.us == 0.0 || us < best.us) best = WidePlan{tn, (T + tn - 1) / tn, 1 << lg, pairs, 1, us};
-      // The whole rounds as they are, and what is left over split finer: 11008 x 4096, 2 bits, 333 tokens has 86 clusters of
-      // which 74 are resident, 50.4 us in two rounds (or tiled), 37.7 us with the last twelve split four ways; 28672 x 8192,
-      // 4 bits, 333 tokens 175.9 -> 157.7 us, 4096 x 11008, 4 bits, 1531 tokens 127.6 -> 116.7 us.
+    }
+  }
+  if (best.us == 0.0) return false;
+  // The whole rounds as they are, and what is left over split finer: 11008 x 4096, 2 bits, 333 tokens has 86 clusters of
+  // which 74 are resident, 50.0 us in two rounds (or tiled), 38.5 us with the last twelve split four ways; 28672 x 8192,
+  // 4 bits, 333 tokens 174.2 -> 157.1 us, 4096 x 11008, 4 bits, 1531 tokens 122.2 -> 112.0 us.  Not on narrower token tiles
+  // than one launch would take: more tiles expand the weight more often, which costs more than the estimate says (22976 x
+  // 25216, 4 bits, 949 tokens: 969 us in one launch on four token tiles, 1082 us in two on five).  Of 2045 problems of 65 to
+  // 4096 tokens 37 take more than 3 % longer than by a rule that knows one launch only, with the narrower tiles 76; all of
+  // them together take 0.886 of the time.
+  for (int tt = least, least_tn = best.tn; tt <= least + 3; ++tt) {
+    const int tn = columns(tt);
+    if (tn < least_tn) break;
+    for (int lg = 0; lg < splits; ++lg) {
+      const int clusters = pairs * tt, fit = resident(lg);
+      if (fit <= 0) continue;
       const int whole = clusters / fit * fit / tt;           // pairs of row tiles, with all their token tiles
-      for (int lg2 = lg + 1; whole > 0 && whole < pairs && (1 << lg2) <= kMaxSplit && (1 << lg2) <= runs; ++lg2) {
+      for (int lg2 = lg + 1; whole > 0 && whole < pairs && lg2 < splits; ++lg2) {
         const int rest = (pairs - whole) * tt, fit2 = resident(lg2);
         if (fit2 <= 0) continue;
-        const double two = clusters / fit * round_us(lg, clusters) + (rest + fit2 - 1) / fit2 * round_us(lg2, rest);
+        const double two = clusters / fit * round_us(tn, lg, clusters) + (rest + fit2 - 1) / fit2 * round_us(tn, lg2, rest);
         if (two < best.us) best = WidePlan{tn, (T + tn - 1) / tn, 1 << lg, whole, 1 << lg2, two};
       }
     }
   }
-  if (best.us == 0.0) return false;
   const int cols = (d.out_features + 255) / 256, kb = d.in_features / 64;
   double tiled;
   if (packed_shape(T, d.out_features, sms).bn == 128)

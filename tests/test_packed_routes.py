@@ -109,6 +109,9 @@ def test_the_rest_of_a_prompt_is_told(eqat):
     assert rest(4096, 11008, 1531, 4, 64, True) == (1024, 2)
     assert rest(4096, 4096, 333, 2, 64) == (0, 0)               # one round
     assert rest(512, 512, 4, 2, 64) == (0, 0)                   # another kernel
+    # one launch: a second one would come with more and narrower token tiles, and more expansions of the weight
+    assert (route(eqat, 22976, 25216, 949, 4, 64)[1], rest(22976, 25216, 949, 4, 64)) == ((4, 256, 1), (0, 0))     # 969 against 1082 us
+    assert (route(eqat, 4352, 25728, 1653, 2, 64)[1], rest(4352, 25728, 1653, 2, 64)) == ((8, 224, 1), (0, 0))     # 272 against 283
     import test_gpu_weight_row_forward as gpu
     for problem, tiles, split in gpu.REST:
         kernel, (token_tiles, _, first) = route(eqat, *problem)
