@@ -7,11 +7,14 @@ from helpers import bits_to_torch, f32, torch_to_f64
 from test_gpu_parity import dev, eqat  # noqa: F401
 from workloads import to_bf16_bits
 
+pytestmark = pytest.mark.filterwarnings("ignore:overflow:RuntimeWarning")
 ZERO_POINTS = (0.0, 1.0, 2.0, 3.0, -2.0, 5.0, 16.0)
 
 
 def steps():
-    for base in (1.0, 0.75, 1.0 / 3.0, 0.0234375, 6.1e-5, 1.5e-30, 1.0e36):
+    # the last four: the ends of what the comparisons stand for, below which 1 / s overflows and above which it is subnormal;
+    # there thresholds are subnormal, and boundaries overflow
+    for base in (1.0, 0.75, 1.0 / 3.0, 0.0234375, 6.1e-5, 1.5e-30, 1.0e36, 1.0e-38, 2.94e-39, 8.4e37, 8.5e37):
         for ulps in (-2, -1, 0, 1, 2):
             s = np.float32(base)
             for _ in range(abs(ulps)):
@@ -76,3 +79,27 @@ def test_codes_on_and_beside_the_thresholds(eqat, group):  # noqa: F811
     assert np.array_equal(codes.cpu().numpy(), want)
     value = (want.astype(np.float32) - z_all) * s_all                     # binary32, then rounded to bf16
     assert np.array_equal(torch_to_f64(What), f32(to_bf16_bits(value)).astype(np.float64))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("group", [64, 256, 512])
+def test_all_bf16_numbers(eqat, group):  # noqa: F811
+    """Every bf16 number, NaN and subnormal ones among them, through quantise + pack and the fake quantiser.  W_hat bit for bit
+    what Eq. 2 gives in binary32, rounded to bf16: its zeros are +0, as the difference of equal integers is."""
+    bits16 = np.arange(65536, dtype=np.uint16).reshape(-1, 512)
+    W, Wd = f32(bits16), bits_to_torch(bits16)
+    out, in_f = bits16.shape
+    d = eqat.make_desc(2, group, out, in_f)
+    P = torch.empty(out, in_f // 4, dtype=torch.uint8, device="cuda")
+    z8, s16 = (torch.empty(out, in_f // group, dtype=t, device="cuda") for t in (torch.uint8, torch.float16))
+    codes, What = torch.empty(out, in_f, dtype=torch.uint8, device="cuda"), torch.empty(out, in_f, dtype=torch.bfloat16, device="cuda")
+    for s in steps():
+        for z in ZERO_POINTS:
+            sd, zd = dev(np.full((out, in_f // group), s, np.float32)), dev(np.full((out, in_f // group), z, np.float32))
+            eqat.eqat_quantize_pack(d, Wd, sd, zd, P, z8, s16)
+            eqat.eqat_unpack(d, P, codes)
+            eqat.eqat_fakequant_weight(d, Wd, sd, zd, What)
+            want = codes_of(W, s, np.float32(z))
+            assert np.array_equal(codes.cpu().numpy(), want), (s, z)
+            value = to_bf16_bits((want.astype(np.float32) - np.float32(z)) * s)
+            assert np.array_equal(What.view(torch.int16).cpu().numpy().view(np.uint16), value), (s, z)
