@@ -125,7 +125,8 @@ int eqat_minmax_init(const eqat_desc* desc, const eqat_bf16* W, float* s, float*
 /* ------------------------------------------------------------------ Block-AP */
 
 /* Eq. 1 followed by Eq. 2: W_hat = (clamp(round(W/s) + round(z), 0, 2^N-1) - round(z)) * s.
- * The quotient W/s is an IEEE binary32 division, rounded half-to-even.
+ * The quotient W/s is an IEEE binary32 division, rounded half-to-even.  Zeros of
+ * W_hat may carry either sign.
  *   W [out,in] bf16, s, z [out,in/g] fp32 (in)   W_hat [out,in] bf16 (out) */
 int eqat_fakequant_weight(const eqat_desc* desc, const eqat_bf16* W, const float* s, const float* z,
                           eqat_bf16* W_hat, void* stream);

@@ -9,8 +9,8 @@
 //     dX   = dY * W_hat   : A = dY [T,out] K-major,  B = W_hat [out,in] MN-major
 //     dW^  = dY^T * X     : A = dY [T,out] MN-major, B = X     [T,in]  MN-major
 //
-// A tile of the output is 256 columns wide and is computed either by one CTA or
-// by a PAIR of CTAs (a cluster of two on neighbouring SMs) that share one MMA
+// A tile of the output is 256 columns wide (128 or 64 where the problem is too small
+// to fill the chip) and is computed either by one CTA or by a PAIR of CTAs (a cluster of two on neighbouring SMs) that share one MMA
 // (tcgen05 cta_group::2): each CTA of a pair holds its own rows of A and of the
 // accumulator, and only HALF of the B operand; the tensor cores of the two SMs
 // exchange the halves.  Per flop a paired CTA therefore stages (loads, or expands
@@ -252,8 +252,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
   // Run by four warps per 128 rows, one per TMEM lane quadrant (warp index mod 4).  `m0` is the first output row of this
   // CTA's part of the tile.  What an epilogue reads from global memory it asks for a step ahead, and for the first step
   // before the accumulators are there.
-  // (The step-size gradient of 4096 x 11008, 4 bits, 1531 tokens: 155.6 -> 126.2 us with this and the second four warps;
-  // waiting for its codes, each step of 32 columns took as long as two K blocks.)
+  // (The step-size gradient of 4096 x 11008, 4 bits, 1531 tokens: 132.0 us with neither this nor the second four warps, 120.2
+  // with this alone, 119.2 with the warps alone, 112.0 with both; waiting for its codes, each step of 32 columns took as long
+  // as two K blocks.  Block-AP backward of 2048 x 2048, 512 tokens: 27.5, 26.3, 27.6, 24.7 us.)
   const int quad = warp & 3;
   const int row_in_tile = quad * 32 + lane;
   auto epilogue_tile = [&](int m0, int n_blk, int acc, uint32_t acc_phase) -> bool {
@@ -771,7 +772,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ 
                 const uint32_t row_sx = smem_base + C::b_offset(stage) + smem_row_sx;
                 if constexpr (LATENT) {
                   // Eq. 1 then Eq. 2 on the unit's 64 latent weights, in place: the same arithmetic, shortcut and
-                  // fallback as the stand-alone fake quantiser, so the operand is bit for bit the W_hat it would store.
+                  // fallback as the stand-alone fake quantiser, so the operand has the values of the W_hat it would store
+                  // (zeros that are -0 here may be +0 there; no sum over more than zeros can tell).
                   // (Rows or columns past the matrix were zero-filled by the copy and stay zero.)
                   if (valid) {
 #pragma unroll
@@ -998,8 +1000,10 @@ int launch(const Operand& a, const Operand& b, const GemmParams& p, cudaStream_t
 // the epilogue sums up lies in one tile); 256 when none does.  A small problem is a chain of latencies: the fill of the ring,
 // a K loop that waits for L2, an epilogue of BN / 32 steps per warp.  A K block takes a CTA about as long with 64 columns
 // (24 KB to fetch) as with 256 of a pair (32 KB), so more and smaller tiles shorten the chain as long as every SM has one.
-// 512 x 512, 256 tokens: Block-AP forward 9.0 -> 6.5 us, backward 20.1 -> 10.6 us, E2E-QP 23.7 -> 15.6 us; packed dX of
-// 2048 x 2048, 200 tokens 29.4 -> 16.4 us.
+// K does not enter: of 1200 problems (grids of up to 148 tiles of 128 x 128, K from 512 to 16384, ten contractions) narrow
+// tiles were slower in two, by 1.3 % (dW and ds on 12 x 12 tiles at K = 16384: 78.9 against 77.8 us).  128 tiles of 128 x 128, Y at K =
+// 512 / 2048 / 8192: 5.9 / 12.0 / 36.0 us, on pairs 7.8 / 14.9 / 43.3.  512 x 512, 256 tokens: Block-AP forward 9.9 -> 7.5 us,
+// backward 21.1 -> 10.2 us, E2E-QP 31 -> 20 us; packed dX of 2048 x 2048, 200 tokens 32.5 -> 18.1 us.
 int narrow_columns(int M, int N, int least, int sms) {
   const long rows = (M + 127) / 128;
   for (int bn = least <= 64 ? 64 : 128; bn < kBN && bn >= least; bn *= 2)

@@ -226,11 +226,15 @@ __device__ __forceinline__ void store_lane(eqat_bf16* dst, const uint4 (&o)[4], 
 // ------------------------------------------------------------------ 2-bit codes by comparison
 // For s > 0 the code of Eq. 1, clamp(round(w / s) + zr, 0, 3), does not fall as w grows, so a group has three bf16 numbers
 // T1 <= T2 <= T3 with code(w) = (w >= T1) + (w >= T2) + (w >= T3), and the packed comparison of bf16 pairs decides two
-// elements at once.  The boundary of "round(w / s) >= m" is at (m - 0.5) s, which fp32 gives to 2^-24; the bf16 numbers
-// beside its nearest one v are 2^-9 away, so they are decided, and v itself is put through the defining sequence.  About
-// 25 instructions per threshold and lane, 3.5 (packing) or 3 (fake quantiser) per element, where the arithmetic on each
-// element takes 9 and redoes the elements near a rounding boundary.  NaN compares false, i.e. code 0, like fmaxf and fminf.
-// 11008 x 4096, groups of 64: quantise + pack 27.7 -> 25.9 us; fake quantiser of 28672 x 8192 179.5 -> 170.0 us.
+// elements at once.  The boundary of "round(w / s) >= m" is at (m - 0.5) s, which fp32 gives to half a unit in its last
+// place; the bf16 numbers beside its nearest one v are at least a quarter of a bf16 unit away, 2^14 of those units, subnormal
+// or not.  So they are decided, and v itself is put through the defining sequence.  About 25 instructions per threshold and
+// lane, 3.5 (packing) or 3 (fake quantiser) per element, where the arithmetic on each element takes 9 and redoes the elements
+// near a rounding boundary.  NaN compares false, i.e. code 0, like fmaxf and fminf.
+// Groups of 64: fake quantiser of 28672 x 8192 175.6 -> 168.9 us, of 4096 x 4096 14.4 -> 13.7; quantise + pack on the min/max
+// grid, whose quotients hit rounding boundaries, 110.0 -> 105.9 and 12.9 -> 12.3 us.  With trained step sizes, which hardly do,
+// the arithmetic is 1 to 3 % ahead there: 103.4 against 106.0 and 12.1 against 12.3 us.  (Tried on that: thresholds from the
+// residual of v instead of a division, or made before the wait for the tile; both 3 % slower, the ALU pipe sets the pace.)
 struct Thresholds2 {
   uint32_t t[3];                                        // bf16 pairs, both halves the same
   __device__ __forceinline__ Thresholds2(float s, float zr) {
@@ -273,7 +277,7 @@ fakequant_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* 
       uint32_t value[4];                                  // the four values of the group, as bf16 pairs
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const float v = fmaf((float)k - zr, sv, 0.0f);    // (a zero is +0)
+        const float v = fmaf((float)k - zr, sv, 0.0f);    // (a zero is +0, as Eq. 2 gives it)
         value[k] = pack_bf16x2(v, v);
       }
       auto pick = [&](uint32_t w) {
@@ -296,7 +300,7 @@ fakequant_stream_kernel(const __grid_constant__ CUtensorMap map_w, const float* 
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const float c = fminf(fmaxf(r[i], lo), hi);
-          w[i] = LONG ? fmaf(c, sv, 0.0f) : c * sv;         // (LONG: a zero is always +0)
+          w[i] = LONG ? fmaf(c, sv, 0.0f) : c * sv;         // (LONG: a zero is always +0; else -0 where r or the clamp is)
         }
         o[u] = pack8(w);
       }
