@@ -63,10 +63,10 @@ EXTRA_CONFIGS = {
 # files change (comments and white space aside) the figures are stale and `roofline.traffic` is reported as null.
 NCU_TRAFFIC = {
     "sources": ("gemm.cu", "expand.cuh", "ptx.cuh", "wait.cuh"),
-    "sources_sha256": "ae0001cdddf7bbcb4fbea7a781313a8fd209ecd2f592748daa1ee4b6737c95a7",
-    "packed_fwd": {"qkvo": 140.6e6 + 98.8e6, "gate_up": 165.2e6 + 317.2e6, "down": 502.7e6 + 120.6e6},
-    "packed_bwd_dx": {"qkvo": 139.6e6 + 95.9e6, "gate_up": 513.8e6 + 115.8e6, "down": 153.4e6 + 316.7e6},
-    "packed_bwd_ds": {"qkvo": 416.4e6 + 1.0e6, "gate_up": 1325.1e6 + 2.8e6, "down": 1079.5e6 + 3.2e6},
+    "sources_sha256": "53e5cc028cee675ceb08c951b8120b557d26d87d1affe4e056f5845671d6af37",
+    "packed_fwd": {"qkvo": 140.8e6 + 95.4e6, "gate_up": 162.5e6 + 314.9e6, "down": 502.9e6 + 116.4e6},
+    "packed_bwd_dx": {"qkvo": 139.5e6 + 95.6e6, "gate_up": 514.7e6 + 116.0e6, "down": 154.7e6 + 315.3e6},
+    "packed_bwd_ds": {"qkvo": 420.7e6 + 0.8e6, "gate_up": 1318.3e6 + 2.7e6, "down": 1086.0e6 + 3.0e6},
 }
 
 
