@@ -229,12 +229,11 @@ __device__ __forceinline__ void store_lane(eqat_bf16* dst, const uint4 (&o)[4], 
 // elements at once.  The boundary of "round(w / s) >= m" is at (m - 0.5) s, which fp32 gives to half a unit in its last
 // place; the bf16 numbers beside its nearest one v are at least a quarter of a bf16 unit away, 2^14 of those units, subnormal
 // or not.  So they are decided, and v itself is put through the defining sequence.  About 25 instructions per threshold and
-// lane, 3.5 (packing) or 3 (fake quantiser) per element, where the arithmetic on each element takes 9 and redoes the elements
-// near a rounding boundary.  NaN compares false, i.e. code 0, like fmaxf and fminf.
+// lane and 3 per element, where the arithmetic on each element takes 9 and redoes the elements near a rounding boundary.  NaN compares false, i.e. code 0, like fmaxf and fminf.
 // Groups of 64: fake quantiser of 28672 x 8192 175.6 -> 168.9 us, of 4096 x 4096 14.4 -> 13.7; quantise + pack on the min/max
-// grid, whose quotients hit rounding boundaries, 110.0 -> 105.9 and 12.9 -> 12.3 us.  With trained step sizes, which hardly do,
-// the arithmetic is 1 to 3 % ahead there: 103.4 against 106.0 and 12.1 against 12.3 us.  (Tried on that: thresholds from the
-// residual of v instead of a division, or made before the wait for the tile; both 3 % slower, the ALU pipe sets the pace.)
+// grid, whose quotients hit rounding boundaries, 109.8 -> 92.8 and 13.0 -> 11.6 us, with trained step sizes, which hardly do,
+// 103.4 -> 93.1 and 12.2 -> 11.6 us.  (The thresholds from the residual of v instead of a division, or made before the wait for
+// the tile, were 3 % slower: the ALU pipe sets the pace, and the divisions run on another.)
 struct Thresholds2 {
   uint32_t t[3];                                        // bf16 pairs, both halves the same
   __device__ __forceinline__ Thresholds2(float s, float zr) {
@@ -452,7 +451,7 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
     const float zr = rintf(gp.z);
     const float rs = group_rcp(sv, zr);                 // NaN: the whole group takes the defining sequence
     uint32_t* dst = reinterpret_cast<uint32_t*>(packed) + (e0 >> 5) * BITS;
-    // Zero point and step size, by the group's first lane: before the comparisons (28672 x 8192, groups of 64: 105.9 against 109.2
+    // Zero point and step size, by the group's first lane: before the comparisons (28672 x 8192, groups of 64: 92.8 against 96.7
     // us with it after them), after everything else (3 bits 111.8 against 114.5 us, 4 bits 120.8 against 124.0 us).
     auto hand_over = [&] {
       const size_t g = group_index<LONG>(e0, group);
@@ -465,21 +464,24 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
     if constexpr (kFirst) hand_over();
     if constexpr (BITS == 2) {
       if (Thresholds2::apply(sv, rs)) {
-        // Codes j and j + 8 of a word are decided as a pair: bit 0 is set where one or all three of the comparisons hold,
-        // bit 1 where the second does.
+        // Codes j and j + 8 of a word are decided as a pair.  With c and d their codes, the three masks, each -1 in a half
+        // where it holds, add up to -(c + 2^16 (d - c)) as 32-bit numbers; so do the sums over all j, shifted by 2 j.  The lower
+        // half, the first eight codes, is missing in the upper one, and is added by the last multiplication.  (Selecting and
+        // masking bits took four logic operations per pair where this takes one addition and one shifted one, and the ALU
+        // pipe sets the pace: 28672 x 8192, groups of 64, 106.5 -> 93.2 us, 11008 x 4096 24.8 -> 22.5 us.)
         const Thresholds2 th(sv, zr);
         const uint32_t w[16] = {raw[0][0].x, raw[0][0].y, raw[0][0].z, raw[0][0].w, raw[0][1].x, raw[0][1].y, raw[0][1].z, raw[0][1].w,
                                 raw[0][2].x, raw[0][2].y, raw[0][2].z, raw[0][2].w, raw[0][3].x, raw[0][3].y, raw[0][3].z, raw[0][3].w};
-        uint32_t word[2] = {0u, 0u};
+        uint32_t word[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+          uint32_t acc = 0u;
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int j = 7; j >= 0; --j) {
             const uint32_t pair = __byte_perm(w[8 * h + (j >> 1)], w[8 * h + 4 + (j >> 1)], (j & 1) ? 0x7632 : 0x5410);
-            const uint32_t m0 = th.at_least(0, pair), m1 = th.at_least(1, pair), m2 = th.at_least(2, pair);
-            word[h] |= (m0 ^ m1 ^ m2) & (0x00010001u << (2 * j));
-            word[h] |= m1 & (0x00020002u << (2 * j));
+            acc = 4u * acc + (th.at_least(0, pair) + th.at_least(1, pair) + th.at_least(2, pair));
           }
+          word[h] = 0u - acc * 0x10001u;
         }
         if constexpr (!kFirst) hand_over();
         *reinterpret_cast<uint2*>(dst) = make_uint2(word[0], word[1]);
