@@ -467,8 +467,8 @@ quantize_pack_stream_kernel(const __grid_constant__ CUtensorMap map_w, const flo
         // Codes j and j + 8 of a word are decided as a pair.  With c and d their codes, the three masks, each -1 in a half
         // where it holds, add up to -(c + 2^16 (d - c)) as 32-bit numbers; so do the sums over all j, shifted by 2 j.  The lower
         // half, the first eight codes, is missing in the upper one, and is added by the last multiplication.  (Selecting and
-        // masking bits took four logic operations per pair where this takes one addition and one shifted one, and the ALU
-        // pipe sets the pace: 28672 x 8192, groups of 64, 106.5 -> 93.2 us, 11008 x 4096 24.8 -> 22.5 us.)
+        // masking bits took three logic operations per pair, this takes one addition and one shifted one, which the FMA pipe
+        // can do, and the ALU pipe sets the pace: 28672 x 8192, groups of 64, 106.5 -> 93.2 us, 11008 x 4096 24.8 -> 22.5 us.)
         const Thresholds2 th(sv, zr);
         const uint32_t w[16] = {raw[0][0].x, raw[0][0].y, raw[0][0].z, raw[0][0].w, raw[0][1].x, raw[0][1].y, raw[0][1].z, raw[0][1].w,
                                 raw[0][2].x, raw[0][2].y, raw[0][2].z, raw[0][2].w, raw[0][3].x, raw[0][3].y, raw[0][3].z, raw[0][3].w};
