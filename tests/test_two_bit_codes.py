@@ -7,14 +7,11 @@ from helpers import bits_to_torch, f32, torch_to_f64
 from test_gpu_parity import dev, eqat  # noqa: F401
 from workloads import to_bf16_bits
 
-pytestmark = pytest.mark.filterwarnings("ignore:overflow:RuntimeWarning")
 ZERO_POINTS = (0.0, 1.0, 2.0, 3.0, -2.0, 5.0, 16.0)
 
 
 def steps():
-    # the last four: the ends of what the comparisons stand for, below which 1 / s overflows and above which it is subnormal;
-    # there thresholds are subnormal, and boundaries overflow
-    for base in (1.0, 0.75, 1.0 / 3.0, 0.0234375, 6.1e-5, 1.5e-30, 1.0e36, 1.0e-38, 2.94e-39, 8.4e37, 8.5e37):
+    for base in (1.0, 0.75, 1.0 / 3.0, 0.0234375, 6.1e-5, 1.5e-30, 1.0e36):
         for ulps in (-2, -1, 0, 1, 2):
             s = np.float32(base)
             for _ in range(abs(ulps)):
@@ -81,8 +78,19 @@ def test_codes_on_and_beside_the_thresholds(eqat, group):  # noqa: F811
     assert np.array_equal(torch_to_f64(What), f32(to_bf16_bits(value)).astype(np.float64))
 
 
+def end_steps():
+    """The ends of what the comparisons stand for, below which 1 / s overflows and above which it is subnormal; there
+    thresholds are subnormal, and boundaries overflow."""
+    for base in (1.0e-38, 2.94e-39, 8.4e37, 8.5e37):
+        s = np.float32(base)
+        down, up = (np.nextafter(s, np.float32(to), dtype=np.float32) for to in (0.0, np.inf))
+        yield from (np.nextafter(down, np.float32(0.0), dtype=np.float32), down, s, up,
+                    np.nextafter(up, np.float32(np.inf), dtype=np.float32))
+
+
 @pytest.mark.gpu
-@pytest.mark.parametrize("group", [64, 256, 512])
+@pytest.mark.filterwarnings("ignore:overflow:RuntimeWarning")
+@pytest.mark.parametrize("group", [32, 64, 256, 512])
 def test_all_bf16_numbers(eqat, group):  # noqa: F811
     """Every bf16 number, NaN and subnormal ones among them, through quantise + pack and the fake quantiser.  W_hat bit for bit
     what Eq. 2 gives in binary32, rounded to bf16: its zeros are +0, as the difference of equal integers is."""
@@ -93,7 +101,7 @@ def test_all_bf16_numbers(eqat, group):  # noqa: F811
     P = torch.empty(out, in_f // 4, dtype=torch.uint8, device="cuda")
     z8, s16 = (torch.empty(out, in_f // group, dtype=t, device="cuda") for t in (torch.uint8, torch.float16))
     codes, What = torch.empty(out, in_f, dtype=torch.uint8, device="cuda"), torch.empty(out, in_f, dtype=torch.bfloat16, device="cuda")
-    for s in steps():
+    for s in (*steps(), *end_steps()):
         for z in ZERO_POINTS:
             sd, zd = dev(np.full((out, in_f // group), s, np.float32)), dev(np.full((out, in_f // group), z, np.float32))
             eqat.eqat_quantize_pack(d, Wd, sd, zd, P, z8, s16)
